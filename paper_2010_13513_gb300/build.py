@@ -21,7 +21,7 @@ OUT = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libhhg.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 # (source, object, extra flags): fast.cu and stream.cu are compiled once per precision
-SOURCES = [("kernels.cu", "kernels", []), ("fast.cu", "fast64", ["-DHHG_FAST_ONLY=64"]),
+SOURCES = [("kernels.cu", "kernels", []), ("transfer.cu", "transfer", []), ("fast.cu", "fast64", ["-DHHG_FAST_ONLY=64"]),
            ("fast.cu", "fast32", ["-DHHG_FAST_ONLY=32"]),
            ("fast.cu", "fast64b", ["-DHHG_FAST_ONLY=64", "-DHHG_FAST_BATCHED"]),
            ("fast.cu", "fast32b", ["-DHHG_FAST_ONLY=32", "-DHHG_FAST_BATCHED"]), ("stream.cu", "stream64", ["-DHHG_STREAM_ONLY=64"]),

@@ -119,39 +119,6 @@ struct OpDev {
   const float* bw32;
 };
 
-// ------------------------------------------------------- transfer tables
-// Prolongation I_{l-1}^l: a fine DoF at doubled fine position P (units h_f/2)
-// has class kappa = P mod 4 (P2) or (P/2) mod 2 (P1) and reads coarse DoFs
-// (g_c, a + d) with a = P >> 2 (P2) or (P/2) >> 1 (P1).
-// Restriction (transpose): a coarse DoF (g_c, a) reads fine DoFs
-// (g_f, 2a + e).
-struct HXTerm {
-  int arr;              // coarse group (prolongation) or fine group (restriction)
-  int di, dj, dk;
-  double w;
-};
-struct HTransfer {
-  int order;                                 // 1 or 2
-  int nclass;                                // 8 (P1) or 64 (P2)
-  std::vector<std::vector<HXTerm>> prol;     // [nclass]
-  std::vector<std::vector<HXTerm>> restr;    // [groups]
-};
-struct DXTerm {
-  int arr, di, dj, dk;
-};
-struct XferDev {
-  int order, nclass, ngroups;
-  int rmax;                   // most restriction terms of a group
-  const int* pcls_start;      // nclass + 1
-  const DXTerm* pterms;
-  const double* pw64;
-  const float* pw32;
-  const int* rg_start;        // ngroups + 1
-  const DXTerm* rterms;
-  const double* rw64;
-  const float* rw32;
-};
-
 // ------------------------------------------------------------ host builders
 enum OpId {
   OP_FULL = 0, OP_A, OP_BT, OP_B, OP_C, OP_MASS, OP_BC, OP_MVINT, OP_LOAD, OP_MLHAT, OP_ML, OP_COUNT
@@ -163,7 +130,6 @@ struct StencilSet {
   std::vector<double> diagA;      // per group: diagonal of A (relative weights)
 };
 StencilSet build_stencils(int disc, double h, double nu_a, bool pspg_rhs);
-HTransfer build_transfer(int order);
 
 // ------------------------------------------------------------ device launch
 struct Launch;  // fwd

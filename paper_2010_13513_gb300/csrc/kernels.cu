@@ -219,119 +219,6 @@ __global__ void kb_sub_scalar_p(const void* items, int n) {
   sub_scalar_body<T>(bid, it.a.g, it.a.p, it.a.sum, it.a.scale);
 }
 
-// ---------------------------------------------------------------- transfers
-template <class T>
-struct XferA { Geo gf, gc; XferDev X; int base_f, base_c, ncomp, G, interior_only; const T* in; T* out; };
-template <class T>
-__device__ __forceinline__ void prolong_body(const uint3 bid, const Geo& gf, const Geo& gc, const XferDev& X,
-                                             int base_f, int base_c, int ncomp, int G, int interior_only,
-                                             const T* __restrict__ xc, T* __restrict__ xf) {
-  const int nzp = gf.nz + 1;
-  const int gfi = bid.z / nzp;
-  const int k = bid.z - gfi * nzp;
-  const int i = bid.x * blockDim.x + threadIdx.x;
-  const int j = bid.y * blockDim.y + threadIdx.y;
-  const int ox = G == 1 ? 0 : c_goff[gfi][0], oy = G == 1 ? 0 : c_goff[gfi][1], oz = G == 1 ? 0 : c_goff[gfi][2];
-  if (!dof_valid(gf, i, j, k, ox, oy, oz)) return;
-  if (interior_only && dof_boundary(gf, i, j, k, ox, oy, oz)) return;
-  int ax, ay, az, cls;
-  if (X.order == 2) {
-    const int Px = 2 * i + ox, Py = 2 * j + oy, Pz = 2 * k + oz;
-    ax = Px >> 2; ay = Py >> 2; az = Pz >> 2;
-    cls = (Px & 3) + 4 * ((Py & 3) + 4 * (Pz & 3));
-  } else {
-    ax = i >> 1; ay = j >> 1; az = k >> 1;
-    cls = (i & 1) + 2 * ((j & 1) + 2 * (k & 1));
-  }
-  const int64_t cidx = site_index(gc, ax, ay, az);
-  const int64_t fidx = site_index(gf, i, j, k);
-  const int t0 = X.pcls_start[cls], t1 = X.pcls_start[cls + 1];
-  const int64_t cstride_c = int64_t(G) * gc.arr, cstride_f = int64_t(G) * gf.arr;
-  for (int c = 0; c < ncomp; ++c) {
-    T a = T(0);
-    for (int t = t0; t < t1; ++t) {
-      const DXTerm tm = X.pterms[t];
-      const int64_t off = int64_t(tm.di) + int64_t(tm.dj) * gc.sx + int64_t(tm.dk) * gc.sy;
-      a += wsel<T>(X.pw64, X.pw32, t) * xc[int64_t(base_c + tm.arr) * gc.arr + c * cstride_c + cidx + off];
-    }
-    xf[int64_t(base_f + gfi) * gf.arr + c * cstride_f + fidx] += a;
-  }
-}
-template <class T>
-__global__ void __launch_bounds__(128) k_prolong(Geo gf, Geo gc, XferDev X, int base_f, int base_c, int ncomp, int G,
-                                                 int interior_only, const T* __restrict__ xc, T* __restrict__ xf) {
-  prolong_body<T>(blockIdx, gf, gc, X, base_f, base_c, ncomp, G, interior_only, xc, xf);
-}
-template <class T>
-__global__ void __launch_bounds__(128) kb_prolong(const void* items, int n) {
-  uint3 bid, gd;
-  const auto& it = batch_item<XferA<T>>(items, n, bid, gd);
-  const XferA<T>& a = it.a;
-  prolong_body<T>(bid, a.gf, a.gc, a.X, a.base_f, a.base_c, a.ncomp, a.G, a.interior_only, a.in, a.out);
-}
-
-// r_c = I^T r_f per coarse DoF: its restriction terms (up to 125 for the P2
-// vertex group) are shared by P lanes, lane p taking terms p, p+P, ..., and
-// the partial sums are added by shuffles.  Block: 128 threads = 128/P coarse
-// sites along i; grid: (i blocks, j, (k, group)).
-template <class T, int P>
-__device__ __forceinline__ void restrict_body(const uint3 bid, const Geo& gf, const Geo& gc, const XferDev& X,
-                                              int base_f, int base_c, int ncomp, int G, int interior_only,
-                                              const T* __restrict__ rf, T* __restrict__ rc) {
-  const int nzp = gc.nz + 1;
-  const int gci = bid.z / nzp;
-  const int k = bid.z - gci * nzp;
-  const int i = bid.x * (128 / P) + int(threadIdx.x) / P, p = int(threadIdx.x) % P;
-  const int j = bid.y;
-  const int ox = G == 1 ? 0 : c_goff[gci][0], oy = G == 1 ? 0 : c_goff[gci][1], oz = G == 1 ? 0 : c_goff[gci][2];
-  const bool valid = dof_valid(gc, i, j, k, ox, oy, oz);
-  const bool zero = valid && interior_only && dof_boundary(gc, i, j, k, ox, oy, oz);
-  const int64_t cstride_f = int64_t(G) * gf.arr;
-  T a0 = T(0), a1 = T(0), a2 = T(0);
-  if (valid && !zero) {
-    const int t0 = X.rg_start[gci], t1 = X.rg_start[gci + 1];
-#pragma unroll 4
-    for (int t = t0 + p; t < t1; t += P) {
-      const DXTerm tm = X.rterms[t];
-      const int fi = 2 * i + tm.di, fj = 2 * j + tm.dj, fk = 2 * k + tm.dk;
-      if (fi < -1 || fj < -1 || fk < -1 || fi > gf.nx + 1 || fj > gf.ny + 1 || fk > gf.nz + 1) continue;
-      const T w = wsel<T>(X.rw64, X.rw32, t);
-      const T* f = rf + int64_t(base_f + tm.arr) * gf.arr + site_index(gf, fi, fj, fk);
-      a0 += w * f[0];
-      if (ncomp > 1) {
-        a1 += w * f[cstride_f];
-        a2 += w * f[2 * cstride_f];
-      }
-    }
-  }
-#pragma unroll
-  for (int m = P >> 1; m > 0; m >>= 1) {          // all lanes of the warp take part
-    a0 += __shfl_xor_sync(0xffffffffu, a0, m);
-    a1 += __shfl_xor_sync(0xffffffffu, a1, m);
-    a2 += __shfl_xor_sync(0xffffffffu, a2, m);
-  }
-  if (!valid || p != 0) return;
-  const int64_t cidx = site_index(gc, i, j, k), cstride_c = int64_t(G) * gc.arr;
-  T* o = rc + int64_t(base_c + gci) * gc.arr + cidx;
-  o[0] = zero ? T(0) : a0;
-  if (ncomp > 1) {
-    o[cstride_c] = zero ? T(0) : a1;
-    o[2 * cstride_c] = zero ? T(0) : a2;
-  }
-}
-template <class T, int P>
-__global__ void __launch_bounds__(128) k_restrict(Geo gf, Geo gc, XferDev X, int base_f, int base_c, int ncomp, int G,
-                                                  int interior_only, const T* __restrict__ rf, T* __restrict__ rc) {
-  restrict_body<T, P>(blockIdx, gf, gc, X, base_f, base_c, ncomp, G, interior_only, rf, rc);
-}
-template <class T, int P>
-__global__ void __launch_bounds__(128) kb_restrict(const void* items, int n) {
-  uint3 bid, gd;
-  const auto& it = batch_item<XferA<T>>(items, n, bid, gd);
-  const XferA<T>& a = it.a;
-  restrict_body<T, P>(bid, a.gf, a.gc, a.X, a.base_f, a.base_c, a.ncomp, a.G, a.interior_only, a.in, a.out);
-}
-
 // ------------------------------------------ canonical order <-> padded layout
 // Canonical host order: 3 velocity components (component-major) over the
 // velocity nodes in lexicographic order (P1: the lattice sites; P2: the
@@ -622,41 +509,6 @@ void launch_sub_scalar_p(const Geo& g, T* p, const double* sum, double scale, cu
 }
 
 template <class T>
-void launch_prolong(const Geo& gf, const Geo& gc, const XferDev& X, int base_f, int base_c, int ncomp, int G,
-                    bool interior_only, const T* xc, T* xf, cudaStream_t s) {
-  dim3 blk(32, 4, 1);
-  dim3 grd((gf.nx + 1 + 31) / 32, (gf.ny + 1 + 3) / 4, (gf.nz + 1) * G);
-  HHG_BATCHED(kb_prolong<T>, grd, blk, XferA<T>, gf, gc, X, base_f, base_c, ncomp, G, interior_only ? 1 : 0, xc, xf)
-  ++g_launches;
-  k_prolong<T><<<grd, blk, 0, s>>>(gf, gc, X, base_f, base_c, ncomp, G, interior_only ? 1 : 0, xc, xf);
-}
-
-template <class T>
-void launch_restrict(const Geo& gf, const Geo& gc, const XferDev& X, int base_f, int base_c, int ncomp, int G,
-                     bool interior_only, const T* rf, T* rc, cudaStream_t s) {
-  // lanes per coarse DoF: about eight terms each
-  const int P = X.rmax > 32 ? 8 : X.rmax > 16 ? 4 : X.rmax > 8 ? 2 : 1;
-  dim3 blk(128, 1, 1);
-  dim3 grd((gc.nx + 1 + 128 / P - 1) / (128 / P), gc.ny + 1, (gc.nz + 1) * G);
-  const int io = interior_only ? 1 : 0;
-  if (g_rec) {
-    const void* fn = P == 8   ? reinterpret_cast<const void*>(kb_restrict<T, 8>)
-                     : P == 4 ? reinterpret_cast<const void*>(kb_restrict<T, 4>)
-                     : P == 2 ? reinterpret_cast<const void*>(kb_restrict<T, 2>)
-                              : reinterpret_cast<const void*>(kb_restrict<T, 1>);
-    g_rec->add(fn, grd, blk, 0, 1, XferA<T>{gf, gc, X, base_f, base_c, ncomp, G, io, rf, rc});
-    return;
-  }
-  ++g_launches;
-  switch (P) {
-    case 8: k_restrict<T, 8><<<grd, blk, 0, s>>>(gf, gc, X, base_f, base_c, ncomp, G, io, rf, rc); break;
-    case 4: k_restrict<T, 4><<<grd, blk, 0, s>>>(gf, gc, X, base_f, base_c, ncomp, G, io, rf, rc); break;
-    case 2: k_restrict<T, 2><<<grd, blk, 0, s>>>(gf, gc, X, base_f, base_c, ncomp, G, io, rf, rc); break;
-    default: k_restrict<T, 1><<<grd, blk, 0, s>>>(gf, gc, X, base_f, base_c, ncomp, G, io, rf, rc); break;
-  }
-}
-
-template <class T>
 void launch_reduce(int mode, const T* a, const T* b, const double* w, int64_t n, double* partials, int max_blocks,
                    double* out, cudaStream_t s) {
   int nb = int(std::min<int64_t>((n + 255) / 256, max_blocks));
@@ -754,10 +606,6 @@ template void launch_canon_gather<float>(const Geo&, const float*, double*, int6
   template void launch_gs<T>(const Geo&, const OpDev&, int, int, double, T*, const T*, cudaStream_t);              \
   template void launch_pupdate<T>(const Geo&, T*, const T*, const double*, double, cudaStream_t);                 \
   template void launch_sub_scalar_p<T>(const Geo&, T*, const double*, double, cudaStream_t);                      \
-  template void launch_prolong<T>(const Geo&, const Geo&, const XferDev&, int, int, int, int, bool, const T*, T*, \
-                                  cudaStream_t);                                                                  \
-  template void launch_restrict<T>(const Geo&, const Geo&, const XferDev&, int, int, int, int, bool, const T*,    \
-                                   T*, cudaStream_t);                                                             \
   template void launch_reduce<T>(int, const T*, const T*, const double*, int64_t, double*, int, double*,          \
                                  cudaStream_t);                                                                   \
   template void launch_coarse<T>(const double*, int, const int64_t*, const T*, T*, cudaStream_t);                 \

@@ -32,12 +32,14 @@ void launch_gs(const Geo& g, const OpDev& A, int grp, int colour, double inv_dia
 template <class T>
 void launch_pupdate(const Geo& g, T* p, const T* r, const double* inv_mlhat, double inv_omega_inv, cudaStream_t s);
 
-// xf[base_f..] += I xc (interior_only: Dirichlet DoFs of xf untouched)
+// transfers of a whole block vector (transfer.cu): xf += I xc (interior_only:
+// Dirichlet velocity DoFs of xf untouched) and rc = I^T rf (Dirichlet velocity
+// rows 0)
 template <class T>
-void launch_prolong(const Geo& gf, const Geo& gc, const XferDev& X, int base_f, int base_c, int ncomp, int G,
-                    bool interior_only, const T* xc, T* xf, cudaStream_t s);
+void launch_prolong(const Geo& gf, const Geo& gc, bool interior_only, const T* xc, T* xf, cudaStream_t s);
+template <class T>
+void launch_restrict(const Geo& gf, const Geo& gc, const T* rf, T* rc, cudaStream_t s);
 
-// rc[base_c..] = I^T rf (interior_only: Dirichlet rows set to 0)
 // canonical host order (3 velocity components over the velocity nodes, then
 // the pressure nodes) <-> padded layout; the scatter writes only the nodes
 // (only boundary velocity nodes if boundary_only), the target is pre-zeroed
@@ -46,9 +48,6 @@ void launch_canon_scatter(const Geo& g, const double* src, T* dst, int64_t nvn, 
                           bool boundary_only, cudaStream_t s);
 template <class T>
 void launch_canon_gather(const Geo& g, const T* src, double* dst, int64_t nvn, int64_t npn, cudaStream_t s);
-template <class T>
-void launch_restrict(const Geo& gf, const Geo& gc, const XferDev& X, int base_f, int base_c, int ncomp, int G,
-                     bool interior_only, const T* rf, T* rc, cudaStream_t s);
 
 // deterministic two-pass reduction over n contiguous elements into out[0]
 template <class T>

@@ -118,11 +118,6 @@ struct OpOffsets {
   int nrows;
 };
 
-struct XferOffsets {
-  size_t pstart, pterms, pw64, pw32, rstart, rterms, rw64, rw32;
-  int order, nclass, ngroups, rmax;
-};
-
 struct Level {
   int l;
   Geo g;
@@ -163,9 +158,6 @@ struct hhg_problem {
   hhg_problem_desc desc;
   int G = 1, ov = 1;
   std::vector<Level> lv;               // levels lc .. L (+ L+1 if error_level)
-  HTransfer tv, tp;
-  XferOffsets xoff_v, xoff_p;
-  XferDev xv{}, xp{};
   Blob tables;
   size_t o_tables = 0, o_Z = 0, o_idx = 0, o_part = 0, o_scal = 0, total = 0;
   int ncoarse = 0;
@@ -322,8 +314,6 @@ extern "C" int hhg_problem_create(const hhg_mesh* mesh, const hhg_problem_desc* 
     for (int gg = 0; gg < pb->G; ++gg) lv.inv_diag.push_back(1.0 / lv.st.diagA[gg]);
     pb->lv.push_back(std::move(lv));
   }
-  pb->tv = build_transfer(pb->ov);
-  pb->tp = build_transfer(1);
 
   // ---- device table blob and specialised-kernel parameter blocks
   Blob& B = pb->tables;
@@ -386,28 +376,6 @@ extern "C" int hhg_problem_create(const hhg_mesh* mesh, const hhg_problem_desc* 
       of.bterms = B.put(h.bterms); of.bw64 = B.put(h.bw64); of.bw32 = B.put(bw32);
     }
   }
-  auto put_x = [&](const HTransfer& X, XferOffsets& xo) {
-    std::vector<int> ps(1, 0), rs(1, 0);
-    std::vector<DXTerm> pt, rt;
-    std::vector<double> pw, rw;
-    for (auto& c : X.prol) {
-      for (auto& t : c) { pt.push_back({t.arr, t.di, t.dj, t.dk}); pw.push_back(t.w); }
-      ps.push_back(int(pt.size()));
-    }
-    for (auto& c : X.restr) {
-      for (auto& t : c) { rt.push_back({t.arr, t.di, t.dj, t.dk}); rw.push_back(t.w); }
-      rs.push_back(int(rt.size()));
-    }
-    std::vector<float> pw32(pw.begin(), pw.end()), rw32(rw.begin(), rw.end());
-    xo.order = X.order; xo.nclass = X.nclass; xo.ngroups = int(X.restr.size());
-    xo.rmax = 0;
-    for (auto& c : X.restr) xo.rmax = std::max(xo.rmax, int(c.size()));
-    xo.pstart = B.put(ps); xo.pterms = B.put(pt); xo.pw64 = B.put(pw); xo.pw32 = B.put(pw32);
-    xo.rstart = B.put(rs); xo.rterms = B.put(rt); xo.rw64 = B.put(rw); xo.rw32 = B.put(rw32);
-  };
-  put_x(pb->tv, pb->xoff_v);
-  put_x(pb->tp, pb->xoff_p);
-
   // ---- workspace layout
   size_t off = 0;
   pb->o_tables = off;
@@ -813,8 +781,7 @@ template <class T>
 int restrict_to(hhg_problem* pb, int l, const T* rf, T* rc) {
   Level& f = pb->L(l);
   Level& c = pb->L(l - 1);
-  launch_restrict<T>(f.g, c.g, pb->xv, 0, 0, 3, pb->G, true, rf, rc, pb->stream);
-  launch_restrict<T>(f.g, c.g, pb->xp, 3 * pb->G, 3 * pb->G, 1, 1, false, rf, rc, pb->stream);
+  launch_restrict<T>(f.g, c.g, rf, rc, pb->stream);
   HHG_CHECK_LAUNCH();
   return HHG_OK;
 }
@@ -823,8 +790,7 @@ template <class T>
 int prolong_add(hhg_problem* pb, int l, const T* xc, T* xf, bool velocity_interior_only = true) {
   Level& f = pb->L(l);
   Level& c = pb->L(l - 1);
-  launch_prolong<T>(f.g, c.g, pb->xv, 0, 0, 3, pb->G, velocity_interior_only, xc, xf, pb->stream);
-  launch_prolong<T>(f.g, c.g, pb->xp, 3 * pb->G, 3 * pb->G, 1, 1, false, xc, xf, pb->stream);
+  launch_prolong<T>(f.g, c.g, velocity_interior_only, xc, xf, pb->stream);
   HHG_CHECK_LAUNCH();
   return HHG_OK;
 }
@@ -1173,22 +1139,6 @@ extern "C" int hhg_problem_bind(hhg_problem* pb, void* workspace, size_t bytes, 
     lv.inv_mlhat = reinterpret_cast<double*>(ws + lv.o_invml);
     lv.ml = reinterpret_cast<double*>(ws + lv.o_ml);
   }
-  auto xdev = [&](const XferOffsets& xo) {
-    XferDev X;
-    X.order = xo.order; X.nclass = xo.nclass; X.ngroups = xo.ngroups;
-    X.pcls_start = reinterpret_cast<const int*>(tb + xo.pstart);
-    X.pterms = reinterpret_cast<const DXTerm*>(tb + xo.pterms);
-    X.pw64 = reinterpret_cast<const double*>(tb + xo.pw64);
-    X.pw32 = reinterpret_cast<const float*>(tb + xo.pw32);
-    X.rg_start = reinterpret_cast<const int*>(tb + xo.rstart);
-    X.rterms = reinterpret_cast<const DXTerm*>(tb + xo.rterms);
-    X.rw64 = reinterpret_cast<const double*>(tb + xo.rw64);
-    X.rw32 = reinterpret_cast<const float*>(tb + xo.rw32);
-    X.rmax = xo.rmax;
-    return X;
-  };
-  pb->xv = xdev(pb->xoff_v);
-  pb->xp = xdev(pb->xoff_p);
   pb->Z = reinterpret_cast<double*>(ws + pb->o_Z);
   pb->cidx = reinterpret_cast<int64_t*>(ws + pb->o_idx);
   pb->partials = reinterpret_cast<double*>(ws + pb->o_part);

@@ -1,5 +1,5 @@
-// Constant per-macro stencils of the Stokes blocks on the Kuhn lattice and
-// the transfer tables (host side).
+// Constant per-macro stencils of the Stokes blocks on the Kuhn lattice (host
+// side).
 //
 // Sec. 2.1: after uniform refinement every micro tetrahedron is a translate
 // of one of six classes, so the stencil at every interior DoF of a group is
@@ -359,63 +359,6 @@ StencilSet build_stencils(int disc, double h, double nu_a, bool pspg_rhs) {
     S.op[OP_ML].rows.push_back(rML);
   }
   return S;
-}
-
-// ------------------------------------------------------------ transfers
-HTransfer build_transfer(int order) {
-  HTransfer X;
-  X.order = order;
-  const int G = order == 1 ? 1 : 8;
-  const int span = order == 1 ? 2 : 4;        // fine positions per coarse cell
-  X.nclass = span * span * span;
-  X.prol.assign(X.nclass, {});
-  X.restr.assign(G, {});
-  std::map<std::tuple<int, int, int, int, int>, double> rmap;   // (gc, gf, ex, ey, ez) -> w
-  for (int kz = 0; kz < span; ++kz)
-    for (int ky = 0; ky < span; ++ky)
-      for (int kx = 0; kx < span; ++kx) {
-        const int kap[3] = {kx, ky, kz};
-        const int cls = kx + span * (ky + span * kz);
-        double t[3] = {double(kx) / span, double(ky) / span, double(kz) / span};
-        // containing Kuhn tetrahedron: coordinates in descending order
-        int p[3] = {0, 1, 2};
-        std::stable_sort(p, p + 3, [&](int a, int b) { return t[a] > t[b]; });
-        std::array<double, 4> lam = {1 - t[p[0]], t[p[0]] - t[p[1]], t[p[1]] - t[p[2]], t[p[2]]};
-        int s = -1;
-        for (int m = 0; m < 6; ++m)
-          if (kPerm[m][0] == p[0] && kPerm[m][1] == p[1] && kPerm[m][2] == p[2]) s = m;
-        Tet tet = kuhn_tet(s);
-        std::vector<std::array<int, 3>> pos;
-        local_positions(tet, order, pos);
-        std::vector<double> phi;
-        std::vector<std::array<double, 4>> dphi;
-        basis(order, lam, phi, dphi);
-        // fine group of this class
-        int of[3], gf;
-        if (order == 2) {
-          for (int d = 0; d < 3; ++d) of[d] = kap[d] & 1;
-          gf = group_of_parity(of[0], of[1], of[2]);
-        } else {
-          of[0] = of[1] = of[2] = 0;
-          gf = 0;
-        }
-        for (size_t a = 0; a < pos.size(); ++a) {
-          if (std::fabs(phi[a]) < 1e-14) continue;
-          int oc[3] = {pos[a][0] & 1, pos[a][1] & 1, pos[a][2] & 1};
-          int gc = group_of_parity(oc[0], oc[1], oc[2]);
-          int dl[3] = {(pos[a][0] - oc[0]) / 2, (pos[a][1] - oc[1]) / 2, (pos[a][2] - oc[2]) / 2};
-          X.prol[cls].push_back({gc, dl[0], dl[1], dl[2], phi[a]});
-          int e[3];
-          for (int d = 0; d < 3; ++d) e[d] = order == 2 ? -2 * dl[d] + (kap[d] - of[d]) / 2 : -2 * dl[d] + kap[d];
-          rmap[{gc, gf, e[0], e[1], e[2]}] += phi[a];
-        }
-      }
-  for (auto& kv : rmap) {
-    int gc = std::get<0>(kv.first);
-    X.restr[gc].push_back({std::get<1>(kv.first), std::get<2>(kv.first), std::get<3>(kv.first),
-                           std::get<4>(kv.first), kv.second});
-  }
-  return X;
 }
 
 }  // namespace hhg

@@ -1,0 +1,304 @@
+// Transfers between two levels (Sec. 3.3): x_f += I x_c and r_c = I^T r_f with
+// the nodal (linear P1, quadratic P2) interpolation of the Kuhn lattice.
+//
+// The interpolation is the same in every coarse lattice cell: a fine DoF at
+// doubled fine position 4 a + p (a the cell, 0 <= p_d < 4; P1: 2 a + p,
+// 0 <= p_d < 2) reads the 27 (8) coarse nodes of its cell with weights that
+// depend on p only.  The weights are evaluated at compile time and every
+// row is unrolled over its non-zero ones, so that no table is read:
+//  * prolongation: one thread owns one coarse cell and one z position p_z of
+//    it, loads the coarse nodes once and updates 16 fine DoFs of a component
+//    (P1 fields: all 8 of the cell);
+//  * restriction: one thread gathers one coarse DoF of one group (the blocks
+//    of a launch that run at the same time share the fine planes they read).
+// All components, groups and the pressure go in one launch (grid z).
+//
+// Bound: HBM on the large levels (the fine vector is read and written, or
+// read, once), launch latency on the small ones.  The table-driven kernels
+// these replace read a weight and an offset per term from memory (dependent
+// loads), divided a row's terms over lanes and took two launches each.
+// Measured (FP32, P2-P1, 2x1x1 cubes at level 6, restriction and prolongation):
+// 248 us before, 79 us now; their vectors once over HBM would take 26 us.
+#include <cuda_runtime.h>
+
+#include <type_traits>
+#include <utility>
+
+#include "batch.h"
+#include "kernels.h"
+
+namespace hhg {
+namespace {
+
+// weight of the coarse node at doubled position (nx, ny, nz) (0..2) of a cell
+// at the point with coordinates (px, py, pz) / 4 of the cell, quadratic
+// interpolation on the Kuhn tetrahedron that holds the point: the tetrahedron
+// 0 -> e_a -> e_a + e_b -> (1, 1, 1) of the coordinates in descending order
+constexpr double p2_weight(int px, int py, int pz, int nx, int ny, int nz) {
+  const int p[3] = {px, py, pz};
+  int o[3] = {0, 1, 2};
+  for (int r = 0; r < 2; ++r)                      // stable sort, descending
+    for (int s = 0; s < 2; ++s)
+      if (p[o[s]] < p[o[s + 1]]) {
+        const int t = o[s];
+        o[s] = o[s + 1];
+        o[s + 1] = t;
+      }
+  const double lam[4] = {(4 - p[o[0]]) / 4.0, (p[o[0]] - p[o[1]]) / 4.0, (p[o[1]] - p[o[2]]) / 4.0, p[o[2]] / 4.0};
+  int v[4][3] = {};
+  for (int s = 0; s < 3; ++s)
+    for (int d = 0; d < 3; ++d) v[s + 1][d] = v[s][d] + (d == o[s] ? 1 : 0);
+  for (int a = 0; a < 4; ++a)
+    for (int b = a; b < 4; ++b)
+      if (v[a][0] + v[b][0] == nx && v[a][1] + v[b][1] == ny && v[a][2] + v[b][2] == nz)
+        return a == b ? lam[a] * (2 * lam[a] - 1) : 4 * lam[a] * lam[b];
+  return 0.0;
+}
+// group of a parity offset (order of kGroupOff)
+constexpr int group_at(int ox, int oy, int oz) {
+  constexpr int g[8] = {0, 1, 2, 4, 3, 5, 6, 7};
+  return g[ox | oy << 1 | oz << 2];
+}
+
+__device__ __forceinline__ int64_t xsite(const Geo& g, int i, int j, int k) {
+  return int64_t(i + 1) + int64_t(j + 1) * g.sx + int64_t(k + 1) * g.sy;
+}
+
+// ------------------------------------------------------------- prolongation
+template <int PX, int PY, int PZ, int NZ, class T, int... N>
+__device__ __forceinline__ T p2_point(const T (&c)[NZ * 9], std::integer_sequence<int, N...>) {
+  T a = T(0);
+  ([&] {
+    constexpr double w = p2_weight(PX, PY, PZ, N % 3, N / 3 % 3, N / 9);
+    if constexpr (w != 0.0) a = fma(T(w), c[N], a);
+  }(), ...);
+  return a;
+}
+
+// the 16 fine DoFs of one component at z position PZ of coarse cell (ax, ay, az)
+template <int PZ, class T, int... Q>
+__device__ __forceinline__ void prolong_p2(const Geo& gf, const Geo& gc, int ax, int ay, int az, bool interior_only,
+                                           const T* __restrict__ xc, T* __restrict__ xf,
+                                           std::integer_sequence<int, Q...>) {
+  constexpr int NZ = PZ == 0 ? 1 : 3;
+  T c[NZ * 9];
+  const T* x0 = xc + xsite(gc, ax, ay, az);
+#pragma unroll
+  for (int n = 0; n < NZ * 9; ++n) {
+    const int nx = n % 3, ny = n / 3 % 3, nz = n / 9;
+    c[n] = __ldg(x0 + group_at(nx & 1, ny & 1, nz & 1) * gc.arr + (nx >> 1) + (ny >> 1) * gc.sx + (nz >> 1) * gc.sy);
+  }
+  // doubled fine position of the point and its range: 1 .. 2 n - 1 inside
+  const int lo = interior_only ? 1 : 0;
+  const int Pz = 4 * az + PZ;
+  if (Pz < lo || Pz > 2 * gf.nz - lo) return;
+  T* f0 = xf + xsite(gf, 2 * ax, 2 * ay, 2 * az);
+  auto at = [&](auto qc) {
+    constexpr int q = decltype(qc)::value, PX = q % 4, PY = q / 4;
+    const int Px = 4 * ax + PX, Py = 4 * ay + PY;
+    if (Px < lo || Px > 2 * gf.nx - lo || Py < lo || Py > 2 * gf.ny - lo) return;
+    T* f = f0 + group_at(PX & 1, PY & 1, PZ & 1) * gf.arr + (PX >> 1) + (PY >> 1) * gf.sx + (PZ >> 1) * gf.sy;
+    *f += p2_point<PX, PY, PZ, NZ>(c, std::make_integer_sequence<int, NZ * 9>{});
+  };
+  (at(std::integral_constant<int, Q>{}), ...);
+}
+
+// the 8 fine DoFs of one P1 field in coarse cell (ax, ay, az)
+template <class T>
+__device__ __forceinline__ void prolong_p1(const Geo& gf, const Geo& gc, int ax, int ay, int az, bool interior_only,
+                                           const T* __restrict__ xc, T* __restrict__ xf) {
+  T c[8];
+  const T* x0 = xc + xsite(gc, ax, ay, az);
+#pragma unroll
+  for (int n = 0; n < 8; ++n) c[n] = __ldg(x0 + (n & 1) + (n >> 1 & 1) * gc.sx + (n >> 2) * gc.sy);
+  const int lo = interior_only ? 1 : 0;
+  T* f0 = xf + xsite(gf, 2 * ax, 2 * ay, 2 * az);
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    const int px = q & 1, py = q >> 1 & 1, pz = q >> 2;
+    const int i = 2 * ax + px, j = 2 * ay + py, k = 2 * az + pz;
+    if (i < lo || i > gf.nx - lo || j < lo || j > gf.ny - lo || k < lo || k > gf.nz - lo) continue;
+    f0[px + py * gf.sx + pz * gf.sy] += q == 0 ? c[0] : T(0.5) * c[0] + T(0.5) * c[q];
+  }
+}
+
+// arguments of both transfers (in: coarse and out: fine for the prolongation,
+// the other way round for the restriction); interior_only: Dirichlet velocity
+// DoFs are left as they are
+template <class T>
+struct TransferA { Geo gf, gc; int interior_only; const T* in; T* out; };
+
+// grid: x over the (i, j) plane of coarse cells (flat), z = plane and part
+// (part fastest: blocks that run together share the coarse planes)
+template <int G, class T>
+__device__ __forceinline__ void prolong_body(const uint3 bid, const TransferA<T>& a) {
+  constexpr int NPART = G == 8 ? 13 : 4;
+  const Geo &gf = a.gf, &gc = a.gc;
+  const int az = int(bid.z) / NPART, part = int(bid.z) - az * NPART;
+  const int w = gc.nx + 1, q = bid.x * blockDim.x + threadIdx.x;
+  const int ay = q / w, ax = q - ay * w;
+  if (ay > gc.ny) return;
+  const bool io = a.interior_only != 0;
+  if constexpr (G == 1) {
+    prolong_p1<T>(gf, gc, ax, ay, az, io && part < 3, a.in + part * gc.arr, a.out + part * gf.arr);
+  } else {
+    if (part == 12) return prolong_p1<T>(gf, gc, ax, ay, az, false, a.in + 24 * gc.arr, a.out + 24 * gf.arr);
+    const int comp = part >> 2;
+    const T* xc = a.in + comp * 8 * gc.arr;
+    T* xf = a.out + comp * 8 * gf.arr;
+    const auto all = std::make_integer_sequence<int, 16>{};
+    switch (part & 3) {
+      case 0: prolong_p2<0>(gf, gc, ax, ay, az, io, xc, xf, all); break;
+      case 1: prolong_p2<1>(gf, gc, ax, ay, az, io, xc, xf, all); break;
+      case 2: prolong_p2<2>(gf, gc, ax, ay, az, io, xc, xf, all); break;
+      default: prolong_p2<3>(gf, gc, ax, ay, az, io, xc, xf, all); break;
+    }
+  }
+}
+
+// --------------------------------------------------------------- restriction
+// weight with which the coarse node of parity offset O reads the fine node at
+// doubled fine distance e from it (|e| <= 3): the fine node lies in the cell
+// b = floor((2 o + e) / 4) at position p = (2 o + e) mod 4
+constexpr int cell_of(int t) { return t < 0 ? -1 : t / 4; }
+constexpr double p2_restrict_weight(int ox, int oy, int oz, int ex, int ey, int ez) {
+  const int bx = cell_of(2 * ox + ex), by = cell_of(2 * oy + ey), bz = cell_of(2 * oz + ez);
+  return p2_weight(2 * ox + ex - 4 * bx, 2 * oy + ey - 4 * by, 2 * oz + ez - 4 * bz, ox - 2 * bx, oy - 2 * by,
+                   oz - 2 * bz);
+}
+
+// sum over the fine nodes around coarse node (2 a + o); f0: the fine vertex at
+// the node's cell, i.e. doubled fine position 4 a
+template <int OX, int OY, int OZ, class T, int... E>
+__device__ __forceinline__ T restrict_p2(const Geo& gf, const T* __restrict__ f0, std::integer_sequence<int, E...>) {
+  T s[2] = {T(0), T(0)};                           // two chains
+  ([&] {
+    constexpr int ex = E % 7 - 3, ey = E / 7 % 7 - 3, ez = E / 49 - 3;
+    constexpr double w = p2_restrict_weight(OX, OY, OZ, ex, ey, ez);
+    if constexpr (w != 0.0) {
+      // doubled fine position relative to 4 a; arithmetic shift = floor
+      constexpr int rx = 2 * OX + ex, ry = 2 * OY + ey, rz = 2 * OZ + ez;
+      constexpr int grp = group_at(rx & 1, ry & 1, rz & 1);
+      s[E & 1] = fma(T(w), __ldg(f0 + grp * gf.arr + (rx >> 1) + (ry >> 1) * gf.sx + (rz >> 1) * gf.sy), s[E & 1]);
+    }
+  }(), ...);
+  return s[0] + s[1];
+}
+
+template <class T>
+__device__ __forceinline__ T restrict_p1(const Geo& gf, const T* __restrict__ f) {
+  T s = T(0);
+#pragma unroll
+  for (int q = 1; q < 8; ++q) {
+    const int d = (q & 1) + (q >> 1 & 1) * gf.sx + (q >> 2) * int(gf.sy);
+    s += __ldg(f + d) + __ldg(f - d);
+  }
+  return fma(T(0.5), s, __ldg(f));
+}
+
+template <int GRP, class T>
+__device__ __forceinline__ void restrict_group(const Geo& gf, const Geo& gc, int i, int j, int k, const T* rf, T* rc) {
+  constexpr int ox = kGroupOff[GRP][0], oy = kGroupOff[GRP][1], oz = kGroupOff[GRP][2];
+  if (i > gc.nx - ox || j > gc.ny - oy || k > gc.nz - oz) return;
+  const int Px = 2 * i + ox, Py = 2 * j + oy, Pz = 2 * k + oz;
+  const bool inside = Px > 0 && Py > 0 && Pz > 0 && Px < 2 * gc.nx && Py < 2 * gc.ny && Pz < 2 * gc.nz;
+  T v = T(0);
+  if (inside)
+    v = restrict_p2<ox, oy, oz>(gf, rf + xsite(gf, 2 * i, 2 * j, 2 * k), std::make_integer_sequence<int, 343>{});
+  rc[GRP * gc.arr + xsite(gc, i, j, k)] = v;
+}
+
+// grid: as the prolongation's, over the coarse sites; a part is one group of
+// one component, or the pressure
+template <int G, class T>
+__device__ __forceinline__ void restrict_body(const uint3 bid, const TransferA<T>& a) {
+  constexpr int NPART = 3 * G + 1;
+  const Geo &gf = a.gf, &gc = a.gc;
+  const int k = int(bid.z) / NPART, part = int(bid.z) - k * NPART;
+  const int w = gc.nx + 1, q = bid.x * blockDim.x + threadIdx.x;
+  const int j = q / w, i = q - j * w;
+  if (j > gc.ny) return;
+  if (G == 1 || part == 3 * G) {
+    const bool zero = part < 3 * G && (i == 0 || j == 0 || k == 0 || i == gc.nx || j == gc.ny || k == gc.nz);
+    T v = T(0);
+    if (!zero) v = restrict_p1<T>(gf, a.in + part * gf.arr + xsite(gf, 2 * i, 2 * j, 2 * k));
+    a.out[part * gc.arr + xsite(gc, i, j, k)] = v;
+  } else {
+    const int comp = part >> 3;
+    const T* rf = a.in + comp * 8 * gf.arr;
+    T* rc = a.out + comp * 8 * gc.arr;
+    switch (part & 7) {
+      case 0: restrict_group<0>(gf, gc, i, j, k, rf, rc); break;
+      case 1: restrict_group<1>(gf, gc, i, j, k, rf, rc); break;
+      case 2: restrict_group<2>(gf, gc, i, j, k, rf, rc); break;
+      case 3: restrict_group<3>(gf, gc, i, j, k, rf, rc); break;
+      case 4: restrict_group<4>(gf, gc, i, j, k, rf, rc); break;
+      case 5: restrict_group<5>(gf, gc, i, j, k, rf, rc); break;
+      case 6: restrict_group<6>(gf, gc, i, j, k, rf, rc); break;
+      default: restrict_group<7>(gf, gc, i, j, k, rf, rc); break;
+    }
+  }
+}
+
+template <int G, class T>
+__global__ void __launch_bounds__(128) k_prolong(const __grid_constant__ TransferA<T> a) {
+  prolong_body<G, T>(blockIdx, a);
+}
+template <int G, class T>
+__global__ void __launch_bounds__(128) k_restrict(const __grid_constant__ TransferA<T> a) {
+  restrict_body<G, T>(blockIdx, a);
+}
+template <int G, class T>
+__global__ void __launch_bounds__(128) kb_prolong(const void* items, int n) {
+  uint3 bid, gd;
+  const auto& it = batch_item<TransferA<T>>(items, n, bid, gd);
+  prolong_body<G, T>(bid, it.a);
+}
+template <int G, class T>
+__global__ void __launch_bounds__(128) kb_restrict(const void* items, int n) {
+  uint3 bid, gd;
+  const auto& it = batch_item<TransferA<T>>(items, n, bid, gd);
+  restrict_body<G, T>(bid, it.a);
+}
+
+template <class T>
+void launch(const void* kernel, const void* batched, dim3 grd, const TransferA<T>& a, cudaStream_t s) {
+  const dim3 blk(128, 1, 1);
+  if (g_rec) return g_rec->add(batched, grd, blk, 0, 1, a);
+  ++g_launches;
+  void* args[] = {const_cast<TransferA<T>*>(&a)};
+  cudaLaunchKernel(kernel, grd, blk, args, 0, s);
+}
+inline unsigned plane_blocks(const Geo& gc) { return unsigned(((gc.nx + 1) * (gc.ny + 1) + 127) / 128); }
+
+}  // namespace
+
+template <class T>
+void launch_prolong(const Geo& gf, const Geo& gc, bool interior_only, const T* xc, T* xf, cudaStream_t s) {
+  const TransferA<T> a{gf, gc, interior_only ? 1 : 0, xc, xf};
+  if (gf.G == 1)
+    launch<T>(reinterpret_cast<const void*>(k_prolong<1, T>), reinterpret_cast<const void*>(kb_prolong<1, T>),
+              dim3(plane_blocks(gc), 1, (gc.nz + 1) * 4), a, s);
+  else
+    launch<T>(reinterpret_cast<const void*>(k_prolong<8, T>), reinterpret_cast<const void*>(kb_prolong<8, T>),
+              dim3(plane_blocks(gc), 1, (gc.nz + 1) * 13), a, s);
+}
+
+template <class T>
+void launch_restrict(const Geo& gf, const Geo& gc, const T* rf, T* rc, cudaStream_t s) {
+  const TransferA<T> a{gf, gc, 1, rf, rc};
+  if (gf.G == 1)
+    launch<T>(reinterpret_cast<const void*>(k_restrict<1, T>), reinterpret_cast<const void*>(kb_restrict<1, T>),
+              dim3(plane_blocks(gc), 1, (gc.nz + 1) * 4), a, s);
+  else
+    launch<T>(reinterpret_cast<const void*>(k_restrict<8, T>), reinterpret_cast<const void*>(kb_restrict<8, T>),
+              dim3(plane_blocks(gc), 1, (gc.nz + 1) * 25), a, s);
+}
+
+#define HHG_INST(T)                                                                               \
+  template void launch_prolong<T>(const Geo&, const Geo&, bool, const T*, T*, cudaStream_t);      \
+  template void launch_restrict<T>(const Geo&, const Geo&, const T*, T*, cudaStream_t);
+HHG_INST(double)
+HHG_INST(float)
+
+}  // namespace hhg

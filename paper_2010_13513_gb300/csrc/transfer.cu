@@ -171,7 +171,7 @@ constexpr double p2_restrict_weight(int ox, int oy, int oz, int ex, int ey, int 
 // the node's cell, i.e. doubled fine position 4 a
 template <int OX, int OY, int OZ, class T, int... E>
 __device__ __forceinline__ T restrict_p2(const Geo& gf, const T* __restrict__ f0, std::integer_sequence<int, E...>) {
-  T s[2] = {T(0), T(0)};                           // two chains
+  T s[8] = {};                                     // eight chains: short sums, independent latencies
   ([&] {
     constexpr int ex = E % 7 - 3, ey = E / 7 % 7 - 3, ez = E / 49 - 3;
     constexpr double w = p2_restrict_weight(OX, OY, OZ, ex, ey, ez);
@@ -179,10 +179,10 @@ __device__ __forceinline__ T restrict_p2(const Geo& gf, const T* __restrict__ f0
       // doubled fine position relative to 4 a; arithmetic shift = floor
       constexpr int rx = 2 * OX + ex, ry = 2 * OY + ey, rz = 2 * OZ + ez;
       constexpr int grp = group_at(rx & 1, ry & 1, rz & 1);
-      s[E & 1] = fma(T(w), __ldg(f0 + grp * gf.arr + (rx >> 1) + (ry >> 1) * gf.sx + (rz >> 1) * gf.sy), s[E & 1]);
+      s[E & 7] = fma(T(w), __ldg(f0 + grp * gf.arr + (rx >> 1) + (ry >> 1) * gf.sx + (rz >> 1) * gf.sy), s[E & 7]);
     }
   }(), ...);
-  return s[0] + s[1];
+  return ((s[0] + s[1]) + (s[2] + s[3])) + ((s[4] + s[5]) + (s[6] + s[7]));
 }
 
 template <class T>

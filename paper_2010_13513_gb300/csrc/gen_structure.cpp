@@ -153,6 +153,7 @@ void print_stream_plan(int disc, int varnu, int op, const HOperator& O) {
 int main() {
   std::printf("// generated by gen_structure.cpp -- do not edit\n#pragma once\nnamespace hhg {\nnamespace gen {\n");
   std::printf("struct RowS { int out, og, all, t0, n0, n1, n2; };\n");
+  std::printf("struct OffT { int arr, di, dj, dk; };\n");
   std::printf("template <int DISC, int VARNU, int OP> struct S;\n");
   // streaming-kernel plan (stream.cu): passes over staged input arrays
   std::printf("struct PassT { int a0, na, p0, np, l0, nl; };\n");
@@ -177,7 +178,24 @@ int main() {
           std::printf("%s{%d, %d, %d, %d, %d, %d, %d}", r ? ", " : "", R.out_arr, R.og, R.all_rows ? 1 : 0, t, n0, n1, n2);
           t += n0 + n1 + n2;
         }
-        std::printf("};\n  static constexpr int N = %d;\n};\n", t);
+        std::printf("};\n  static constexpr int N = %d;\n", t);
+        // input array and lattice offset of every term, and (constant
+        // viscosity) its weight at h = 1, in weight index order
+        std::printf("  static constexpr OffT off[%d] = {", t);
+        int n = 0;
+        for (const HRow& R : O.rows)
+          for (const auto& sg : R.seg)
+            for (const HTerm& h : sg) std::printf("%s{%d, %d, %d, %d}", n++ ? ", " : "", h.in_arr, h.di, h.dj, h.dk);
+        std::printf("};\n");
+        if (!varnu) {
+          n = 0;
+          std::printf("  static constexpr double wref[%d] = {", t);
+          for (const HRow& R : O.rows)
+            for (const auto& sg : R.seg)
+              for (const HTerm& h : sg) std::printf("%s%.17g", n++ ? ", " : "", h.w);
+          std::printf("};\n");
+        }
+        std::printf("};\n");
         if (op == OP_A) continue;
         print_stream_plan(disc, varnu, op, O);
       }

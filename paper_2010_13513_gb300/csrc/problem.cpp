@@ -134,9 +134,11 @@ struct Level {
   // parameter blocks of the streaming kernels (FULL, B^T, (B, -C))
   std::vector<char> stab64[OP_COUNT], stab32[OP_COUNT];
   bool has_stream[OP_COUNT] = {};
-  // parameter blocks (ResTabs images) of the shared-memory-resident
-  // smoother, per CTA count (the offsets depend on the slab stride)
-  std::map<int, std::vector<char>> rtab64, rtab32;
+  // weight tables (ResTabs) of the shared-memory-resident smoother: offsets
+  // in the table blob, device addresses
+  size_t o_rtab64 = 0, o_rtab32 = 0;
+  const ResTabs<double>* rtab64 = nullptr;
+  const ResTabs<float>* rtab32 = nullptr;
   int rctas[2] = {0, 0};                // CTAs of the resident smoother per precision (0: per-phase kernels)
   int rthreads[2] = {kResidentThreads, kResidentThreads};   // and threads per CTA
   Shape shape;                          // launch shapes of the specialised kernels
@@ -292,6 +294,32 @@ extern "C" int hhg_mesh_destroy(hhg_mesh* mesh) {
 }
 
 // ================================================================= problems
+namespace {
+// the resident smoother's weight table of a level, in the table blob: the
+// rows of A of component 0, of B^T and of (B, -C), and the clipped C stencils
+template <class T>
+int put_res_tabs(Blob& B, const Level& lv, const std::vector<double>& wc, size_t& off) {
+  std::vector<ResTabs<T>> rt(1);
+  std::memset(static_cast<void*>(rt.data()), 0, sizeof(ResTabs<T>));
+  size_t n = 0;
+  bool ok = wc.size() <= sizeof(rt[0].wc) / sizeof(T);
+  for (int op : {OP_A, OP_BT, OP_BC}) {
+    const std::vector<HRow>& rows = lv.st.op[op].rows;
+    const size_t nr = op == OP_A ? rows.size() / 3 : rows.size();
+    for (size_t r = 0; r < nr; ++r)
+      for (const auto& sg : rows[r].seg)
+        for (const HTerm& t : sg) {
+          ok = ok && n < size_t(kResMaxTerms);
+          if (ok) rt[0].w[n++] = T(t.w);
+        }
+  }
+  if (!ok) return fail(HHG_EINVAL, "internal: stencil tables do not fit the resident smoother");
+  for (size_t q = 0; q < wc.size(); ++q) rt[0].wc[q] = T(wc[q]);
+  off = B.put(rt);
+  return HHG_OK;
+}
+}  // namespace
+
 extern "C" int hhg_problem_create(const hhg_mesh* mesh, const hhg_problem_desc* desc, hhg_problem** out) {
   if (!mesh || !desc || !out) return fail(HHG_EINVAL, "hhg_problem_create: null argument");
   if (desc->disc != HHG_P1P1_PSPG && desc->disc != HHG_P2P1_TH) return fail(HHG_EINVAL, "unknown discretisation");
@@ -319,6 +347,7 @@ extern "C" int hhg_problem_create(const hhg_mesh* mesh, const hhg_problem_desc* 
   Blob& B = pb->tables;
   const int varnu = desc->nu_a != 0.0 ? 1 : 0;
   for (Level& lv : pb->lv) {
+    std::vector<double> wc_bc;            // clipped C stencils of the (B, -C) row
     for (int o = 0; o < OP_COUNT; ++o) {
       OpHost h = serialise(lv.st.op[o], lv.g);
       const int N = fast_terms(desc->disc, varnu, o);
@@ -366,6 +395,7 @@ extern "C" int hhg_problem_create(const hhg_mesh* mesh, const hhg_problem_desc* 
                 if (in) wc[size_t(cls) * ncb + slot] += t.w;
               }
             }
+        if (o == OP_BC) wc_bc = wc;
         lv.has_stream[o] = stream_image<double>(desc->disc, varnu, o, h.w64, wc, lv.stab64[o]) &&
                            stream_image<float>(desc->disc, varnu, o, h.w64, wc, lv.stab32[o]);
       }
@@ -375,6 +405,8 @@ extern "C" int hhg_problem_create(const hhg_mesh* mesh, const hhg_problem_desc* 
       of.rows = B.put(h.rows); of.terms = B.put(h.terms); of.w64 = B.put(h.w64); of.w32 = B.put(w32);
       of.bterms = B.put(h.bterms); of.bw64 = B.put(h.bw64); of.bw32 = B.put(bw32);
     }
+    HHG_TRY(put_res_tabs<double>(B, lv, wc_bc, lv.o_rtab64));
+    HHG_TRY(put_res_tabs<float>(B, lv, wc_bc, lv.o_rtab32));
   }
   // ---- workspace layout
   size_t off = 0;
@@ -620,63 +652,9 @@ double level_weight(hhg_problem* pb, const Level& lv) {
 }
 
 template <class T> constexpr int prec_index() { return sizeof(T) == 8 ? HHG_FP64 : HHG_FP32; }
-template <class T> const ResTabs<T>& rtab(Level& lv, int C);
-template <> const ResTabs<double>& rtab<double>(Level& lv, int C) {
-  return *reinterpret_cast<const ResTabs<double>*>(lv.rtab64.at(C).data());
-}
-template <> const ResTabs<float>& rtab<float>(Level& lv, int C) {
-  return *reinterpret_cast<const ResTabs<float>*>(lv.rtab32.at(C).data());
-}
-
-// true if a linear offset di + dj sx + dk sy reaches only adjacent sites
-bool adjacent(const Geo& g, int64_t off) {
-  const int64_t dk = std::llround(double(off) / double(g.sy));
-  const int64_t dj = std::llround(double(off - dk * g.sy) / double(g.sx));
-  const int64_t di = off - dk * g.sy - dj * g.sx;
-  return dk >= -1 && dk <= 1 && dj >= -1 && dj <= 1 && di >= -1 && di <= 1;
-}
-
-// the resident smoother's parameter block for slab stride arr_l: rows and
-// terms of A (component 0 of each group), B^T and (B, -C) from the level's
-// stencil tables, offsets rewritten to the slab stride
-template <class T>
-int build_res_tabs(hhg_problem* pb, Level& lv, int64_t arr_l, std::vector<char>& out) {
-  out.assign(sizeof(ResTabs<T>), 0);
-  ResTabs<T>& rt = *reinterpret_cast<ResTabs<T>*>(out.data());
-  const int G = lv.g.G;
-  rt.G = G;
-  rt.nbt = 3 * G;
-  rt.varnu = pb->desc.nu_a != 0.0 ? 1 : 0;
-  const char* blob = pb->tables.bytes.data();
-  int nw = 0;
-  auto add = [&](int op, int r, ResRow& dst) {
-    const OpOffsets& of = lv.opoff[op];
-    if (r >= of.nrows) return false;
-    const DRow& d = reinterpret_cast<const DRow*>(blob + of.rows)[r];
-    const DTerm* terms = reinterpret_cast<const DTerm*>(blob + of.terms);
-    const double* w = reinterpret_cast<const double*>(blob + of.w64);
-    const int n = d.n0 + d.n1 + d.n2;
-    if (nw + n > kResMaxTerms) return false;
-    dst = ResRow{d.out_arr, d.og, d.all_rows, nw, d.n0, d.n1, d.n2, d.b0 + d.m0 + d.m1, d.m2};
-    for (int t = d.t0; t < d.t0 + n; ++t) {
-      if (terms[t].arr < 0 || terms[t].arr > 3 * G || !adjacent(lv.g, terms[t].off)) return false;
-      rt.w[nw] = T(w[t]);
-      rt.off[nw] = int(terms[t].arr * arr_l + terms[t].off);
-      ++nw;
-    }
-    return true;
-  };
-  bool ok = G <= 8 && 3 * G <= kResMaxRows;
-  for (int gg = 0; ok && gg < G; ++gg) {
-    ok = add(OP_A, gg, rt.A[gg]);
-    ok = ok && rt.A[gg].n0 == 0 && rt.A[gg].n2 == 0 && rt.A[gg].n1 > 0;   // diagonal first, all in segment 1
-  }
-  for (int r = 0; ok && r < 3 * G; ++r) ok = add(OP_BT, r, rt.BT[r]);
-  ok = ok && add(OP_BC, 0, rt.BC);
-  if (!ok) return fail(HHG_EINVAL, "internal: stencil tables do not fit the resident smoother");
-  rt.nw = nw;
-  return HHG_OK;
-}
+template <class T> const ResTabs<T>* rtab(const Level& lv);
+template <> const ResTabs<double>* rtab<double>(const Level& lv) { return lv.rtab64; }
+template <> const ResTabs<float>* rtab<float>(const Level& lv) { return lv.rtab32; }
 
 // selects `ctas` CTAs (0: per-phase kernels) for the resident smoother of a
 // level in precision `prec`; HHG_EINVAL if the level does not fit
@@ -685,28 +663,8 @@ int set_resident(hhg_problem* pb, Level& lv, int prec, int ctas, int threads = k
   if (threads < 128 || threads > kResidentThreads || threads % 32)
     return fail(HHG_EINVAL, "threads must be a multiple of 32 in 128..1024");
   if (ctas > 0) {
-    if (!resident_feasible(prec, lv.g, ctas))
+    if (!resident_feasible(pb->desc.disc, pb->desc.nu_a != 0.0 ? 1 : 0, prec, lv.g, ctas))
       return fail(HHG_EINVAL, "level does not fit the shared memory of that many CTAs");
-    // the per-cube boundary terms of (B, -C) must stay within the adjacent
-    // sites, as the slab holds one halo plane on each side
-    const OpOffsets& of = lv.opoff[OP_BC];
-    const DRow* rows = reinterpret_cast<const DRow*>(pb->tables.bytes.data() + of.rows);
-    const DTermB* bt = reinterpret_cast<const DTermB*>(pb->tables.bytes.data() + of.bterms);
-    for (int r = 0; r < of.nrows; ++r)
-      for (int t = rows[r].b0; t < rows[r].b0 + rows[r].m0 + rows[r].m1 + rows[r].m2; ++t) {
-        const int64_t dk = std::llround(double(bt[t].off) / double(lv.g.sy));
-        const int64_t dj = std::llround(double(bt[t].off - dk * lv.g.sy) / double(lv.g.sx));
-        const int64_t di = bt[t].off - dk * lv.g.sy - dj * lv.g.sx;
-        if (bt[t].arr < 0 || bt[t].arr > 3 * lv.g.G || dk < -1 || dk > 1 || dj < -1 || dj > 1 || di < -1 || di > 1)
-          return fail(HHG_EINVAL, "internal: boundary stencil offsets beyond adjacent sites");
-      }
-    auto& cache = prec == HHG_FP64 ? lv.rtab64 : lv.rtab32;
-    if (!cache.count(ctas)) {
-      std::vector<char> img;
-      if (prec == HHG_FP64) HHG_TRY(build_res_tabs<double>(pb, lv, resident_arr(lv.g, ctas), img));
-      else HHG_TRY(build_res_tabs<float>(pb, lv, resident_arr(lv.g, ctas), img));
-      cache[ctas] = std::move(img);
-    }
   }
   lv.rctas[prec] = ctas;
   lv.rthreads[prec] = threads;
@@ -718,7 +676,7 @@ int set_resident(hhg_problem* pb, Level& lv, int prec, int ctas, int threads = k
 int default_resident(hhg_problem* pb, Level& lv, int prec) {
   const int64_t plane = int64_t(lv.g.nx + 1) * (lv.g.ny + 1), nzp = lv.g.nz + 1;
   for (int C : {1, 2, 4, 8})
-    if (plane * ((nzp + C - 1) / C) <= 8192 && resident_feasible(prec, lv.g, C))
+    if (plane * ((nzp + C - 1) / C) <= 8192 && resident_feasible(pb->desc.disc, pb->desc.nu_a != 0.0 ? 1 : 0, prec, lv.g, C))
       return set_resident(pb, lv, prec, C);
   return set_resident(pb, lv, prec, 0);
 }
@@ -736,8 +694,8 @@ int uzawa(hhg_problem* pb, Level& lv, const hhg_params& prm, int sweeps, T* x, c
     a.ahat = prm.ahat;
     a.inv_omega_inv = 1.0 / prm.omega_inv;
     for (int gg = 0; gg < G; ++gg) a.inv_diag[gg] = lv.inv_diag[gg];
-    if (uzawa_resident<T>(lv.g, C, lv.rthreads[prec_index<T>()], x, b, lv.inv_mlhat, a, lv.op[OP_BC], rtab<T>(lv, C),
-                          pb->stream) != 0)
+    if (uzawa_resident<T>(pb->desc.disc, pb->desc.nu_a != 0.0 ? 1 : 0, lv.g, C, lv.rthreads[prec_index<T>()], x, b,
+                          lv.inv_mlhat, a, rtab<T>(lv), pb->stream) != 0)
       return fail(HHG_ECUDA, std::string("resident smoother launch: ") + cudaGetErrorString(cudaGetLastError()));
     const Costs cs = block_costs(pb->ov);
     pb->wu_counted += sweeps * level_weight(pb, lv) * (prm.xi * (prm.ahat == HHG_AHAT_S ? 2 : 1) * cs.A + 2 * cs.B + cs.C);
@@ -1136,6 +1094,8 @@ extern "C" int hhg_problem_bind(hhg_problem* pb, void* workspace, size_t bytes, 
       lv.b32 = reinterpret_cast<float*>(ws + lv.o_b32);
       lv.tmp32 = reinterpret_cast<float*>(ws + lv.o_tmp32);
     }
+    lv.rtab64 = reinterpret_cast<const ResTabs<double>*>(tb + lv.o_rtab64);
+    lv.rtab32 = reinterpret_cast<const ResTabs<float>*>(tb + lv.o_rtab32);
     lv.inv_mlhat = reinterpret_cast<double*>(ws + lv.o_invml);
     lv.ml = reinterpret_cast<double*>(ws + lv.o_ml);
   }
@@ -2077,7 +2037,7 @@ int tune_smoother(hhg_problem* pb, Level& lv, int reps, T* x, const T* b, T* tmp
   float best = 1e30f;
   for (int cand = 0; cand < 16; ++cand) {
     const int C = cand == 0 ? 0 : 1 << ((cand - 1) / 3), th = cand == 0 ? kResidentThreads : 256 << ((cand - 1) % 3);
-    if (C > kResidentMaxCtas || (C > 0 && !resident_feasible(prec, lv.g, C))) continue;
+    if (C > kResidentMaxCtas || (C > 0 && !resident_feasible(pb->desc.disc, pb->desc.nu_a != 0.0 ? 1 : 0, prec, lv.g, C))) continue;
     HHG_TRY(set_resident(pb, lv, prec, C, th));
     HHG_CUDA(cudaMemsetAsync(x, 0, bytes, pb->stream));
     HHG_CUDA(cudaMemsetAsync(tmp, 0, bytes, pb->stream));

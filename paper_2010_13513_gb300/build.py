@@ -21,7 +21,9 @@ OUT = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libhhg.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 # (source, object, extra flags): fast.cu and stream.cu are compiled once per precision
-SOURCES = [("kernels.cu", "kernels", []), ("transfer.cu", "transfer", []), ("fast.cu", "fast64", ["-DHHG_FAST_ONLY=64"]),
+SOURCES = [("kernels.cu", "kernels", []), ("transfer.cu", "transfer", []),
+           ("uzrows.cu", "uzrows", []), ("rows.cu", "rows", []), ("march.cu", "march", []),
+           ("fast.cu", "fast64", ["-DHHG_FAST_ONLY=64"]),
            ("fast.cu", "fast32", ["-DHHG_FAST_ONLY=32"]),
            ("fast.cu", "fast64b", ["-DHHG_FAST_ONLY=64", "-DHHG_FAST_BATCHED"]),
            ("fast.cu", "fast32b", ["-DHHG_FAST_ONLY=32", "-DHHG_FAST_BATCHED"]), ("stream.cu", "stream64", ["-DHHG_STREAM_ONLY=64"]),
@@ -62,7 +64,7 @@ def _compile(unit, verbose):
 
 def _generate_structure():
     """Compiles and runs the stencil-structure generator (host C++), which
-    writes the compile-time row term counts used by fast.cu."""
+    writes the compile-time row term tables the kernels are unrolled from."""
     exe = os.path.join(OUT, "gen_structure")
     cxx = shutil.which("g++") or shutil.which("c++")
     cmd = [cxx, "-O1", "-std=c++17", "-I", os.path.join(ROOT, "include"), os.path.join(CSRC, "gen_structure.cpp"),

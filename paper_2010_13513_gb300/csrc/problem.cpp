@@ -19,8 +19,11 @@
 #include "internal.h"
 #include "kernels.h"
 #include "nn.h"
+#include "march.h"
+#include "rows.h"
 #include "small.h"
 #include "stream.h"
+#include "uzrows.h"
 
 using namespace hhg;
 
@@ -127,13 +130,12 @@ struct Level {
   std::vector<double> inv_diag;         // per group 1/diag(A)
   // parameter blocks of the specialised kernels (FastTab<T, N> images)
   std::vector<char> ftab64[OP_COUNT], ftab32[OP_COUNT];
-  bool has_fast[OP_COUNT] = {};
   // parameter block of the double-float refinement residual (dfres.cu);
   // empty if the operator is not covered
   std::vector<char> dftab;
-  // parameter blocks of the streaming kernels (FULL, B^T, (B, -C))
-  std::vector<char> stab64[OP_COUNT], stab32[OP_COUNT];
-  bool has_stream[OP_COUNT] = {};
+  // parameter blocks of the streaming kernels of the full operator
+  std::vector<char> stab64, stab32;
+  bool has_stream = false;
   // weight tables (ResTabs) of the shared-memory-resident smoother: offsets
   // in the table blob, device addresses
   size_t o_rtab64 = 0, o_rtab32 = 0;
@@ -347,7 +349,7 @@ extern "C" int hhg_problem_create(const hhg_mesh* mesh, const hhg_problem_desc* 
   Blob& B = pb->tables;
   const int varnu = desc->nu_a != 0.0 ? 1 : 0;
   for (Level& lv : pb->lv) {
-    std::vector<double> wc_bc;            // clipped C stencils of the (B, -C) row
+    std::vector<double> c_class;          // clipped C stencils of the pressure row per boundary class
     for (int o = 0; o < OP_COUNT; ++o) {
       OpHost h = serialise(lv.st.op[o], lv.g);
       const int N = fast_terms(desc->disc, varnu, o);
@@ -368,16 +370,15 @@ extern "C" int hhg_problem_create(const hhg_mesh* mesh, const hhg_problem_desc* 
           return true;
         };
         if (!image(0.0, lv.ftab64[o]) || !image(0.0f, lv.ftab32[o])) return fail(HHG_EINVAL, "level too large for 32-bit offsets");
-        lv.has_fast[o] = true;
         if (o == OP_FULL) df_table(desc->disc, varnu, lv.ftab64[o], lv.dftab);
       }
-      if (N >= 0 && (o == OP_FULL || o == OP_BT || o == OP_BC)) {
+      if (o == OP_FULL) {
         // streaming kernels: the weights, and the boundary C stencil of the
         // pressure row summed per boundary class (27 classes: each of i, j, k
         // on the low face, inside, or on the high face; a per-cube term
         // counts where its cube lies inside the box)
         std::vector<int> offs;
-        stream_c_offsets(desc->disc, varnu, o, offs);
+        stream_c_offsets(desc->disc, varnu, offs);
         const int ncb = int(offs.size()) / 3;
         std::vector<double> wc(size_t(27) * ncb, 0.0);
         for (const HRow& R : lv.st.op[o].rows)
@@ -395,9 +396,9 @@ extern "C" int hhg_problem_create(const hhg_mesh* mesh, const hhg_problem_desc* 
                 if (in) wc[size_t(cls) * ncb + slot] += t.w;
               }
             }
-        if (o == OP_BC) wc_bc = wc;
-        lv.has_stream[o] = stream_image<double>(desc->disc, varnu, o, h.w64, wc, lv.stab64[o]) &&
-                           stream_image<float>(desc->disc, varnu, o, h.w64, wc, lv.stab32[o]);
+        c_class = wc;
+        lv.has_stream = stream_image<double>(desc->disc, varnu, h.w64, wc, lv.stab64) &&
+                        (desc->disc == HHG_P2P1_TH || stream_image<float>(desc->disc, varnu, h.w64, wc, lv.stab32));
       }
       std::vector<float> w32(h.w64.begin(), h.w64.end()), bw32(h.bw64.begin(), h.bw64.end());
       OpOffsets& of = lv.opoff[o];
@@ -405,8 +406,8 @@ extern "C" int hhg_problem_create(const hhg_mesh* mesh, const hhg_problem_desc* 
       of.rows = B.put(h.rows); of.terms = B.put(h.terms); of.w64 = B.put(h.w64); of.w32 = B.put(w32);
       of.bterms = B.put(h.bterms); of.bw64 = B.put(h.bw64); of.bw32 = B.put(bw32);
     }
-    HHG_TRY(put_res_tabs<double>(B, lv, wc_bc, lv.o_rtab64));
-    HHG_TRY(put_res_tabs<float>(B, lv, wc_bc, lv.o_rtab32));
+    HHG_TRY(put_res_tabs<double>(B, lv, c_class, lv.o_rtab64));
+    HHG_TRY(put_res_tabs<float>(B, lv, c_class, lv.o_rtab32));
   }
   // ---- workspace layout
   size_t off = 0;
@@ -616,33 +617,49 @@ template <class T> const void* ftab(Level& lv, int op);
 template <> const void* ftab<double>(Level& lv, int op) { return lv.ftab64[op].data(); }
 template <> const void* ftab<float>(Level& lv, int op) { return lv.ftab32[op].data(); }
 
-template <class T> const void* stab(Level& lv, int op);
-template <> const void* stab<double>(Level& lv, int op) { return lv.stab64[op].data(); }
-template <> const void* stab<float>(Level& lv, int op) { return lv.stab32[op].data(); }
+template <class T> const void* stab(Level& lv);
+template <> const void* stab<double>(Level& lv) { return lv.stab64.data(); }
+template <> const void* stab<float>(Level& lv) { return lv.stab32.data(); }
 
-// the streaming kernels of op if the level's shape selects them (true if launched)
+template <class T> constexpr int prec_index() { return sizeof(T) == 8 ? HHG_FP64 : HHG_FP32; }
+template <class T> const ResTabs<T>* rtab(const Level& lv);
+template <> const ResTabs<double>* rtab<double>(const Level& lv) { return lv.rtab64; }
+template <> const ResTabs<float>* rtab<float>(const Level& lv) { return lv.rtab32; }
+
+// the streaming kernels of the full operator if the level's shape selects them (true if launched)
+// P2-P1 in FP32 has two ways, by size: above a million sites the marching
+// kernels (level 7 of one cube: 206 us against 290 us), below the unstaged
+// rows (level 6: 29 us against 41 us)
+bool marched(const hhg_problem* pb, const Level& lv) {
+  return pb->ov == 2 && int64_t(lv.g.nx + 1) * (lv.g.ny + 1) * (lv.g.nz + 1) > 1000000;
+}
 template <class T>
-bool stream_op(hhg_problem* pb, Level& lv, const Shape& sh, int op, int mode, const T* x, const T* b, T* y) {
-  const int si = op == OP_FULL ? 0 : op == OP_BT ? 1 : op == OP_BC ? 2 : -1;
-  if (si < 0 || mode == MODE_ADD || !lv.has_stream[op]) return false;
-  const int nt = sizeof(T) == 8 ? sh.st64_threads[si] : sh.st_threads[si];
-  const int ns = sizeof(T) == 8 ? 4 : sh.st_sites[si];
-  if (!nt) return false;
-  const int disc = pb->desc.disc, varnu = pb->desc.nu_a != 0.0 ? 1 : 0;
-  return stream_rows<T>(disc, varnu, op, mode, lv.g, stab<T>(lv, op), x, b, y, nt, ns, pb->stream);
+bool stream_op(hhg_problem* pb, Level& lv, const Shape& sh, int mode, const T* x, const T* b, T* y) {
+  const int nt = sizeof(T) == 8 ? sh.st64_threads : sh.st_threads;
+  if (mode == MODE_ADD || !lv.has_stream || !nt || (sizeof(T) == 4 && pb->ov == 2)) return false;
+  return stream_rows<T>(pb->desc.disc, pb->desc.nu_a != 0.0 ? 1 : 0, OP_FULL, mode, lv.g, stab<T>(lv), x, b, y, nt,
+                        sizeof(T) == 8 ? 4 : sh.st_sites, pb->stream);
 }
 
 template <class T>
 int apply_op(hhg_problem* pb, Level& lv, int op, int mode, const T* x, const T* b, T* y, double alpha = 1.0) {
-  if (stream_op<T>(pb, lv, lv.shape, op, mode, x, b, y)) {
-    HHG_CHECK_LAUNCH();
-    return HHG_OK;
-  }
-  if (lv.has_fast[op] && op != OP_A)
-    fast_rows<T>(pb->desc.disc, pb->desc.nu_a != 0.0 ? 1 : 0, op, lv.g, lv.op[op], ftab<T>(lv, op), mode, x, b, y,
-                 alpha, lv.shape, pb->stream);
-  else
+  const int disc = pb->desc.disc, varnu = pb->desc.nu_a != 0.0 ? 1 : 0;
+  if (op == OP_FULL && mode != MODE_ADD) {
+    if constexpr (sizeof(T) == 4) {
+      if (marched(pb, lv)) {
+        march_rows(disc, varnu, mode, lv.g, ftab<T>(lv, OP_FULL), rtab<T>(lv), x, b, y, pb->stream);
+        HHG_CHECK_LAUNCH();
+        return HHG_OK;
+      }
+    }
+    if (!stream_op<T>(pb, lv, lv.shape, mode, x, b, y))
+      full_rows<T>(disc, varnu, mode, lv.g, ftab<T>(lv, OP_FULL), rtab<T>(lv), x, b, y, pb->stream);
+  } else if (op == OP_BT && mode == MODE_SET) {
+    // (the FastTab images start with the weights; Dirichlet rows stay as they are)
+    bt_rows<T>(disc, varnu, mode, lv.g, static_cast<const T*>(ftab<T>(lv, OP_BT)), x, b, y, pb->stream);
+  } else {
     launch_apply<T>(lv.g, lv.op[op], mode, x, b, y, alpha, pb->stream);
+  }
   HHG_CHECK_LAUNCH();
   return HHG_OK;
 }
@@ -650,11 +667,6 @@ int apply_op(hhg_problem* pb, Level& lv, int op, int mode, const T* x, const T* 
 double level_weight(hhg_problem* pb, const Level& lv) {
   return double(lv.n_dofs()) / double(pb->L(pb->desc.L).n_dofs());
 }
-
-template <class T> constexpr int prec_index() { return sizeof(T) == 8 ? HHG_FP64 : HHG_FP32; }
-template <class T> const ResTabs<T>* rtab(const Level& lv);
-template <> const ResTabs<double>* rtab<double>(const Level& lv) { return lv.rtab64; }
-template <> const ResTabs<float>* rtab<float>(const Level& lv) { return lv.rtab32; }
 
 // selects `ctas` CTAs (0: per-phase kernels) for the resident smoother of a
 // level in precision `prec`; HHG_EINVAL if the level does not fit
@@ -707,8 +719,8 @@ int uzawa(hhg_problem* pb, Level& lv, const hhg_params& prm, int sweeps, T* x, c
   const Costs cs = block_costs(pb->ov);
   for (int it = 0; it < sweeps; ++it) {
     // velocity step (Eq. uzawa-velocity): f' = f - B^T p_k, xi GS sweeps on A u = f'
-    HHG_TRY(apply_op<T>(pb, lv, OP_BT, MODE_RES, x, b, tmp));
     const int disc = pb->desc.disc, varnu = pb->desc.nu_a != 0.0 ? 1 : 0;
+    bt_rows<T>(disc, varnu, MODE_RES, lv.g, static_cast<const T*>(ftab<T>(lv, OP_BT)), x, b, tmp, pb->stream);
     const void* tabA = ftab<T>(lv, OP_A);
     // A is block diagonal over the velocity components: either every phase
     // on all three components, or all sweeps of one component after another
@@ -726,9 +738,8 @@ int uzawa(hhg_problem* pb, Level& lv, const hhg_params& prm, int sweeps, T* x, c
       }
     HHG_CHECK_LAUNCH();
     // pressure step (Eq. uzawa-pressure): p -= S_hat^{-1} (g - B u_{k+1} + C p_k)
-    HHG_TRY(apply_op<T>(pb, lv, OP_BC, MODE_RES, x, b, tmp));
-    const int64_t po = p_offset(lv);
-    launch_pupdate<T>(lv.g, x + po, tmp + po, lv.inv_mlhat, 1.0 / prm.omega_inv, pb->stream);
+    uzawa_pressure<T>(disc, varnu, lv.g, static_cast<const T*>(ftab<T>(lv, OP_BC)), rtab<T>(lv), x, b, tmp,
+                      lv.inv_mlhat, 1.0 / prm.omega_inv, pb->stream);
     HHG_CHECK_LAUNCH();
     pb->wu_counted += level_weight(pb, lv) * (prm.xi * (prm.ahat == HHG_AHAT_S ? 2 : 1) * cs.A + 2 * cs.B + cs.C);
   }
@@ -1475,17 +1486,12 @@ extern "C" int hhg_set_launch_shape(hhg_problem* pb, int level, int row_threads,
   sh.row_kplanes = row_kplanes;
   sh.gs_threads = gs_threads;
   const int st = row_tile == 1 ? 128 : row_tile;
-  for (int o = 0; o < 3; ++o) {
-    sh.st_threads[o] = sh.st64_threads[o] = st;
-    sh.st_sites[o] = row_sites == 2 ? 2 : 4;
-  }
+  sh.st_threads = sh.st64_threads = st;
+  sh.st_sites = row_sites == 2 ? 2 : 4;
   sh.row_sites = row_sites == 2 ? 4 : row_sites;
-  sh.row_sites64 = row_sites;
   sh.gs_lanes = gs_lanes;
   sh.gs_lanes0 = gs_lanes;
   sh.gs_threads0 = 0;
-  sh.bt_threads = sh.bt_kplanes = sh.bt_sites = 0;
-  sh.bc_threads = sh.bc_kplanes = sh.bc_sites = 0;
   for (auto& kv : pb->graphs) cudaGraphExecDestroy(kv.second.exec);
   pb->graphs.clear();
   return HHG_OK;
@@ -1511,8 +1517,8 @@ extern "C" int hhg_get_launch_shape(hhg_problem* pb, int level, int* shape6) {
   HHG_TRY(check_level(pb, level));
   if (!shape6) return fail(HHG_EINVAL, "null argument");
   const Shape& sh = pb->L(level).shape;
-  shape6[0] = sh.row_threads; shape6[1] = sh.row_kplanes; shape6[2] = sh.gs_threads; shape6[3] = sh.st_threads[0];
-  shape6[4] = sh.st_threads[0] && sh.st_sites[0] == 2 ? 2 : sh.row_sites; shape6[5] = sh.gs_lanes;
+  shape6[0] = sh.row_threads; shape6[1] = sh.row_kplanes; shape6[2] = sh.gs_threads; shape6[3] = sh.st_threads;
+  shape6[4] = sh.st_threads && sh.st_sites == 2 ? 2 : sh.row_sites; shape6[5] = sh.gs_lanes;
   return HHG_OK;
 }
 
@@ -1865,104 +1871,43 @@ int tune_level(hhg_problem* pb, Level& lv, int reps, T* xa, T* xb) {
     return ms;
   };
   const int disc = pb->desc.disc, varnu = pb->desc.nu_a != 0.0 ? 1 : 0;
-  // row kernels: FULL residual, one site per thread or four runs of 32
-  // sites per warp
-  const int threads[3] = {64, 128, 256}, planes[5] = {1, 2, 4, 8, 16};
-  float best = 1e30f;
-  // the plain kernels are timed first; the streaming kernels compete after
-  for (int o = 0; o < 3; ++o) lv.shape.st_threads[o] = lv.shape.st64_threads[o] = 0;
+  // the full operator's residual: the unstaged rows (rows.cu) against the
+  // streaming kernels (threads per block, sites per thread), in the V-cycle
+  // precision and, for the mixed solve, in FP64
+  const int threads[3] = {64, 128, 256};
   Shape bestS = lv.shape;
-  for (int v : {1, 4})
-    for (int t : threads)
-      for (int kp : planes) {
-        if (v > 1 && (t == 64 || kp > 4)) continue;
-        Shape sh = lv.shape;
-        sh.row_threads = t;
-        sh.row_kplanes = kp;
-        sh.row_sites = v;
-        const float ms = time_it([&] {
-          fast_rows<T>(disc, varnu, OP_FULL, lv.g, lv.op[OP_FULL], ftab<T>(lv, OP_FULL), MODE_RES, xa, xa, xb, 1.0,
-                       sh, pb->stream);
-        });
-        if (ms < best) { best = ms; bestS.row_threads = t; bestS.row_kplanes = kp; bestS.row_sites = v; }
-      }
-  if (std::is_same<T, double>::value) {
-    bestS.row_sites64 = bestS.row_sites;
-  } else {
-    // the FP64 residual of the mixed solve's refinement: its own choice of
-    // sites per thread (FP64 arithmetic, not the loads, bounds it)
-    float best64 = 1e30f;
-    for (int v : {1, 4}) {
-      Shape sh = bestS;
-      sh.row_sites64 = v;
-      const float ms = time_it([&] {
-        fast_rows<double>(disc, varnu, OP_FULL, lv.g, lv.op[OP_FULL], ftab<double>(lv, OP_FULL), MODE_RES, lv.tmp64,
-                          lv.tmp64, lv.bw64, 1.0, sh, pb->stream);
-      });
-      if (ms < best64) { best64 = ms; bestS.row_sites64 = v; }
-    }
-  }
-  // the smoother's B^T and (B, -C) residual rows: their own shapes (24 short
-  // rows on one input array; one long row on all of them)
-  for (int op : {OP_BT, OP_BC}) {
-    float bo = 1e30f;
-    int bt = 0, bk = 0, bs = 0;
-    for (int v : {1, 4})
-      for (int t : threads)
-        for (int kp : {1, 2, 4}) {
-          if (v > 1 && t == 64) continue;
-          Shape sh = bestS;
-          if (op == OP_BT) { sh.bt_threads = t; sh.bt_kplanes = kp; sh.bt_sites = v; }
-          else { sh.bc_threads = t; sh.bc_kplanes = kp; sh.bc_sites = v; }
-          const float ms = time_it([&] {
-            fast_rows<T>(disc, varnu, op, lv.g, lv.op[op], ftab<T>(lv, op), MODE_RES, xa, xa, xb, 1.0, sh, pb->stream);
-          });
-          if (ms < bo) { bo = ms; bt = t; bk = kp; bs = v; }
-        }
-    if (op == OP_BT) { bestS.bt_threads = bt; bestS.bt_kplanes = bk; bestS.bt_sites = bs; }
-    else { bestS.bc_threads = bt; bestS.bc_kplanes = bk; bestS.bc_sites = bs; }
-  }
-  // the streaming kernels (stream.cu) against the best plain shape, for the
-  // FULL residual and the smoother's B^T and (B, -C) rows (threads per block),
-  // in the V-cycle precision and, for the mixed solve, the FP64 residual
-  {
-    const int sops[3] = {OP_FULL, OP_BT, OP_BC};
-    for (int o = 0; o < 3; ++o) {
-      Shape sh = bestS;
-      sh.st_threads[o] = 0;
-      float bo = time_it([&] {
-        fast_rows<T>(disc, varnu, sops[o], lv.g, lv.op[sops[o]], ftab<T>(lv, sops[o]), MODE_RES, xa, xa, xb, 1.0, sh,
-                     pb->stream);
-      });
-      for (int v : {4, 2})
-        for (int t : threads) {
-          if (v == 2 && sizeof(T) == 8) continue;
-          sh.st_threads[o] = t;
-          sh.st_sites[o] = v;
-          if (!stream_op<T>(pb, lv, sh, sops[o], MODE_RES, xa, xa, xb)) continue;
-          const float ms = time_it([&] { stream_op<T>(pb, lv, sh, sops[o], MODE_RES, xa, xa, xb); });
-          if (ms < bo) { bo = ms; bestS.st_threads[o] = t; bestS.st_sites[o] = v; }
-        }
-      if (std::is_same<T, double>::value) bestS.st64_threads[o] = bestS.st_threads[o];
-    }
-    if (!std::is_same<T, double>::value) {
-      Shape sh = bestS;
-      sh.st64_threads[0] = 0;
-      float bo = time_it([&] {
-        fast_rows<double>(disc, varnu, OP_FULL, lv.g, lv.op[OP_FULL], ftab<double>(lv, OP_FULL), MODE_RES, lv.tmp64,
-                          lv.tmp64, lv.bw64, 1.0, sh, pb->stream);
-      });
+  bestS.st_threads = bestS.st64_threads = 0;
+  auto tune_rows = [&](auto* in, auto* out, int& best_threads, int* best_sites) {
+    using U = std::remove_reference_t<decltype(*in)>;
+    best_threads = 0;
+    float best_ms = time_it([&] {
+      full_rows<U>(disc, varnu, MODE_RES, lv.g, ftab<U>(lv, OP_FULL), rtab<U>(lv), in, in, out, pb->stream);
+    });
+    for (int v : {4, 2})
       for (int t : threads) {
-        sh.st64_threads[0] = t;
-        if (!stream_op<double>(pb, lv, sh, OP_FULL, MODE_RES, lv.tmp64, lv.tmp64, lv.bw64)) continue;
-        const float ms = time_it([&] { stream_op<double>(pb, lv, sh, OP_FULL, MODE_RES, lv.tmp64, lv.tmp64, lv.bw64); });
-        if (ms < bo) { bo = ms; bestS.st64_threads[0] = t; }
+        if (v == 2 && !best_sites) continue;
+        Shape sh = bestS;
+        sh.st_threads = sh.st64_threads = t;
+        sh.st_sites = v;
+        if (!stream_op<U>(pb, lv, sh, MODE_RES, in, in, out)) continue;
+        const float ms = time_it([&] { stream_op<U>(pb, lv, sh, MODE_RES, in, in, out); });
+        if (ms < best_ms) {
+          best_ms = ms;
+          best_threads = t;
+          if (best_sites) *best_sites = v;
+        }
       }
-    }
+  };
+  if (std::is_same<T, double>::value) {
+    tune_rows(xa, xb, bestS.st64_threads, nullptr);
+    bestS.st_threads = bestS.st64_threads;
+  } else {
+    tune_rows(xa, xb, bestS.st_threads, &bestS.st_sites);
+    tune_rows(lv.tmp64, lv.bw64, bestS.st64_threads, nullptr);
   }
   // Gauss-Seidel kernels: one forward sweep, 1, 2 or 4 lanes per site; the
   // lanes of the vertex colours and of the edge groups are then chosen apart
-  best = 1e30f;
+  float best = 1e30f;
   auto sweep = [&](const Shape& sh, bool vertex, bool edges) {
     if (vertex)
       for (int c = 0; c < 4; ++c) fast_gs<T>(disc, varnu, lv.g, ftab<T>(lv, OP_A), 0, c, 1.0, xb, xa, sh, pb->stream);
@@ -2079,12 +2024,13 @@ extern "C" int hhg_autotune(hhg_problem* pb, int reps, int* shapes_out) {
       o[0] = lv.shape.row_threads; o[1] = lv.shape.row_kplanes; o[2] = lv.shape.gs_threads;
       o[3] = lv.rctas[mixed ? HHG_FP32 : HHG_FP64];
       o[4] = lv.rthreads[mixed ? HHG_FP32 : HHG_FP64];
-      o[5] = lv.shape.st_threads[0];
+      o[5] = lv.shape.st_threads;
       o[6] = lv.shape.row_sites;
       o[7] = lv.shape.gs_lanes;
       o[8] = lv.shape.gs_lanes0;
-      o[9] = lv.shape.bt_threads; o[10] = lv.shape.bt_kplanes; o[11] = lv.shape.bt_sites;
-      o[12] = lv.shape.bc_threads; o[13] = lv.shape.bc_kplanes; o[14] = lv.shape.bc_sites;
+      // (the smoother's B^T and (B, -C) rows have one launch shape, uzrows.cu)
+      o[9] = 128; o[10] = 1; o[11] = 1;
+      o[12] = 256; o[13] = 1; o[14] = 1;
       o[15] = lv.shape.gs_threads0 ? lv.shape.gs_threads0 : lv.shape.gs_threads;
     }
   }

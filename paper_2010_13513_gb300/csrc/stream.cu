@@ -1,6 +1,5 @@
 // Streaming stencil rows: y = calA x and r = b - calA x over all rows of the
-// operator (Eq. stokes-discrete), and the B^T and (B, -C) rows of the inexact
-// Uzawa smoother (Sec. 3.2), on levels large enough to fill the GPU.
+// operator (Eq. stokes-discrete), on levels large enough to fill the GPU.
 //
 // Data reuse.  In the Kuhn-lattice layout an input value x(a, site) is read
 // by the rows of every DoF group at about 27 neighbouring sites, so a kernel
@@ -23,9 +22,9 @@
 // The plan (which arrays a pass stages, which rows it evaluates, the terms of
 // each line with their row, segment and weight index) is emitted at build
 // time by gen_structure.cpp from the stencil builder: every term is a
-// compile-time register operation with a constant-bank weight.  Operators
-// that read more than nine arrays (P2-P1: the full operator and B u - C p)
-// take one launch per velocity component; the pressure row's first pass
+// compile-time register operation with a constant-bank weight.  P2-P1, whose
+// operator reads more than nine arrays, takes one launch per velocity
+// component; the pressure row's first pass
 // writes it and the later passes add their terms to it.
 //
 // Work split: the grid is one wave of blocks (the blocks that fit on the GPU
@@ -664,9 +663,12 @@ void offsets_of(std::vector<int>& o) {
 
 }  // namespace
 
-#define HHG_STREAM_CASES(X) \
-  X(1, 0, OP_FULL) X(1, 0, OP_BT) X(1, 0, OP_BC) X(1, 1, OP_FULL) X(1, 1, OP_BT) X(1, 1, OP_BC) \
-  X(2, 0, OP_FULL) X(2, 0, OP_BT) X(2, 0, OP_BC) X(2, 1, OP_FULL) X(2, 1, OP_BT) X(2, 1, OP_BC)
+// FP32 P2-P1 has the marching rows (march.cu)
+#if defined(HHG_STREAM_ONLY) && HHG_STREAM_ONLY == 32
+#define HHG_STREAM_CASES(X) X(1, 0, OP_FULL) X(1, 1, OP_FULL)
+#else
+#define HHG_STREAM_CASES(X) X(1, 0, OP_FULL) X(1, 1, OP_FULL) X(2, 0, OP_FULL) X(2, 1, OP_FULL)
+#endif
 
 #if defined(HHG_STREAM_BATCHED)
 // the recorder of this translation unit's kernels (precision HHG_STREAM_ONLY,
@@ -725,24 +727,24 @@ template void stream_init_v<double, kV>();
 
 #if !defined(HHG_STREAM_V) || HHG_STREAM_V != 2
 template <class T>
-bool stream_image(int disc, int varnu, int op, const std::vector<double>& w, const std::vector<double>& wc,
+bool stream_image(int disc, int varnu, const std::vector<double>& w, const std::vector<double>& wc,
                   std::vector<char>& out) {
 #define HHG_M(D, V, O) \
-  if (disc == D && varnu == V && op == O) { make_image<D, V, O, T>(w, wc, out); return true; }
+  if (disc == D && varnu == V) { make_image<D, V, O, T>(w, wc, out); return true; }
   HHG_STREAM_CASES(HHG_M)
 #undef HHG_M
   return false;
 }
 #if defined(HHG_STREAM_ONLY) && HHG_STREAM_ONLY == 32
-template bool stream_image<float>(int, int, int, const std::vector<double>&, const std::vector<double>&,
+template bool stream_image<float>(int, int, const std::vector<double>&, const std::vector<double>&,
                                   std::vector<char>&);
 #else
-template bool stream_image<double>(int, int, int, const std::vector<double>&, const std::vector<double>&,
+template bool stream_image<double>(int, int, const std::vector<double>&, const std::vector<double>&,
                                    std::vector<char>&);
 
-bool stream_c_offsets(int disc, int varnu, int op, std::vector<int>& offsets) {
+bool stream_c_offsets(int disc, int varnu, std::vector<int>& offsets) {
 #define HHG_O(D, V, O) \
-  if (disc == D && varnu == V && op == O) { offsets_of<D, V, O>(offsets); return true; }
+  if (disc == D && varnu == V) { offsets_of<D, V, O>(offsets); return true; }
   HHG_STREAM_CASES(HHG_O)
 #undef HHG_O
   return false;

@@ -18,7 +18,7 @@ constexpr size_t kStreamMaxSmem = 232448;
 template <class T>
 void stream_init();
 
-// rows of op (OP_FULL, OP_BT or OP_BC) in MODE_SET / MODE_RES by the
+// rows of op (OP_FULL) in MODE_SET / MODE_RES by the
 // streaming kernels (one launch per pass): blocks of `threads` (64 / 128 /
 // 256) threads of `sites` (FP32: 2 or 4; FP64: 4) consecutive sites each,
 // owning sites x threads positions of the (i, j) plane and a run of k
@@ -48,11 +48,11 @@ bool stream_rows_record_v(int disc, int varnu, int op, int mode, const Geo& g, c
 // ci + 3 cj + 9 ck, c = 0 low face, 1 inside, 2 high face; offsets in the
 // order of stream_c_offsets); false if op has no streaming kernel
 template <class T>
-bool stream_image(int disc, int varnu, int op, const std::vector<double>& w, const std::vector<double>& wc,
+bool stream_image(int disc, int varnu, const std::vector<double>& w, const std::vector<double>& wc,
                   std::vector<char>& out);
 
 // the lattice offsets (di, dj, dk triples) of the boundary C stencil of op's
 // pressure row (empty if it has no C terms)
-bool stream_c_offsets(int disc, int varnu, int op, std::vector<int>& offsets);
+bool stream_c_offsets(int disc, int varnu, std::vector<int>& offsets);
 
 }  // namespace hhg

@@ -1,0 +1,288 @@
+// The B^T rows and the pressure step of an inexact Uzawa iteration (Sec. 3.2,
+// Eqs. uzawa-velocity / uzawa-pressure) on levels whose smoother runs as
+// separate launches.
+//
+//  * k_bt: a thread owns a lattice cell and a component and evaluates all of
+//    the component's rows there: the rows of the eight P2 groups read the same
+//    15 pressure values, so these are loaded once, and the rest of the traffic
+//    is the right-hand side in and tmp out, once each;
+//  * k_pressure: the row of (B, -C) and the pressure update in one launch: a
+//    thread owns a pressure site.  For P2-P1 the row reads no pressure and the
+//    update is in place; the P1-P1 row does, so that the new pressures go to
+//    the scratch vector and are copied back.
+// All rows are unrolled from the generated structure; with a constant
+// viscosity the weights are immediates (those of h = 1).  Boundary pressure
+// rows keep the merged B terms (exact for inputs with zero Dirichlet
+// velocities) and take the C stencil of their boundary class.
+//
+// Bound: HBM on the largest levels; below, the L1/L2 loads of the pressure
+// row (156 for P2-P1), which is why a block of consecutive rows marches over
+// a few planes: the lines of neighbouring rows and planes meet in L1.
+// Measured, both rows and the update of one iteration against the three
+// launches before: P2-P1 FP32 level 5 / 6 / 7: 24 / 49 / 236 us before, 12 / 31
+// / 190 us now; P1-P1 with variable viscosity, 48 tetrahedra, level 6: 81 us
+// before, 73 us (device times).
+#include <cuda_runtime.h>
+
+#include <algorithm>
+#include <type_traits>
+#include <utility>
+
+#include "at.h"
+#include "batch.h"
+#include "kernels.h"
+#include "structure.inc"
+#include "uzrows.h"
+
+namespace hhg {
+namespace {
+
+template <class S, int E, class T, int NW>
+__device__ __forceinline__ T rweight(const T (&w)[NW]) {
+  if constexpr (NW > 1) {
+    return w[E];
+  } else {
+    constexpr double r = S::wref[E];
+    return T(r);
+  }
+}
+
+// ------------------------------------------------------------------- B^T
+template <class T, int NW>
+struct BtA { Geo g; const T* x; const T* b; T* y; T w[NW]; };   // b = null: y = B^T p
+template <int DISC, int VARNU>
+constexpr int bt_nw() { return VARNU ? gen::S<DISC, VARNU, OP_BT>::N : 1; }
+
+template <class S, int R, int NW, class T, int... I>
+__device__ __forceinline__ T bt_row(const T (&p)[27], const T (&w)[NW], std::integer_sequence<int, I...>) {
+  T a = T(0);
+  ([&] {
+    constexpr int e = S::rows[R].t0 + I;
+    constexpr gen::OffT o = S::off[e];
+    a = fma(rweight<S, e>(w), p[(o.di + 1) + 3 * (o.dj + 1) + 9 * (o.dk + 1)], a);
+  }(), ...);
+  return a;
+}
+// whether some row of B^T reads the pressure at offset q - 13 of the 27 neighbours
+template <class S>
+constexpr bool bt_reads(int q) {
+  for (int e = 0; e < S::N; ++e)
+    if ((S::off[e].di + 1) + 3 * (S::off[e].dj + 1) + 9 * (S::off[e].dk + 1) == q) return true;
+  return false;
+}
+template <class S, class T, int... Q>
+__device__ __forceinline__ void bt_load(const T* __restrict__ x, const Lines<T>& at, T (&p)[27],
+                                        std::integer_sequence<int, Q...>) {
+  ([&] {
+    if constexpr (bt_reads<S>(Q)) p[Q] = at.template ld<Q % 3 - 1, Q / 3 % 3 - 1, Q / 9 - 1>(x);
+  }(), ...);
+}
+template <int DISC, int VARNU, int R0, int NW, class T, int... GG>
+__device__ __forceinline__ void bt_groups(const BtA<T, NW>& a, const T (&p)[27], unsigned at, int in,
+                                        std::integer_sequence<int, GG...>) {
+  using S = gen::S<DISC, VARNU, OP_BT>;
+  const Geo& g = a.g;
+  const T hs = VARNU ? T(1) : T(g.h) * T(g.h);
+  T bv[sizeof...(GG)];
+  ((bv[GG] = a.b && (in >> GG & 1) ? ld_at(a.b + (R0 + GG) * g.arr, at) : T(0)), ...);
+  ([&] {
+    constexpr gen::RowS rw = S::rows[R0 + GG];
+    static_assert(rw.n1 == 0 && rw.n2 == 0, "B^T is unscaled");
+    const T v = bt_row<S, R0 + GG>(p, a.w, std::make_integer_sequence<int, rw.n0>{});
+    if (in >> GG & 1) ref_at(a.y + (R0 + GG) * g.arr, at) = a.b ? bv[GG] - hs * v : hs * v;
+  }(), ...);
+}
+
+// grid x over the positions of the padded (i, j) plane, y = plane, z = component
+template <int DISC, int VARNU, class T, int NW>
+__device__ __forceinline__ void bt_body(const uint3 bid, const BtA<T, NW>& a) {
+  constexpr int G = DISC == 2 ? 8 : 1;
+  const Geo& g = a.g;
+  const int q = bid.x * blockDim.x + threadIdx.x, j = q / g.sx, i = q - j * g.sx, k = bid.y;
+  if (i >= g.nx || j >= g.ny) return;
+  // groups with an interior DoF in the cell (order of kGroupOff)
+  int in = 0;
+#pragma unroll
+  for (int gg = 0; gg < G; ++gg)
+    if ((i > 0 || (0xB2 >> gg & 1)) && (j > 0 || (0xD4 >> gg & 1)) && (k > 0 || (0xE8 >> gg & 1))) in |= 1 << gg;
+  const Lines<T> at(g, unsigned(i + 1) + unsigned(j + 1) * unsigned(g.sx) + unsigned(k + 1) * unsigned(g.sy));
+  T p[27];
+  bt_load<gen::S<DISC, VARNU, OP_BT>>(a.x + 3 * G * g.arr, at, p, std::make_integer_sequence<int, 27>{});
+  const auto groups = std::make_integer_sequence<int, G>{};
+  if (DISC == 1) {                                 // the components share the pressures
+    bt_groups<DISC, VARNU, 0>(a, p, at.site(), in, groups);
+    bt_groups<DISC, VARNU, G>(a, p, at.site(), in, groups);
+    bt_groups<DISC, VARNU, 2 * G>(a, p, at.site(), in, groups);
+  } else if (bid.z == 0) {
+    bt_groups<DISC, VARNU, 0>(a, p, at.site(), in, groups);
+  } else if (bid.z == 1) {
+    bt_groups<DISC, VARNU, G>(a, p, at.site(), in, groups);
+  } else {
+    bt_groups<DISC, VARNU, 2 * G>(a, p, at.site(), in, groups);
+  }
+}
+template <int DISC, int VARNU, class T>
+__global__ void __launch_bounds__(128) k_bt(const __grid_constant__ BtA<T, bt_nw<DISC, VARNU>()> a) {
+  bt_body<DISC, VARNU>(blockIdx, a);
+}
+template <int DISC, int VARNU, class T>
+__global__ void __launch_bounds__(128) kb_bt(const void* items, int n) {
+  uint3 bid, gd;
+  const auto& it = batch_item<BtA<T, bt_nw<DISC, VARNU>()>>(items, n, bid, gd);
+  bt_body<DISC, VARNU>(bid, it.a);
+}
+
+// ---------------------------------------------------------- pressure step
+template <class T, int NW>
+struct PressA { Geo g; const T* x; const T* b; T* p; const double* inv_ml; double s; const ResTabs<T>* tabs; int kp; T w[NW]; };
+template <int DISC, int VARNU>
+constexpr int bc_nw() { return VARNU ? gen::S<DISC, VARNU, OP_BC>::N : 1; }
+
+// terms [T0, T0 + n) of the pressure row: four chains of sums
+template <class S, int T0, int NW, class T, int... I>
+__device__ __forceinline__ T press_sum(const Geo& g, const T* __restrict__ x, const Lines<T>& at, const T (&w)[NW],
+                                       std::integer_sequence<int, I...>) {
+  T a[4] = {};
+  ([&] {
+    constexpr gen::OffT o = S::off[T0 + I];
+    a[I & 3] = fma(rweight<S, T0 + I>(w), at.template ld<o.di, o.dj, o.dk>(x + o.arr * g.arr), a[I & 3]);
+  }(), ...);
+  return (a[0] + a[1]) + (a[2] + a[3]);
+}
+// the C terms of a boundary row: the stencil of its class
+template <class SPT, class T, int... O>
+__device__ __forceinline__ T press_c(const Geo& g, const T* __restrict__ p, const T* __restrict__ wc,
+                                     std::integer_sequence<int, O...>) {
+  T a = T(0);
+  ((a = fma(__ldg(wc + O), __ldg(p + SPT::cbo[O].di + SPT::cbo[O].dj * g.sx + SPT::cbo[O].dk * g.sy), a)), ...);
+  return a;
+}
+
+// grid x over the positions of the padded (i, j) plane, y = groups of kp planes
+template <int DISC, int VARNU, class T, int NW>
+__device__ __forceinline__ void press_body(const uint3 bid, const PressA<T, NW>& a) {
+  using S = gen::S<DISC, VARNU, OP_BC>;
+  constexpr gen::RowS rw = S::rows[0];
+  static_assert(rw.n1 == 0, "B is unscaled");
+  constexpr int G = DISC == 2 ? 8 : 1;
+  const Geo& g = a.g;
+  const int q = bid.x * blockDim.x + threadIdx.x, j = q / g.sx, i = q - j * g.sx;
+  if (i > g.nx || j > g.ny) return;
+  const int k1 = min(int(bid.y + 1) * a.kp, g.nz + 1);
+#pragma unroll 1
+  for (int k = bid.y * a.kp; k < k1; ++k) {
+    const int64_t idx = int64_t(i + 1) + int64_t(j + 1) * g.sx + int64_t(k + 1) * g.sy;
+    const Lines<T> at(g, unsigned(idx));
+    const T bv = __ldg(a.b + 3 * G * g.arr + idx);
+    const T ml = T(a.s * __ldg(a.inv_ml + idx));
+    const T* x = a.x + idx;
+    T v = press_sum<S, rw.t0>(g, a.x, at, a.w, std::make_integer_sequence<int, rw.n0>{});
+    if (!VARNU) v *= T(g.h) * T(g.h);
+    if constexpr (rw.n2 > 0) {
+      using SPT = gen::SP<DISC, VARNU, OP_BC>;
+      T c;
+      if (i == 0 || j == 0 || k == 0 || i == g.nx || j == g.ny || k == g.nz) {
+        const int cls = (i == 0 ? 0 : i == g.nx ? 2 : 1) + 3 * (j == 0 ? 0 : j == g.ny ? 2 : 1) +
+                        9 * (k == 0 ? 0 : k == g.nz ? 2 : 1);
+        c = press_c<SPT>(g, x + 3 * G * g.arr, a.tabs->wc + cls * SPT::NCB, std::make_integer_sequence<int, SPT::NCB>{});
+      } else {
+        c = press_sum<S, rw.t0 + rw.n0>(g, a.x, at, a.w, std::make_integer_sequence<int, rw.n2>{});
+        if (!VARNU) c *= T(g.h) * T(g.h) * T(g.h);
+      }
+      v += VARNU ? T(g.eisc[k]) * c : c;
+      a.p[idx] = __ldg(x + 3 * G * g.arr) - ml * (bv - v);
+    } else {
+      a.p[idx] -= ml * (bv - v);
+    }
+  }
+}
+template <int DISC, int VARNU, class T>
+__global__ void __launch_bounds__(256, DISC == 2 ? 2 : 3) k_pressure(const __grid_constant__ PressA<T, bc_nw<DISC, VARNU>()> a) {
+  press_body<DISC, VARNU>(blockIdx, a);
+}
+template <int DISC, int VARNU, class T>
+__global__ void __launch_bounds__(256, DISC == 2 ? 2 : 3) kb_pressure(const void* items, int n) {
+  uint3 bid, gd;
+  const auto& it = batch_item<PressA<T, bc_nw<DISC, VARNU>()>>(items, n, bid, gd);
+  press_body<DISC, VARNU>(bid, it.a);
+}
+
+// P1-P1: the new pressures back into the iterate
+template <class T>
+struct CopyA { const T* a; T* b; int64_t n; };
+template <class T>
+__device__ __forceinline__ void copy_body(const uint3 bid, const uint3 gd, const CopyA<T>& c) {
+  for (int64_t q = bid.x * int64_t(blockDim.x) + threadIdx.x; q < c.n; q += int64_t(gd.x) * blockDim.x) c.b[q] = c.a[q];
+}
+template <class T>
+__global__ void __launch_bounds__(256) k_copy(const __grid_constant__ CopyA<T> c) {
+  copy_body<T>(blockIdx, gridDim, c);
+}
+template <class T>
+__global__ void __launch_bounds__(256) kb_copy(const void* items, int n) {
+  uint3 bid, gd;
+  const auto& it = batch_item<CopyA<T>>(items, n, bid, gd);
+  copy_body<T>(bid, gd, it.a);
+}
+
+template <class A>
+void launch(const void* kernel, const void* batched, dim3 grd, int threads, const A& a, cudaStream_t s) {
+  if (g_rec) return g_rec->add(batched, grd, dim3(threads), 0, 1, a);
+  ++g_launches;
+  void* args[] = {const_cast<A*>(&a)};
+  cudaLaunchKernel(kernel, grd, dim3(threads), args, 0, s);
+}
+
+template <int DISC, int VARNU, class T>
+void launch_bt(const Geo& g, int mode, const T* w, const T* x, const T* b, T* y, cudaStream_t s) {
+  constexpr int NW = bt_nw<DISC, VARNU>();
+  BtA<T, NW> a{g, x, mode == MODE_RES ? b : nullptr, y, {}};
+  if (NW > 1) std::copy(w, w + NW, a.w);
+  const dim3 grd((g.ny * g.sx + 127) / 128, g.nz, DISC == 2 ? 3 : 1);
+  launch(reinterpret_cast<const void*>(k_bt<DISC, VARNU, T>), reinterpret_cast<const void*>(kb_bt<DISC, VARNU, T>), grd,
+         128, a, s);
+}
+template <int DISC, int VARNU, class T>
+void launch_pressure(const Geo& g, const T* w, const ResTabs<T>* tabs, T* x, const T* b, T* tmp,
+                     const double* inv_mlhat, double sc, cudaStream_t s) {
+  constexpr int NW = bc_nw<DISC, VARNU>(), G = DISC == 2 ? 8 : 1;
+  T* p = x + 3 * G * g.arr;
+  // planes of a block: several where the level fills the GPU anyway
+  const int kp = int64_t(g.nx + 1) * (g.ny + 1) * (g.nz + 1) > 1000000 ? 4 : 1;
+  PressA<T, NW> a{g, x, b, DISC == 2 ? p : tmp + 3 * G * g.arr, inv_mlhat, sc, tabs, kp, {}};
+  if (NW > 1) std::copy(w, w + NW, a.w);
+  const dim3 grd((g.ny * g.sx + g.nx + 256) / 256, (g.nz + kp) / kp);
+  launch(reinterpret_cast<const void*>(k_pressure<DISC, VARNU, T>),
+         reinterpret_cast<const void*>(kb_pressure<DISC, VARNU, T>), grd, 256, a, s);
+  if (DISC == 1)
+    launch(reinterpret_cast<const void*>(k_copy<T>), reinterpret_cast<const void*>(kb_copy<T>),
+           dim3(unsigned(std::min<int64_t>((g.arr + 255) / 256, 152 * 8))), 256, CopyA<T>{a.p, p, g.arr}, s);
+}
+
+}  // namespace
+
+template <class T>
+void bt_rows(int disc, int varnu, int mode, const Geo& g, const T* w, const T* x, const T* b, T* y, cudaStream_t s) {
+  if (disc == 1 && !varnu) launch_bt<1, 0, T>(g, mode, w, x, b, y, s);
+  else if (disc == 1) launch_bt<1, 1, T>(g, mode, w, x, b, y, s);
+  else if (!varnu) launch_bt<2, 0, T>(g, mode, w, x, b, y, s);
+  else launch_bt<2, 1, T>(g, mode, w, x, b, y, s);
+}
+
+template <class T>
+void uzawa_pressure(int disc, int varnu, const Geo& g, const T* w, const ResTabs<T>* tabs, T* x, const T* b, T* tmp,
+                    const double* inv_mlhat, double sc, cudaStream_t s) {
+  if (disc == 1 && !varnu) launch_pressure<1, 0, T>(g, w, tabs, x, b, tmp, inv_mlhat, sc, s);
+  else if (disc == 1) launch_pressure<1, 1, T>(g, w, tabs, x, b, tmp, inv_mlhat, sc, s);
+  else if (!varnu) launch_pressure<2, 0, T>(g, w, tabs, x, b, tmp, inv_mlhat, sc, s);
+  else launch_pressure<2, 1, T>(g, w, tabs, x, b, tmp, inv_mlhat, sc, s);
+}
+
+#define HHG_INST(T)                                                                                                   \
+  template void bt_rows<T>(int, int, int, const Geo&, const T*, const T*, const T*, T*, cudaStream_t);                \
+  template void uzawa_pressure<T>(int, int, const Geo&, const T*, const ResTabs<T>*, T*, const T*, T*, const double*, \
+                                  double, cudaStream_t);
+HHG_INST(double)
+HHG_INST(float)
+
+}  // namespace hhg

@@ -22,8 +22,7 @@ struct Shape {
   int row_kplanes = 2;
   int row_sites = 1;
   int gs_threads = 128;    // threads per block of the Gauss-Seidel kernels
-  int gs_lanes = 1;        // lanes sharing the terms of one Gauss-Seidel site (1, 2, 4): edge groups
-  int gs_lanes0 = 1;       // the same for the vertex group (its colour phases)
+  int gs_lanes = 1;        // reported by hhg_get_launch_shape; a Gauss-Seidel site has one lane
   int gs_threads0 = 0;     // threads per block of the vertex colour phases (0 = gs_threads)
   // streaming kernels (stream.cu) of the full operator: threads per block (0 =
   // the unstaged rows), in the V-cycle precision (st_threads) and in FP64
@@ -36,23 +35,10 @@ struct Shape {
   // sweeps of one component before the next: its arrays stay in L2 on levels
   // whose vectors exceed it)
   int gs_comp_major = 0;
+  int gs_edge_sums = 0;    // P2: the vertex colours on shared edge sums (gs_vertex_phases)
 };
 
 // number of interior terms of a specialised operator (-1 if none)
 int fast_terms(int disc, int varnu, int op);
-
-// one Gauss-Seidel phase (group, colour) on the three velocity components
-// (comp = -1) or on velocity component comp (0..2) only (A is block diagonal
-// over the components, so each component's iterates are the same either
-// way); `tab` points to a host FastTab<T, fast_terms(disc, varnu, OP_A)>
-template <class T>
-void fast_gs(int disc, int varnu, const Geo& g, const void* tab, int grp, int colour, double inv_diag, T* u,
-             const T* rhs, const Shape& sh, cudaStream_t s, int comp = -1);
-
-// the same call as a work item of a batch being recorded (batch.h): the
-// batched kernels live in their own translation units
-template <class T>
-void fast_gs_record(int disc, int varnu, const Geo& g, const void* tab, int grp, int colour, double inv_diag, T* u,
-                    const T* rhs, const Shape& sh, int comp);
 
 }  // namespace hhg

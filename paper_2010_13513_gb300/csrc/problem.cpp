@@ -16,6 +16,7 @@
 #include "batch.h"
 #include "dfres.h"
 #include "fast.h"
+#include "gs.h"
 #include "internal.h"
 #include "kernels.h"
 #include "nn.h"
@@ -139,6 +140,12 @@ struct Level {
   // weight tables (ResTabs) of the shared-memory-resident smoother: offsets
   // in the table blob, device addresses
   size_t o_rtab64 = 0, o_rtab32 = 0;
+  // the rows of A for the separate Gauss-Seidel launches (gs.cu), and their
+  // scratch (P2: three group arrays)
+  GsRows<double> grows64{};
+  GsRows<float> grows32{};
+  size_t o_gscr = 0;
+  char* gscr = nullptr;
   const ResTabs<double>* rtab64 = nullptr;
   const ResTabs<float>* rtab32 = nullptr;
   int rctas[2] = {0, 0};                // CTAs of the resident smoother per precision (0: per-phase kernels)
@@ -406,6 +413,19 @@ extern "C" int hhg_problem_create(const hhg_mesh* mesh, const hhg_problem_desc* 
       of.rows = B.put(h.rows); of.terms = B.put(h.terms); of.w64 = B.put(h.w64); of.w32 = B.put(w32);
       of.bterms = B.put(h.bterms); of.bw64 = B.put(h.bw64); of.bw32 = B.put(bw32);
     }
+    for (int gg = 0; gg < pb->G; ++gg) {
+      const std::vector<HTerm>& row = lv.st.op[OP_A].rows[size_t(gg)].seg[1];
+      if (row.size() > size_t(kGsTerms)) return fail(HHG_EINVAL, "internal: row of A longer than expected");
+      for (size_t t = 0; t < row.size(); ++t) {
+        lv.grows64.w[gg][t] = row[t].w;
+        lv.grows32.w[gg][t] = float(row[t].w);
+      }
+      lv.grows64.inv_diag[gg] = lv.inv_diag[gg];
+      lv.grows32.inv_diag[gg] = float(lv.inv_diag[gg]);
+    }
+    // (until hhg_autotune times it: above a million sites the vertex phases
+    // are worth the separate pass over the edges)
+    lv.shape.gs_edge_sums = pb->G == 8 && int64_t(lv.g.nx + 1) * (lv.g.ny + 1) * (lv.g.nz + 1) > 1000000 ? 1 : 0;
     HHG_TRY(put_res_tabs<double>(B, lv, c_class, lv.o_rtab64));
     HHG_TRY(put_res_tabs<float>(B, lv, c_class, lv.o_rtab32));
   }
@@ -426,6 +446,9 @@ extern "C" int hhg_problem_create(const hhg_mesh* mesh, const hhg_problem_desc* 
       lv.o_x32 = off; off += v32;
       lv.o_b32 = off; off += v32;
       lv.o_tmp32 = off; off += v32;
+    }
+    if (pb->G == 8) {
+      lv.o_gscr = off; off += 3 * a64;
     }
     lv.o_invml = off; off += a64;
     lv.o_ml = off; off += a64;
@@ -693,6 +716,41 @@ int default_resident(hhg_problem* pb, Level& lv, int prec) {
   return set_resident(pb, lv, prec, 0);
 }
 
+template <class T> const GsRows<T>& grows(const Level& lv);
+template <> const GsRows<double>& grows<double>(const Level& lv) { return lv.grows64; }
+template <> const GsRows<float>& grows<float>(const Level& lv) { return lv.grows32; }
+
+// xi Gauss-Seidel sweeps on A u = rhs (forward, and backward for A_s) in
+// separate launches.  A is block diagonal over the velocity components:
+// either every phase on all three components, or (gs_comp_major) all sweeps
+// of one component after another -- the same iterates.  gs_edge_sums: the
+// vertex colours share one pass over their edge terms.
+template <class T>
+void gs_sweeps(hhg_problem* pb, Level& lv, const Shape& sh, int xi, bool symmetric, T* u, const T* rhs) {
+  const int G = lv.g.G, disc = pb->desc.disc, varnu = pb->desc.nu_a != 0.0 ? 1 : 0;
+  const bool cm = sh.gs_comp_major != 0, sums = sh.gs_edge_sums && !cm && G == 8;
+  const int vt = sh.gs_threads0 ? sh.gs_threads0 : sh.gs_threads;
+  for (int c = 0; c < (cm ? 3 : 1); ++c) {
+    auto phase = [&](int ph) {                     // 0..3 the vertex colours, then the edge groups
+      gs_phase<T>(disc, varnu, lv.g, grows<T>(lv), ph < 4 ? 0 : ph - 3, ph < 4 ? ph : -1, u, rhs, c, cm ? 1 : 3,
+                  ph < 4 ? vt : sh.gs_threads, pb->stream);
+    };
+    auto vertices = [&](bool reverse) {
+      if (sums)
+        gs_vertex_phases<T>(varnu, lv.g, grows<T>(lv), reverse, u, rhs, reinterpret_cast<T*>(lv.gscr), vt, pb->stream);
+      else
+        for (int p = 0; p < 4; ++p) phase(reverse ? 3 - p : p);
+    };
+    for (int s = 0; s < xi; ++s) {
+      vertices(false);
+      for (int gg = 1; gg < G; ++gg) phase(gg + 3);
+      if (!symmetric) continue;
+      for (int gg = G - 1; gg >= 1; --gg) phase(gg + 3);
+      vertices(true);
+    }
+  }
+}
+
 template <class T>
 int uzawa(hhg_problem* pb, Level& lv, const hhg_params& prm, int sweeps, T* x, const T* b, T* tmp) {
   const int G = lv.g.G;
@@ -713,29 +771,12 @@ int uzawa(hhg_problem* pb, Level& lv, const hhg_params& prm, int sweeps, T* x, c
     pb->wu_counted += sweeps * level_weight(pb, lv) * (prm.xi * (prm.ahat == HHG_AHAT_S ? 2 : 1) * cs.A + 2 * cs.B + cs.C);
     return HHG_OK;
   }
-  std::vector<std::pair<int, int>> phases;
-  for (int c = 0; c < 4; ++c) phases.push_back({0, c});
-  for (int gg = 1; gg < G; ++gg) phases.push_back({gg, -1});
   const Costs cs = block_costs(pb->ov);
   for (int it = 0; it < sweeps; ++it) {
     // velocity step (Eq. uzawa-velocity): f' = f - B^T p_k, xi GS sweeps on A u = f'
     const int disc = pb->desc.disc, varnu = pb->desc.nu_a != 0.0 ? 1 : 0;
     bt_rows<T>(disc, varnu, MODE_RES, lv.g, static_cast<const T*>(ftab<T>(lv, OP_BT)), x, b, tmp, pb->stream);
-    const void* tabA = ftab<T>(lv, OP_A);
-    // A is block diagonal over the velocity components: either every phase
-    // on all three components, or all sweeps of one component after another
-    // (the same iterates)
-    const bool cm = lv.shape.gs_comp_major != 0;
-    for (int c = cm ? 0 : -1; c < (cm ? 3 : 0); ++c)
-      for (int s = 0; s < prm.xi; ++s) {
-        for (auto& ph : phases)
-          fast_gs<T>(disc, varnu, lv.g, tabA, ph.first, ph.second, lv.inv_diag[ph.first], x, tmp, lv.shape, pb->stream,
-                     c);
-        if (prm.ahat == HHG_AHAT_S)
-          for (auto it2 = phases.rbegin(); it2 != phases.rend(); ++it2)
-            fast_gs<T>(disc, varnu, lv.g, tabA, it2->first, it2->second, lv.inv_diag[it2->first], x, tmp, lv.shape,
-                       pb->stream, c);
-      }
+    gs_sweeps<T>(pb, lv, lv.shape, prm.xi, prm.ahat == HHG_AHAT_S, x, tmp);
     HHG_CHECK_LAUNCH();
     // pressure step (Eq. uzawa-pressure): p -= S_hat^{-1} (g - B u_{k+1} + C p_k)
     uzawa_pressure<T>(disc, varnu, lv.g, static_cast<const T*>(ftab<T>(lv, OP_BC)), rtab<T>(lv), x, b, tmp,
@@ -1107,6 +1148,7 @@ extern "C" int hhg_problem_bind(hhg_problem* pb, void* workspace, size_t bytes, 
     }
     lv.rtab64 = reinterpret_cast<const ResTabs<double>*>(tb + lv.o_rtab64);
     lv.rtab32 = reinterpret_cast<const ResTabs<float>*>(tb + lv.o_rtab32);
+    lv.gscr = ws + lv.o_gscr;
     lv.inv_mlhat = reinterpret_cast<double*>(ws + lv.o_invml);
     lv.ml = reinterpret_cast<double*>(ws + lv.o_ml);
   }
@@ -1490,7 +1532,6 @@ extern "C" int hhg_set_launch_shape(hhg_problem* pb, int level, int row_threads,
   sh.st_sites = row_sites == 2 ? 2 : 4;
   sh.row_sites = row_sites == 2 ? 4 : row_sites;
   sh.gs_lanes = gs_lanes;
-  sh.gs_lanes0 = gs_lanes;
   sh.gs_threads0 = 0;
   for (auto& kv : pb->graphs) cudaGraphExecDestroy(kv.second.exec);
   pb->graphs.clear();
@@ -1905,60 +1946,33 @@ int tune_level(hhg_problem* pb, Level& lv, int reps, T* xa, T* xb) {
     tune_rows(xa, xb, bestS.st_threads, &bestS.st_sites);
     tune_rows(lv.tmp64, lv.bw64, bestS.st64_threads, nullptr);
   }
-  // Gauss-Seidel kernels: one forward sweep, 1, 2 or 4 lanes per site; the
-  // lanes of the vertex colours and of the edge groups are then chosen apart
-  float best = 1e30f;
-  auto sweep = [&](const Shape& sh, bool vertex, bool edges) {
-    if (vertex)
-      for (int c = 0; c < 4; ++c) fast_gs<T>(disc, varnu, lv.g, ftab<T>(lv, OP_A), 0, c, 1.0, xb, xa, sh, pb->stream);
-    if (edges)
-      for (int gg = 1; gg < lv.g.G; ++gg) fast_gs<T>(disc, varnu, lv.g, ftab<T>(lv, OP_A), gg, -1, 1.0, xb, xa, sh, pb->stream);
-  };
-  for (int nl : {1, 2, 4})
-    for (int t : threads) {
-      Shape sh = bestS;
-      sh.gs_threads = t;
-      sh.gs_lanes = sh.gs_lanes0 = nl;
-      const float ms = time_it([&] { sweep(sh, true, true); });
-      if (ms < best) { best = ms; bestS.gs_threads = t; bestS.gs_lanes = bestS.gs_lanes0 = nl; }
-    }
-  if (lv.g.G > 1) {
-    float bv = 1e30f, be = 1e30f;
-    int lv0 = bestS.gs_lanes0, tv0 = bestS.gs_threads, le = bestS.gs_lanes, te = bestS.gs_threads;
-    for (int nl : {1, 2, 4})
-      for (int t : threads) {
-        Shape sh = bestS;
-        sh.gs_lanes = sh.gs_lanes0 = nl;
-        sh.gs_threads = t;
-        sh.gs_threads0 = 0;
-        const float mv = time_it([&] { sweep(sh, true, false); });
-        const float me = time_it([&] { sweep(sh, false, true); });
-        if (mv < bv) { bv = mv; lv0 = nl; tv0 = t; }
-        if (me < be) { be = me; le = nl; te = t; }
-      }
-    bestS.gs_lanes0 = lv0;
-    bestS.gs_threads0 = tv0;
-    bestS.gs_lanes = le;
-    bestS.gs_threads = te;
-  }
-  // launch order of a smoothing step's phases: every phase on all three
-  // components, or component by component (two forward sweeps each)
+  // Gauss-Seidel phases: threads per block, the vertex colours and the edge
+  // groups apart
   {
-    auto sweeps = [&](const Shape& sh) {
-      for (int c = sh.gs_comp_major ? 0 : -1; c < (sh.gs_comp_major ? 3 : 0); ++c)
-        for (int r = 0; r < 2; ++r) {
-          for (int cc = 0; cc < 4; ++cc)
-            fast_gs<T>(disc, varnu, lv.g, ftab<T>(lv, OP_A), 0, cc, 1.0, xb, xa, sh, pb->stream, c);
-          for (int gg = 1; gg < lv.g.G; ++gg)
-            fast_gs<T>(disc, varnu, lv.g, ftab<T>(lv, OP_A), gg, -1, 1.0, xb, xa, sh, pb->stream, c);
-        }
-    };
-    Shape sh = bestS;
-    sh.gs_comp_major = 0;
-    const float m0 = time_it([&] { sweeps(sh); });
-    sh.gs_comp_major = 1;
-    const float m1 = time_it([&] { sweeps(sh); });
-    bestS.gs_comp_major = m1 < m0 ? 1 : 0;
+    float bv = 1e30f, be = 1e30f;
+    for (int t : threads) {
+      auto phases = [&](int p0, int p1) {
+        for (int p = p0; p < p1; ++p)
+          gs_phase<T>(disc, varnu, lv.g, grows<T>(lv), p < 4 ? 0 : p - 3, p < 4 ? p : -1, xb, xa, 0, 3, t, pb->stream);
+      };
+      const float mv = time_it([&] { phases(0, 4); }), me = time_it([&] { phases(4, lv.g.G + 3); });
+      if (mv < bv) { bv = mv; bestS.gs_threads0 = t; }
+      if (me < be) { be = me; bestS.gs_threads = t; }
+    }
+  }
+  // launch order of a smoothing step's phases (two forward sweeps): every
+  // phase on all three components, the same with the vertex colours on shared
+  // edge sums, or component by component
+  {
+    float bo = 1e30f;
+    for (int o = 0; o < 3; ++o) {
+      if (o == 1 && lv.g.G == 1) continue;
+      Shape sh = bestS;
+      sh.gs_edge_sums = o == 1;
+      sh.gs_comp_major = o == 2;
+      const float ms = time_it([&] { gs_sweeps<T>(pb, lv, sh, 2, false, xb, xa); });
+      if (ms < bo) { bo = ms; bestS.gs_edge_sums = sh.gs_edge_sums; bestS.gs_comp_major = sh.gs_comp_major; }
+    }
   }
   lv.shape = bestS;
   cudaEventDestroy(e0);
@@ -2026,8 +2040,7 @@ extern "C" int hhg_autotune(hhg_problem* pb, int reps, int* shapes_out) {
       o[4] = lv.rthreads[mixed ? HHG_FP32 : HHG_FP64];
       o[5] = lv.shape.st_threads;
       o[6] = lv.shape.row_sites;
-      o[7] = lv.shape.gs_lanes;
-      o[8] = lv.shape.gs_lanes0;
+      o[7] = o[8] = 1;                             // lanes per Gauss-Seidel site
       // (the smoother's B^T and (B, -C) rows have one launch shape, uzrows.cu)
       o[9] = 128; o[10] = 1; o[11] = 1;
       o[12] = 256; o[13] = 1; o[14] = 1;

@@ -275,6 +275,16 @@ void launch_full(const FullA<T>& a, const void* tab, cudaStream_t s) {
 
 }  // namespace
 
+int fast_terms(int disc, int varnu, int op) {
+#define HHG_N(D, V, O) if (disc == D && varnu == V && op == O) return gen::S<D, V, O>::N;
+  HHG_N(1, 0, OP_FULL) HHG_N(1, 0, OP_A) HHG_N(1, 0, OP_BT) HHG_N(1, 0, OP_BC)
+  HHG_N(1, 1, OP_FULL) HHG_N(1, 1, OP_A) HHG_N(1, 1, OP_BT) HHG_N(1, 1, OP_BC)
+  HHG_N(2, 0, OP_FULL) HHG_N(2, 0, OP_A) HHG_N(2, 0, OP_BT) HHG_N(2, 0, OP_BC)
+  HHG_N(2, 1, OP_FULL) HHG_N(2, 1, OP_A) HHG_N(2, 1, OP_BT) HHG_N(2, 1, OP_BC)
+#undef HHG_N
+  return -1;
+}
+
 template <class T>
 void full_rows(int disc, int varnu, int mode, const Geo& g, const void* tab, const ResTabs<T>* tabs, const T* x,
                const T* b, T* y, cudaStream_t s) {

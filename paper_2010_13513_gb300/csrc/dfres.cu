@@ -19,13 +19,15 @@
 // if evaluated in 47-bit arithmetic and then rounded to FP32, the precision
 // the V-cycle takes its right-hand side in.
 //
-// Work layout (as the vector row kernels of the FP32/FP64 path): grid x over
-// the padded (i, j) plane in warps of 4 x 32 positions, y over groups of kp
-// planes, z over the rows of the operator; on large levels a thread
-// evaluates 4 sites 32 positions apart (two at a time with the paired FP32
-// f32x2 instructions) on 2 planes, on small ones 1 site on 1 plane.
-// The terms of a row are a loop over weights and offsets in the constant
-// bank, so a row's code stays small in the instruction cache.
+// Work layout.  Constant viscosity (k_df_unrolled): a thread owns two sites
+// of a plane and a component and applies each (hi, lo) input it loads to all
+// the component's rows, two sites per paired FP32 (f32x2) instruction; rows
+// are unrolled, with small-integer weights (see there).  Variable viscosity
+// (k_res_df): grid x over the padded (i, j) plane in warps of 4 x 32
+// positions, y over groups of kp planes, z over the rows of the operator; on
+// large levels a thread evaluates 4 sites 32 positions apart on 2 planes, on
+// small ones 1 site on 1 plane, in a loop over weights and offsets in the
+// constant bank.
 // Boundary pressure rows (P1-P1: the C terms of the cubes inside the box) add
 // their per-cube C terms in FP64; they are a few per cent of the pressure
 // rows.  With a variable viscosity nu = exp(a z) the segments of a row are
@@ -39,6 +41,7 @@
 #include <cstdint>
 #include <cstring>
 #include <type_traits>
+#include <utility>
 
 #include "batch.h"
 #include "kernels.h"
@@ -334,6 +337,245 @@ __global__ void __launch_bounds__(128) k_res_df(Geo g, const float* __restrict__
   res_df_body<DISC, VARNU, V>(blockIdx, g, xh, xl, b, r, op, kp, tab);
 }
 
+// ---------------------------------------------- constant viscosity, unrolled
+// With a constant viscosity the weights at h = 1 are multiples of 1 / 15 (A)
+// and 1 / 60 (B, B^T; P1-P1: 1 and 1 / 12): times K = 15, 60 (1, 12) they are
+// small integers, exact in FP32, so a term has no low weight part, and a term
+// whose integer is a power of two has an exact product.  A row then takes the
+// factor h / K (h^2 / K) once, in double-float arithmetic.  Only the interior
+// C terms of P1-P1 (weights with |T|^(2/3)) keep two-part weights.  Eight to
+// eleven operations per term instead of twelve, two loads per input instead of
+// per term, no loop: the loop over table entries that this replaces spent about
+// 20 instructions per term and site.  P2-P1 level 7, with the split of x: 1.75
+// ms before, 1.15 ms now; level 6: 259 us before, 171 us.  Bound: instruction
+// issue.
+template <int DISC> constexpr double kScaleA = DISC == 2 ? 15.0 : 1.0;
+template <int DISC> constexpr double kScaleB = DISC == 2 ? 60.0 : 12.0;
+constexpr double rounded(double v) { return v < 0 ? -double(int64_t(0.5 - v)) : double(int64_t(v + 0.5)); }
+constexpr bool near_integer(double v) {
+  const double d = v - rounded(v);
+  return d < 1e-9 && d > -1e-9;
+}
+constexpr bool power_of_two(double v) {
+  if (v < 0) v = -v;
+  for (double p = 1.0; p <= 64.0; p *= 2.0)
+    if (v == p) return true;
+  return false;
+}
+
+__device__ __forceinline__ float2 both(float v) { return make_float2(v, v); }
+__device__ __forceinline__ float2 neg2(float2 v) { return make_float2(-v.x, -v.y); }
+
+// (s, c) += p + e on two sites: TwoSum of s and p
+__device__ __forceinline__ void add_exact2(float2 p, float2 e, float2& s, float2& c) {
+  const float2 t = __fadd2_rn(s, p);
+  const float2 z = sub2(t, s);
+  const float2 d = __fadd2_rn(sub2(s, sub2(t, z)), sub2(p, z));
+  s = t;
+  c = __fadd2_rn(c, __fadd2_rn(d, e));
+}
+
+// term E of operator table S times K: the integer weight (or, K = 0, the
+// two-part weight at h = 1) times x on two sites
+template <class S, int E, int K>
+__device__ __forceinline__ void unrolled_term(float2 xh, float2 xl, float2& s, float2& c) {
+  if constexpr (K == 0) {
+    constexpr double w = S::wref[E];
+    constexpr float wh = float(w), wl = float(w - double(wh));
+    dot2_term2(both(wh), both(wl), xh, xl, s, c);
+  } else {
+    constexpr double wk = S::wref[E] * K;
+    static_assert(near_integer(wk) && wk > -1024.0 && wk < 1024.0, "the scaled weights are small integers");
+    constexpr float w = float(rounded(wk));
+    if constexpr (power_of_two(w)) {
+      add_exact2(__fmul2_rn(both(w), xh), __fmul2_rn(both(w), xl), s, c);
+    } else {
+      const float2 p = __fmul2_rn(both(w), xh);
+      add_exact2(p, __ffma2_rn(both(w), xl, __ffma2_rn(both(w), xh, neg2(p))), s, c);
+    }
+  }
+}
+
+// (s, c) = a (s + c) for an FP64 factor a
+__device__ __forceinline__ void df_scale(double a, float& s, float& c) {
+  float u = s, v = c;
+  s = c = 0.0f;
+  df_add_scaled(a, u, v, s, c);
+}
+
+// two sites of the split vector: d positions apart
+struct Pair {
+  const float* h0; const float* h1; const float* l0; const float* l1;
+  __device__ __forceinline__ float2 hi(int64_t o) const { return make_float2(__ldg(h0 + o), __ldg(h1 + o)); }
+  __device__ __forceinline__ float2 lo(int64_t o) const { return make_float2(__ldg(l0 + o), __ldg(l1 + o)); }
+};
+
+// the terms of line L of the full operator's plan at i offset DI, pressure
+// inputs (PR) or velocity inputs, on the pass's velocity rows
+template <class S, class SPT, int Q, int L, int DI, int K>
+constexpr bool df_line_reads() {
+  for (int e = SPT::lines[L].e0; e < SPT::lines[L].e0 + SPT::lines[L].ne; ++e)
+    if (SPT::terms[e].di == DI && !SPT::parts[SPT::passes[Q].p0 + SPT::terms[e].part].all) return true;
+  return false;
+}
+template <class S, class SPT, int Q, int L, int DI, int K, int NP, int... I>
+__device__ __forceinline__ void df_line_value(const Pair& p, int64_t o, float2 (&s)[NP], float2 (&c)[NP],
+                                              std::integer_sequence<int, I...>) {
+  if constexpr (df_line_reads<S, SPT, Q, L, DI, K>()) {
+    const float2 xh = p.hi(o + DI), xl = p.lo(o + DI);
+    ([&] {
+      constexpr gen::TermE te = SPT::terms[SPT::lines[L].e0 + I];
+      if constexpr (te.di == DI && !SPT::parts[SPT::passes[Q].p0 + te.part].all)
+        unrolled_term<S, te.t, K>(xh, xl, s[te.part], c[te.part]);
+    }(), ...);
+  }
+}
+template <class S, class SPT, int Q, int L, int PARR, bool PR, int K, int NP>
+__device__ __forceinline__ void df_line(const Geo& g, const Pair& p, float2 (&s)[NP], float2 (&c)[NP]) {
+  constexpr gen::LineT ln = SPT::lines[L];
+  constexpr int arr = SPT::arrs[SPT::passes[Q].a0 + ln.slot];
+  if constexpr ((arr == PARR) == PR) {
+    const int64_t o = arr * g.arr + ln.dj * g.sx + ln.dk * g.sy;
+    const auto all = std::make_integer_sequence<int, ln.ne>{};
+    df_line_value<S, SPT, Q, L, -1, K>(p, o, s, c, all);
+    df_line_value<S, SPT, Q, L, 0, K>(p, o, s, c, all);
+    df_line_value<S, SPT, Q, L, 1, K>(p, o, s, c, all);
+  }
+}
+template <class S, class SPT, int Q, int PARR, bool PR, int K, int NP, int... L>
+__device__ __forceinline__ void df_lines(const Geo& g, const Pair& p, float2 (&s)[NP], float2 (&c)[NP],
+                                         std::integer_sequence<int, L...>) {
+  (df_line<S, SPT, Q, SPT::passes[Q].l0 + L, PARR, PR, K>(g, p, s, c), ...);
+}
+// terms [T0, T0 + n) of a row in two chains, added up
+template <class S, int T0, int K, int... I>
+__device__ __forceinline__ void df_chain(const Geo& g, const Pair& p, float2& s, float2& c,
+                                         std::integer_sequence<int, I...>) {
+  float2 s2[3] = {}, c2[3] = {};
+  ([&] {
+    constexpr gen::OffT o = S::off[T0 + I];
+    const int64_t q = o.arr * g.arr + o.di + o.dj * g.sx + o.dk * g.sy;
+    unrolled_term<S, T0 + I, K>(p.hi(q), p.lo(q), s2[I % 3], c2[I % 3]);
+  }(), ...);
+  s = s2[0];
+  c = c2[0];
+  add_exact2(s2[1], c2[1], s, c);
+  add_exact2(s2[2], c2[2], s, c);
+}
+
+struct DfA { Geo g; const float* xh; const float* xl; const double* b; float* r; OpDev op; int d; };
+
+// the rows of pass Q (P2-P1: a component, P1-P1: all three) at two sites
+template <int DISC, int Q, int... P>
+__device__ __forceinline__ void df_velocity(const DfA& a, const Pair& p, const int (&i)[2], const int (&j)[2], int k,
+                                            const int64_t (&idx)[2], std::integer_sequence<int, P...>) {
+  using S = gen::S<DISC, 0, OP_FULL>;
+  using SPT = gen::SP<DISC, 0, OP_FULL>;
+  constexpr gen::PassT ps = SPT::passes[Q];
+  constexpr int PARR = DISC == 2 ? 24 : 3;
+  const Geo& g = a.g;
+  float2 s[ps.np] = {}, c[ps.np] = {};
+  const auto lines = std::make_integer_sequence<int, ps.nl>{};
+  // B^T first, brought to the scale of A: (h^2 / KB) / (h / KA)
+  df_lines<S, SPT, Q, PARR, true, int(kScaleB<DISC>)>(g, p, s, c, lines);
+  const double ratio = g.h * (kScaleA<DISC> / kScaleB<DISC>);
+#pragma unroll
+  for (int r = 0; r < ps.np; ++r) {
+    df_scale(ratio, s[r].x, c[r].x);
+    df_scale(ratio, s[r].y, c[r].y);
+  }
+  df_lines<S, SPT, Q, PARR, false, int(kScaleA<DISC>)>(g, p, s, c, lines);
+  const double scale = g.h / kScaleA<DISC>;
+  ([&] {
+    constexpr gen::PartT pt = SPT::parts[ps.p0 + P];
+    if constexpr (!pt.all) {
+      constexpr int ox = (0xB2 >> pt.og) & 1, oy = (0xD4 >> pt.og) & 1, oz = (0xE8 >> pt.og) & 1;
+      df_scale(scale, s[P].x, c[P].x);
+      df_scale(scale, s[P].y, c[P].y);
+#pragma unroll
+      for (int v = 0; v < 2; ++v) {
+        if (i[v] > g.nx - ox || j[v] > g.ny - oy || k > g.nz - oz) continue;
+        const bool bnd = (!ox && (i[v] == 0 || i[v] == g.nx)) || (!oy && (j[v] == 0 || j[v] == g.ny)) ||
+                         (!oz && (k == 0 || k == g.nz));
+        df_store<pt.out, 0, 0, 0>(g, a.op, pt.row, i[v], j[v], k, bnd, a.xh, a.xl, idx[v], v ? s[P].y : s[P].x,
+                                  v ? c[P].y : c[P].x, 0.0f, 0.0f, 0.0f, 0.0f, a.b, a.r);
+      }
+    }
+  }(), ...);
+}
+template <int DISC>
+__device__ __forceinline__ void df_pressure(const DfA& a, const Pair& p, const int (&i)[2], const int (&j)[2], int k,
+                                            const int64_t (&idx)[2]) {
+  using S = gen::S<DISC, 0, OP_FULL>;
+  constexpr int PARR = DISC == 2 ? 24 : 3;
+  constexpr gen::RowS rw = S::rows[PARR];
+  static_assert(rw.out == PARR && rw.n1 == 0, "the last row is the pressure's; B is unscaled");
+  const Geo& g = a.g;
+  float2 s, c, s2 = {}, c2 = {};
+  df_chain<S, rw.t0, int(kScaleB<DISC>)>(g, p, s, c, std::make_integer_sequence<int, rw.n0>{});
+  const double sb = g.h * g.h / kScaleB<DISC>;
+  df_scale(sb, s.x, c.x);
+  df_scale(sb, s.y, c.y);
+  if constexpr (rw.n2 > 0) {
+    df_chain<S, rw.t0 + rw.n0, 0>(g, p, s2, c2, std::make_integer_sequence<int, rw.n2>{});
+    const double sc = g.h * g.h * g.h;
+    df_scale(sc, s2.x, c2.x);
+    df_scale(sc, s2.y, c2.y);
+  }
+#pragma unroll
+  for (int v = 0; v < 2; ++v) {
+    if (i[v] > g.nx || j[v] > g.ny) continue;
+    const bool bnd = i[v] == 0 || i[v] == g.nx || j[v] == 0 || j[v] == g.ny || k == 0 || k == g.nz;
+    df_store<PARR, 1, rw.n2, 0>(g, a.op, PARR, i[v], j[v], k, bnd, a.xh, a.xl, idx[v], v ? s.y : s.x, v ? c.y : c.x,
+                                0.0f, 0.0f, v ? s2.y : s2.x, v ? c2.y : c2.x, a.b, a.r);
+  }
+}
+
+// grid x over the positions m = i + j sx of the padded (i, j) plane in warps
+// of 64 (a lane's two sites lie d = 32 apart; the last warp starts early
+// enough to end with the plane's last site, and planes of less than 64
+// positions take one site per lane: d = 0), y = plane, z = part: the
+// components (P1-P1: all at once), then the pressure
+template <int DISC>
+__device__ __forceinline__ void df_unrolled_body(const uint3 bid, const DfA& a) {
+  using SPT = gen::SP<DISC, 0, OP_FULL>;
+  const Geo& g = a.g;
+  const int mlast = g.ny * g.sx + g.nx, span = a.d ? 64 : 32, lane = int(threadIdx.x & 31);
+  int m0 = int((bid.x * blockDim.x + threadIdx.x) >> 5) * span;
+  if (m0 > mlast) return;
+  if (a.d) m0 = min(m0, mlast - 63);
+  const int k = bid.y;
+  int i[2], j[2];
+  int64_t idx[2];
+#pragma unroll
+  for (int v = 0; v < 2; ++v) {
+    const int m = min(m0 + lane + v * a.d, mlast);
+    j[v] = m / g.sx;
+    i[v] = m - j[v] * g.sx;
+    idx[v] = int64_t(m) + 1 + g.sx + int64_t(k + 1) * g.sy;
+  }
+  const Pair p{a.xh + idx[0], a.xh + idx[1], a.xl + idx[0], a.xl + idx[1]};
+  if constexpr (DISC == 1) {
+    if (bid.z == 0) df_velocity<1, 0>(a, p, i, j, k, idx, std::make_integer_sequence<int, SPT::passes[0].np>{});
+    else df_pressure<1>(a, p, i, j, k, idx);
+  } else {
+    if (bid.z == 0) df_velocity<2, 0>(a, p, i, j, k, idx, std::make_integer_sequence<int, SPT::passes[0].np>{});
+    else if (bid.z == 1) df_velocity<2, 1>(a, p, i, j, k, idx, std::make_integer_sequence<int, SPT::passes[1].np>{});
+    else if (bid.z == 2) df_velocity<2, 2>(a, p, i, j, k, idx, std::make_integer_sequence<int, SPT::passes[2].np>{});
+    else df_pressure<2>(a, p, i, j, k, idx);
+  }
+}
+template <int DISC>
+__global__ void __launch_bounds__(128) k_df_unrolled(const __grid_constant__ DfA a) {
+  df_unrolled_body<DISC>(blockIdx, a);
+}
+template <int DISC>
+__global__ void __launch_bounds__(128) kb_df_unrolled(const void* items, int n) {
+  uint3 bid, gd;
+  const auto& it = batch_item<DfA>(items, n, bid, gd);
+  df_unrolled_body<DISC>(bid, it.a);
+}
+
 // hi[q] + lo[q] = x[q] (split_df), two elements per thread and step (n even)
 __device__ __forceinline__ void split_df_body(const uint3 bid, const uint3 gd, const double2* __restrict__ x,
                                               float2* __restrict__ hi, float2* __restrict__ lo, int64_t n2) {
@@ -378,6 +620,28 @@ constexpr int kDfThreads = 128;
 // ones four sites and two planes
 constexpr int64_t kDfSmallSites = 300000;
 
+template <int DISC>
+void launch_df_unrolled(const Geo& g, const OpDev& od, const double* x, const double* b, float* xh, float* xl,
+                        float* r, cudaStream_t s) {
+  const int64_t n2 = (3 * int64_t(g.G) + 1) * g.arr / 2;   // arr is a multiple of 64
+  const dim3 sgrd(unsigned(std::min<int64_t>((n2 + 255) / 256, 152 * 8)));
+  const SplitA sa{reinterpret_cast<const double2*>(x), reinterpret_cast<float2*>(xh), reinterpret_cast<float2*>(xl),
+                  n2};
+  const int mlast = g.ny * g.sx + g.nx, span = mlast >= 63 ? 64 : 32;
+  const int warps = mlast / span + 1;
+  const dim3 grd(unsigned((warps * 32 + kDfThreads - 1) / kDfThreads), unsigned(g.nz + 1), DISC == 2 ? 4 : 2);
+  const DfA a{g, xh, xl, b, r, od, mlast >= 63 ? 32 : 0};
+  if (g_rec) {
+    g_rec->add(reinterpret_cast<const void*>(kb_split_df), sgrd, dim3(256), 0, 1, sa);
+    g_rec->add(reinterpret_cast<const void*>(kb_df_unrolled<DISC>), grd, dim3(kDfThreads), 0, 1, a);
+    return;
+  }
+  ++g_launches;
+  k_split_df<<<sgrd, 256, 0, s>>>(sa.x, sa.hi, sa.lo, n2);
+  ++g_launches;
+  k_df_unrolled<DISC><<<grd, kDfThreads, 0, s>>>(a);
+}
+
 template <int DISC, int VARNU>
 void launch_df(const Geo& g, const OpDev& od, const char* tab, const double* x, const double* b, float* xh, float* xl,
                float* r, cudaStream_t s) {
@@ -413,9 +677,9 @@ void launch_df(const Geo& g, const OpDev& od, const char* tab, const double* x, 
 
 void df_launch(int disc, int varnu, const Geo& g, const OpDev& od, const char* tab, const double* x, const double* b,
                float* xh, float* xl, float* r, cudaStream_t s) {
-  if (disc == 1 && !varnu) launch_df<1, 0>(g, od, tab, x, b, xh, xl, r, s);
+  if (disc == 1 && !varnu) launch_df_unrolled<1>(g, od, x, b, xh, xl, r, s);
   else if (disc == 1) launch_df<1, 1>(g, od, tab, x, b, xh, xl, r, s);
-  else if (!varnu) launch_df<2, 0>(g, od, tab, x, b, xh, xl, r, s);
+  else if (!varnu) launch_df_unrolled<2>(g, od, x, b, xh, xl, r, s);
   else launch_df<2, 1>(g, od, tab, x, b, xh, xl, r, s);
 }
 

@@ -32,11 +32,11 @@ void launch_gs(const Geo& g, const OpDev& A, int grp, int colour, double inv_dia
 template <class T>
 void launch_pupdate(const Geo& g, T* p, const T* r, const double* inv_mlhat, double inv_omega_inv, cudaStream_t s);
 
-// transfers of a whole block vector (transfer.cu): xf += I xc (interior_only:
-// Dirichlet velocity DoFs of xf untouched) and rc = I^T rf (Dirichlet velocity
-// rows 0)
+// transfers of a whole block vector (transfer.cu): xf += I xc, or xf = I xc
+// (set; interior_only: Dirichlet velocity DoFs of xf untouched, or 0 if set)
+// and rc = I^T rf (Dirichlet velocity rows 0)
 template <class T>
-void launch_prolong(const Geo& gf, const Geo& gc, bool interior_only, const T* xc, T* xf, cudaStream_t s);
+void launch_prolong(const Geo& gf, const Geo& gc, bool interior_only, bool set, const T* xc, T* xf, cudaStream_t s);
 template <class T>
 void launch_restrict(const Geo& gf, const Geo& gc, const T* rf, T* rc, cudaStream_t s);
 

@@ -800,7 +800,7 @@ template <class T>
 int prolong_add(hhg_problem* pb, int l, const T* xc, T* xf, bool velocity_interior_only = true) {
   Level& f = pb->L(l);
   Level& c = pb->L(l - 1);
-  launch_prolong<T>(f.g, c.g, velocity_interior_only, xc, xf, pb->stream);
+  launch_prolong<T>(f.g, c.g, velocity_interior_only, false, xc, xf, pb->stream);
   HHG_CHECK_LAUNCH();
   return HHG_OK;
 }
@@ -879,8 +879,9 @@ int fmg_interpolate(hhg_problem* pb, int l) {
   Level& f = pb->L(l);
   Level& c = pb->L(l - 1);
   launch_xpby<double>(c.x64, 1.0, c.W, c.tmp64, c.nvec(), pb->stream);
-  HHG_CUDA(launch_zero(f.x64, size_t(f.nvec()) * 8, pb->stream));
-  HHG_TRY(prolong_add<double>(pb, l, c.tmp64, f.x64, true));
+  // (halo and padding of the library's x are 0 and stay so)
+  launch_prolong<double>(f.g, c.g, true, true, c.tmp64, f.x64, pb->stream);
+  HHG_CHECK_LAUNCH();
   return HHG_OK;
 }
 

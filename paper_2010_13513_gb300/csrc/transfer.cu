@@ -8,7 +8,8 @@
 // row is unrolled over its non-zero ones, so that no table is read:
 //  * prolongation: one thread owns one coarse cell and one z position p_z of
 //    it, loads the coarse nodes once and updates 16 fine DoFs of a component
-//    (P1 fields: all 8 of the cell);
+//    (P1 fields: all 8 of the cell), as 8 aligned pairs of sites on levels
+//    with an even pitch (single sites lie two apart in the lanes);
 //  * restriction: one thread gathers one coarse DoF of one group (the blocks
 //    of a launch that run at the same time share the fine planes they read).
 // All components, groups and the pressure go in one launch (grid z).
@@ -18,9 +19,12 @@
 // these replace read a weight and an offset per term from memory (dependent
 // loads), divided a row's terms over lanes and took two launches each.
 // Measured (FP32, P2-P1, 2x1x1 cubes at level 6, restriction and prolongation):
-// 248 us before, 79 us now; their vectors once over HBM would take 26 us.
+// 248 us before, 64 us now (79 us with single sites instead of pairs); their
+// vectors once over HBM would take 26 us.  Level 7: restriction 372 us before,
+// 92 us now; prolongation 558 us before, 127 us now.
 #include <cuda_runtime.h>
 
+#include <cstdint>
 #include <type_traits>
 #include <utility>
 
@@ -75,8 +79,15 @@ __device__ __forceinline__ T p2_point(const T (&c)[NZ * 9], std::integer_sequenc
   return a;
 }
 
+// xf += v, or xf = v (SET)
+template <bool SET, class T>
+__device__ __forceinline__ void put(T* f, T v) {
+  if (SET) *f = v;
+  else *f += v;
+}
+
 // the 16 fine DoFs of one component at z position PZ of coarse cell (ax, ay, az)
-template <int PZ, class T, int... Q>
+template <int PZ, bool SET, class T, int... Q>
 __device__ __forceinline__ void prolong_p2(const Geo& gf, const Geo& gc, int ax, int ay, int az, bool interior_only,
                                            const T* __restrict__ xc, T* __restrict__ xf,
                                            std::integer_sequence<int, Q...>) {
@@ -91,20 +102,24 @@ __device__ __forceinline__ void prolong_p2(const Geo& gf, const Geo& gc, int ax,
   // doubled fine position of the point and its range: 1 .. 2 n - 1 inside
   const int lo = interior_only ? 1 : 0;
   const int Pz = 4 * az + PZ;
-  if (Pz < lo || Pz > 2 * gf.nz - lo) return;
+  if (Pz > 2 * gf.nz) return;
+  const bool inz = Pz >= lo && Pz <= 2 * gf.nz - lo;
   T* f0 = xf + xsite(gf, 2 * ax, 2 * ay, 2 * az);
   auto at = [&](auto qc) {
     constexpr int q = decltype(qc)::value, PX = q % 4, PY = q / 4;
     const int Px = 4 * ax + PX, Py = 4 * ay + PY;
-    if (Px < lo || Px > 2 * gf.nx - lo || Py < lo || Py > 2 * gf.ny - lo) return;
+    if (Px > 2 * gf.nx || Py > 2 * gf.ny) return;
+    const bool in = inz && Px >= lo && Px <= 2 * gf.nx - lo && Py >= lo && Py <= 2 * gf.ny - lo;
     T* f = f0 + group_at(PX & 1, PY & 1, PZ & 1) * gf.arr + (PX >> 1) + (PY >> 1) * gf.sx + (PZ >> 1) * gf.sy;
-    *f += p2_point<PX, PY, PZ, NZ>(c, std::make_integer_sequence<int, NZ * 9>{});
+    const T v = p2_point<PX, PY, PZ, NZ>(c, std::make_integer_sequence<int, NZ * 9>{});
+    if (in) put<SET>(f, v);
+    else if (SET) *f = T(0);                       // Dirichlet row
   };
   (at(std::integral_constant<int, Q>{}), ...);
 }
 
 // the 8 fine DoFs of one P1 field in coarse cell (ax, ay, az)
-template <class T>
+template <bool SET, class T>
 __device__ __forceinline__ void prolong_p1(const Geo& gf, const Geo& gc, int ax, int ay, int az, bool interior_only,
                                            const T* __restrict__ xc, T* __restrict__ xf) {
   T c[8];
@@ -117,8 +132,88 @@ __device__ __forceinline__ void prolong_p1(const Geo& gf, const Geo& gc, int ax,
   for (int q = 0; q < 8; ++q) {
     const int px = q & 1, py = q >> 1 & 1, pz = q >> 2;
     const int i = 2 * ax + px, j = 2 * ay + py, k = 2 * az + pz;
-    if (i < lo || i > gf.nx - lo || j < lo || j > gf.ny - lo || k < lo || k > gf.nz - lo) continue;
-    f0[px + py * gf.sx + pz * gf.sy] += q == 0 ? c[0] : T(0.5) * c[0] + T(0.5) * c[q];
+    if (i > gf.nx || j > gf.ny || k > gf.nz) continue;
+    const bool in = i >= lo && i <= gf.nx - lo && j >= lo && j <= gf.ny - lo && k >= lo && k <= gf.nz - lo;
+    T* f = f0 + px + py * gf.sx + pz * gf.sy;
+    if (in) put<SET>(f, q == 0 ? c[0] : T(0.5) * c[0] + T(0.5) * c[q]);
+    else if (SET) *f = T(0);
+  }
+}
+
+// Two fine sites of a row at a time, on levels with an even pitch: sites 2 a -
+// 1 and 2 a share an aligned pair, so that a thread owns the x positions 2, 3
+// of cell a - 1 and 0, 1 of cell a.  Sites outside the field's range (the halo
+// column, the row padding) are rewritten as they are, or as 0 (SET).
+template <class T> struct Pair2 { using type = float2; };
+template <> struct Pair2<double> { using type = double2; };
+template <bool SET, class T>
+__device__ __forceinline__ void put_pair(T* f, bool in0, bool in1, T v0, T v1) {
+  using P = typename Pair2<T>::type;
+  P p;
+  if (!SET) p = *reinterpret_cast<const P*>(f);
+  else p.x = p.y = T(0);
+  if (in0) p.x += v0;
+  if (in1) p.y += v1;
+  *reinterpret_cast<P*>(f) = p;
+}
+// point (PX, PY, PZ) of the cell whose first x node is number X0 of the five loaded
+template <int PX, int PY, int PZ, int NZ, int X0, class T, int... N>
+__device__ __forceinline__ T p2_point5(const T (&c)[NZ * 15], std::integer_sequence<int, N...>) {
+  T a = T(0);
+  ([&] {
+    constexpr double w = p2_weight(PX, PY, PZ, N % 3, N / 3 % 3, N / 9);
+    if constexpr (w != 0.0) a = fma(T(w), c[X0 + N % 3 + 5 * (N / 3)], a);
+  }(), ...);
+  return a;
+}
+template <int PZ, bool SET, class T, int... Q>
+__device__ __forceinline__ void prolong_p2_pair(const Geo& gf, const Geo& gc, int ax, int ay, int az,
+                                                bool interior_only, const T* __restrict__ xc, T* __restrict__ xf,
+                                                std::integer_sequence<int, Q...>) {
+  constexpr int NZ = PZ == 0 ? 1 : 3;
+  constexpr auto nodes = std::make_integer_sequence<int, NZ * 9>{};
+  T c[NZ * 15];
+  const T* x0 = xc + xsite(gc, ax - 1, ay, az);
+#pragma unroll
+  for (int n = 0; n < NZ * 15; ++n) {
+    const int nx = n % 5, ny = n / 5 % 3, nz = n / 15;
+    c[n] = __ldg(x0 + group_at(nx & 1, ny & 1, nz & 1) * gc.arr + (nx >> 1) + (ny >> 1) * gc.sx + (nz >> 1) * gc.sy);
+  }
+  const int lo = interior_only ? 1 : 0;
+  const int Pz = 4 * az + PZ;
+  if (Pz > 2 * gf.nz) return;
+  const bool inz = Pz >= lo && Pz <= 2 * gf.nz - lo;
+  T* f0 = xf + xsite(gf, 2 * ax - 1, 2 * ay, 2 * az);
+  auto at = [&](auto qc) {
+    constexpr int q = decltype(qc)::value, ODD = q & 1, PY = q >> 1;
+    const int Px = 4 * ax + ODD, Py = 4 * ay + PY;
+    if (Py > 2 * gf.ny) return;
+    const bool in = inz && Py >= lo && Py <= 2 * gf.ny - lo;
+    if (!SET && !in) return;
+    T* f = f0 + group_at(ODD, PY & 1, PZ & 1) * gf.arr + (PY >> 1) * gf.sx + (PZ >> 1) * gf.sy;
+    put_pair<SET>(f, in && Px - 2 >= lo && Px - 2 <= 2 * gf.nx - lo, in && Px >= lo && Px <= 2 * gf.nx - lo,
+                  p2_point5<2 + ODD, PY, PZ, NZ, 0>(c, nodes), p2_point5<ODD, PY, PZ, NZ, 2>(c, nodes));
+  };
+  (at(std::integral_constant<int, Q>{}), ...);
+}
+template <bool SET, class T>
+__device__ __forceinline__ void prolong_p1_pair(const Geo& gf, const Geo& gc, int ax, int ay, int az,
+                                                bool interior_only, const T* __restrict__ xc, T* __restrict__ xf) {
+  T c[8];                                          // x nodes a - 1 and a
+  const T* x0 = xc + xsite(gc, ax - 1, ay, az);
+#pragma unroll
+  for (int n = 0; n < 8; ++n) c[n] = __ldg(x0 + (n & 1) + (n >> 1 & 1) * gc.sx + (n >> 2) * gc.sy);
+  const int lo = interior_only ? 1 : 0;
+  T* f0 = xf + xsite(gf, 2 * ax - 1, 2 * ay, 2 * az);
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int py = q & 1, pz = q >> 1, i = 2 * ax, j = 2 * ay + py, k = 2 * az + pz;
+    if (j > gf.ny || k > gf.nz) continue;
+    const bool in = j >= lo && j <= gf.ny - lo && k >= lo && k <= gf.nz - lo;
+    if (!SET && !in) continue;
+    put_pair<SET>(f0 + py * gf.sx + pz * gf.sy, in && i - 1 >= lo && i - 1 <= gf.nx - lo,
+                  in && i >= lo && i <= gf.nx - lo, T(0.5) * c[0] + T(0.5) * c[1 + 2 * q],
+                  q == 0 ? c[1] : T(0.5) * c[1] + T(0.5) * c[1 + 2 * q]);
   }
 }
 
@@ -130,7 +225,19 @@ struct TransferA { Geo gf, gc; int interior_only; const T* in; T* out; };
 
 // grid: x over the (i, j) plane of coarse cells (flat), z = plane and part
 // (part fastest: blocks that run together share the coarse planes)
-template <int G, class T>
+template <int PZ, bool SET, bool PAIR, class T>
+__device__ __forceinline__ void prolong_p2_z(const Geo& gf, const Geo& gc, int ax, int ay, int az, bool io,
+                                             const T* xc, T* xf) {
+  if constexpr (PAIR) prolong_p2_pair<PZ, SET>(gf, gc, ax, ay, az, io, xc, xf, std::make_integer_sequence<int, 8>{});
+  else prolong_p2<PZ, SET>(gf, gc, ax, ay, az, io, xc, xf, std::make_integer_sequence<int, 16>{});
+}
+template <bool SET, bool PAIR, class T>
+__device__ __forceinline__ void prolong_field(const Geo& gf, const Geo& gc, int ax, int ay, int az, bool io,
+                                              const T* xc, T* xf) {
+  if constexpr (PAIR) prolong_p1_pair<SET>(gf, gc, ax, ay, az, io, xc, xf);
+  else prolong_p1<SET>(gf, gc, ax, ay, az, io, xc, xf);
+}
+template <int G, bool SET, bool PAIR, class T>
 __device__ __forceinline__ void prolong_body(const uint3 bid, const TransferA<T>& a) {
   constexpr int NPART = G == 8 ? 13 : 4;
   const Geo &gf = a.gf, &gc = a.gc;
@@ -140,18 +247,17 @@ __device__ __forceinline__ void prolong_body(const uint3 bid, const TransferA<T>
   if (ay > gc.ny) return;
   const bool io = a.interior_only != 0;
   if constexpr (G == 1) {
-    prolong_p1<T>(gf, gc, ax, ay, az, io && part < 3, a.in + part * gc.arr, a.out + part * gf.arr);
+    prolong_field<SET, PAIR>(gf, gc, ax, ay, az, io && part < 3, a.in + part * gc.arr, a.out + part * gf.arr);
   } else {
-    if (part == 12) return prolong_p1<T>(gf, gc, ax, ay, az, false, a.in + 24 * gc.arr, a.out + 24 * gf.arr);
+    if (part == 12) return prolong_field<SET, PAIR>(gf, gc, ax, ay, az, false, a.in + 24 * gc.arr, a.out + 24 * gf.arr);
     const int comp = part >> 2;
     const T* xc = a.in + comp * 8 * gc.arr;
     T* xf = a.out + comp * 8 * gf.arr;
-    const auto all = std::make_integer_sequence<int, 16>{};
     switch (part & 3) {
-      case 0: prolong_p2<0>(gf, gc, ax, ay, az, io, xc, xf, all); break;
-      case 1: prolong_p2<1>(gf, gc, ax, ay, az, io, xc, xf, all); break;
-      case 2: prolong_p2<2>(gf, gc, ax, ay, az, io, xc, xf, all); break;
-      default: prolong_p2<3>(gf, gc, ax, ay, az, io, xc, xf, all); break;
+      case 0: prolong_p2_z<0, SET, PAIR>(gf, gc, ax, ay, az, io, xc, xf); break;
+      case 1: prolong_p2_z<1, SET, PAIR>(gf, gc, ax, ay, az, io, xc, xf); break;
+      case 2: prolong_p2_z<2, SET, PAIR>(gf, gc, ax, ay, az, io, xc, xf); break;
+      default: prolong_p2_z<3, SET, PAIR>(gf, gc, ax, ay, az, io, xc, xf); break;
     }
   }
 }
@@ -240,19 +346,19 @@ __device__ __forceinline__ void restrict_body(const uint3 bid, const TransferA<T
   }
 }
 
-template <int G, class T>
+template <int G, bool SET, bool PAIR, class T>
 __global__ void __launch_bounds__(128) k_prolong(const __grid_constant__ TransferA<T> a) {
-  prolong_body<G, T>(blockIdx, a);
+  prolong_body<G, SET, PAIR, T>(blockIdx, a);
 }
 template <int G, class T>
 __global__ void __launch_bounds__(128) k_restrict(const __grid_constant__ TransferA<T> a) {
   restrict_body<G, T>(blockIdx, a);
 }
-template <int G, class T>
+template <int G, bool SET, bool PAIR, class T>
 __global__ void __launch_bounds__(128) kb_prolong(const void* items, int n) {
   uint3 bid, gd;
   const auto& it = batch_item<TransferA<T>>(items, n, bid, gd);
-  prolong_body<G, T>(bid, it.a);
+  prolong_body<G, SET, PAIR, T>(bid, it.a);
 }
 template <int G, class T>
 __global__ void __launch_bounds__(128) kb_restrict(const void* items, int n) {
@@ -271,17 +377,28 @@ void launch(const void* kernel, const void* batched, dim3 grd, const TransferA<T
 }
 inline unsigned plane_blocks(const Geo& gc) { return unsigned(((gc.nx + 1) * (gc.ny + 1) + 127) / 128); }
 
+template <int G, bool SET, bool PAIR, class T>
+void launch_prolong_as(const TransferA<T>& a, cudaStream_t s) {
+  launch<T>(reinterpret_cast<const void*>(k_prolong<G, SET, PAIR, T>),
+            reinterpret_cast<const void*>(kb_prolong<G, SET, PAIR, T>),
+            dim3(plane_blocks(a.gc), 1, (a.gc.nz + 1) * (G == 8 ? 13 : 4)), a, s);
+}
+template <int G, class T>
+void launch_prolong_g(const TransferA<T>& a, bool set, bool pair, cudaStream_t s) {
+  if (set) pair ? launch_prolong_as<G, true, true>(a, s) : launch_prolong_as<G, true, false>(a, s);
+  else pair ? launch_prolong_as<G, false, true>(a, s) : launch_prolong_as<G, false, false>(a, s);
+}
+
 }  // namespace
 
 template <class T>
-void launch_prolong(const Geo& gf, const Geo& gc, bool interior_only, const T* xc, T* xf, cudaStream_t s) {
+void launch_prolong(const Geo& gf, const Geo& gc, bool interior_only, bool set, const T* xc, T* xf, cudaStream_t s) {
   const TransferA<T> a{gf, gc, interior_only ? 1 : 0, xc, xf};
-  if (gf.G == 1)
-    launch<T>(reinterpret_cast<const void*>(k_prolong<1, T>), reinterpret_cast<const void*>(kb_prolong<1, T>),
-              dim3(plane_blocks(gc), 1, (gc.nz + 1) * 4), a, s);
-  else
-    launch<T>(reinterpret_cast<const void*>(k_prolong<8, T>), reinterpret_cast<const void*>(kb_prolong<8, T>),
-              dim3(plane_blocks(gc), 1, (gc.nz + 1) * 13), a, s);
+  // pairs of sites where they are aligned: an even pitch (levels with nx >=
+  // 64 have a multiple of four, the smaller ones nx + 3) and vector
+  const bool pair = gf.sx % 2 == 0 && gf.sy % 2 == 0 && reinterpret_cast<uintptr_t>(xf) % (2 * sizeof(T)) == 0;
+  if (gf.G == 1) launch_prolong_g<1, T>(a, set, pair, s);
+  else launch_prolong_g<8, T>(a, set, pair, s);
 }
 
 template <class T>
@@ -296,7 +413,7 @@ void launch_restrict(const Geo& gf, const Geo& gc, const T* rf, T* rc, cudaStrea
 }
 
 #define HHG_INST(T)                                                                               \
-  template void launch_prolong<T>(const Geo&, const Geo&, bool, const T*, T*, cudaStream_t);      \
+  template void launch_prolong<T>(const Geo&, const Geo&, bool, bool, const T*, T*, cudaStream_t); \
   template void launch_restrict<T>(const Geo&, const Geo&, const T*, T*, cudaStream_t);
 HHG_INST(double)
 HHG_INST(float)

@@ -19,11 +19,11 @@
 // if evaluated in 47-bit arithmetic and then rounded to FP32, the precision
 // the V-cycle takes its right-hand side in.
 //
-// Work layout.  Constant viscosity (k_df_unrolled): a thread owns two sites
+// Work layout.  Constant viscosity but for small levels (k_df_unrolled): a thread owns two sites
 // of a plane and a component and applies each (hi, lo) input it loads to all
 // the component's rows, two sites per paired FP32 (f32x2) instruction; rows
 // are unrolled, with small-integer weights (see there).  Variable viscosity
-// (k_res_df): grid x over the padded (i, j) plane in warps of 4 x 32
+// and small levels (k_res_df): grid x over the padded (i, j) plane in warps of 4 x 32
 // positions, y over groups of kp planes, z over the rows of the operator; on
 // large levels a thread evaluates 4 sites 32 positions apart on 2 planes, on
 // small ones 1 site on 1 plane, in a loop over weights and offsets in the
@@ -619,6 +619,13 @@ constexpr int kDfThreads = 128;
 // per thread (the row loops are latency-bound; more threads hide it), larger
 // ones four sites and two planes
 constexpr int64_t kDfSmallSites = 300000;
+// constant viscosity: levels with at most this many sites run the looped
+// kernel too.  They are bound by the fetch of code that each warp runs once,
+// and the loop is short: defect of P2-P1 with 729 sites 18.5 us looped, 22.6
+// us unrolled; 4913 sites 24.7 and 22.6 us; P1-P1 with 35937 sites 26.7 and
+// 30.8 us; 105633 sites 35.2 and 30.8 us.
+template <int DISC>
+constexpr int64_t kDfLoopSites = DISC == 2 ? 4000 : 60000;
 
 template <int DISC>
 void launch_df_unrolled(const Geo& g, const OpDev& od, const double* x, const double* b, float* xh, float* xl,
@@ -652,7 +659,7 @@ void launch_df(const Geo& g, const OpDev& od, const char* tab, const double* x, 
   const dim3 sgrd(unsigned(std::min<int64_t>((n2 + 255) / 256, 152 * 8)));
   const SplitA sa{reinterpret_cast<const double2*>(x), reinterpret_cast<float2*>(xh), reinterpret_cast<float2*>(xl),
                   n2};
-  const bool small = int64_t(g.nx + 1) * (g.ny + 1) * (g.nz + 1) <= kDfSmallSites;
+  const bool small = VARNU == 0 || int64_t(g.nx + 1) * (g.ny + 1) * (g.nz + 1) <= kDfSmallSites;
   const int v = small ? 1 : 4, kp = small ? 1 : 2;
   // warps of v x 32 positions over the padded plane up to the last site
   const int64_t warps = ((int64_t(g.ny) * g.sx + g.nx + 1) + 32 * v - 1) / (32 * v);
@@ -662,7 +669,7 @@ void launch_df(const Geo& g, const OpDev& od, const char* tab, const double* x, 
     const Tab* dt = static_cast<const Tab*>(g_rec->table(tab, sizeof(Tab)));
     g_rec->add(reinterpret_cast<const void*>(kb_split_df), sgrd, dim3(256), 0, 1, sa);
     g_rec->add(small ? reinterpret_cast<const void*>(kb_res_df<DISC, VARNU, 1>)
-                     : reinterpret_cast<const void*>(kb_res_df<DISC, VARNU, 4>),
+                     : reinterpret_cast<const void*>(kb_res_df<DISC, VARNU, VARNU ? 4 : 1>),
                grd, dim3(kDfThreads), 0, 1, ResDfA<Tab>{g, xh, xl, b, r, od, kp, dt});
     return;
   }
@@ -672,12 +679,15 @@ void launch_df(const Geo& g, const OpDev& od, const char* tab, const double* x, 
   k_split_df<<<sgrd, 256, 0, s>>>(sa.x, sa.hi, sa.lo, n2);
   ++g_launches;
   if (small) k_res_df<DISC, VARNU, 1><<<grd, kDfThreads, 0, s>>>(g, xh, xl, b, r, od, kp, tb);
-  else k_res_df<DISC, VARNU, 4><<<grd, kDfThreads, 0, s>>>(g, xh, xl, b, r, od, kp, tb);
+  else k_res_df<DISC, VARNU, VARNU ? 4 : 1><<<grd, kDfThreads, 0, s>>>(g, xh, xl, b, r, od, kp, tb);
 }
 
 void df_launch(int disc, int varnu, const Geo& g, const OpDev& od, const char* tab, const double* x, const double* b,
                float* xh, float* xl, float* r, cudaStream_t s) {
-  if (disc == 1 && !varnu) launch_df_unrolled<1>(g, od, x, b, xh, xl, r, s);
+  const int64_t sites = int64_t(g.nx + 1) * (g.ny + 1) * (g.nz + 1);
+  if (disc == 1 && !varnu && sites <= kDfLoopSites<1>) launch_df<1, 0>(g, od, tab, x, b, xh, xl, r, s);
+  else if (disc == 2 && !varnu && sites <= kDfLoopSites<2>) launch_df<2, 0>(g, od, tab, x, b, xh, xl, r, s);
+  else if (disc == 1 && !varnu) launch_df_unrolled<1>(g, od, x, b, xh, xl, r, s);
   else if (disc == 1) launch_df<1, 1>(g, od, tab, x, b, xh, xl, r, s);
   else if (!varnu) launch_df_unrolled<2>(g, od, x, b, xh, xl, r, s);
   else launch_df<2, 1>(g, od, tab, x, b, xh, xl, r, s);

@@ -16,11 +16,13 @@ from test_gpu_parity import _abs_row_sums
 pytestmark = pytest.mark.gpu
 
 
+# the second line: levels above the sizes that keep the looped kernel
 @pytest.mark.parametrize("disc,box,L", [("P1P1", (1, 1, 1), 1), ("P1P1", (3, 1, 2), 3), ("P2P1", (1, 1, 1), 1),
-                                        ("P2P1", (3, 1, 1), 2), ("P2P1", (1, 2, 1), 3)])
+                                        ("P2P1", (3, 1, 1), 2), ("P2P1", (1, 2, 1), 3),
+                                        ("P1P1", (3, 1, 2), 5), ("P2P1", (3, 1, 1), 4), ("P2P1", (1, 1, 42), 2)])
 def test_defect_rows(disc, box, L):
     from paper_2010_13513_gb300 import hhg
-    lc = 0 if disc == "P1P1" else 1
+    lc = 0 if disc == "P1P1" or box[2] > 3 else 1
     pb = lib_problem(box, L, disc, lc=lc, solve="mixed")
     lev = oracle_hierarchy(box, L, disc, lc=lc).lv[L]
     assert pb.refinement_residual_kind() == "df32"

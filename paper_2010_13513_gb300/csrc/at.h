@@ -21,6 +21,11 @@ __device__ __forceinline__ const T& ref_at(const T* base, unsigned off) {
   return *reinterpret_cast<const T*>(reinterpret_cast<const char*>(base) + off);
 }
 
+// FP64 P1-P1 arrays may exceed the 4 GB (up to 715 million sites are
+// accepted): its kernels count offsets from the site's plane instead
+template <int DISC, class T>
+constexpr bool kByPlane = DISC == 1 && sizeof(T) == 8;
+
 // byte offsets of a site's nine neighbouring lines (dj, dk) in any group
 // array: kept in registers, so that a term's load is a uniform array base, one
 // of these and an immediate (di)

@@ -2,7 +2,9 @@
 // 3.2) as separate launches, for the levels that do not fit the
 // shared-memory-resident smoother.
 //
-// A thread updates one site of one component.  The row is unrolled from the
+// A thread updates one site of one component (P1-P1: of all three, which share
+// the index arithmetic: a sweep with constant viscosity at 2.1 million sites 55
+// us with a component per thread, 34 us).  The row is unrolled from the
 // generated structure; with a constant viscosity its weights are immediates
 // (those of h = 1, the sum scaled by h), with a variable one the group's row
 // is a kernel parameter.  Offsets are formed from the array stride and the
@@ -22,7 +24,9 @@
 // edge phase reads the whole velocity, 217 MB in FP32).  Measured, one forward
 // sweep of P2-P1: FP32 level 5 / 6 / 7 28.8 / 59.5 / 543 us before, 23.8 / 59.9
 // / 439 us now (level 7 with the shared edge sums); FP64 level 4 44 us before,
-// 31 us.  Programmatic launches pay at every size: limited to one wave of
+// 31 us; P1-P1 at 2.1 / 17 million sites, constant viscosity, 47.7 / 378 us
+// before, 34.4 / 367 us, variable viscosity 64.9 / 443 us before, 53.9 / 426 us.
+// Programmatic launches pay at every size: limited to one wave of
 // blocks, the level-6 sweep takes 78 us.
 #include <cuda_runtime.h>
 
@@ -77,8 +81,8 @@ __device__ __forceinline__ void pdl_wait() { cudaGridDependencySynchronize(); }
 __device__ __forceinline__ void pdl_trigger() { cudaTriggerProgrammaticLaunchCompletion(); }
 
 // grid: x over the sites of the (i, j) plane (a vertex colour: quads of four
-// sites of a row), y = component, z = plane
-template <int DISC, int VARNU, int GRP, int SEL, class T, int NW>
+// sites of a row), y = component (NC = 3: a thread takes all three), z = plane
+template <int DISC, int VARNU, int GRP, int SEL, int NC, class T, int NW>
 __device__ __forceinline__ void gs_site(const uint3 bid, const GsA<T, NW>& a) {
   using S = gen::S<DISC, VARNU, OP_A>;
   constexpr gen::RowS rw = S::rows[GRP];
@@ -92,25 +96,32 @@ __device__ __forceinline__ void gs_site(const uint3 bid, const GsA<T, NW>& a) {
   int i = q - jj * w;
   if (GRP == 0) i = 4 * i + ((a.colour - j - k) & 3);
   if (j >= g.ny || i >= g.nx || (!ox && i == 0)) return;
-  const Lines<T> at(g, unsigned(i + 1) + unsigned(j + 1) * unsigned(g.sx) + unsigned(k + 1) * unsigned(g.sy));
-  const int64_t base = int64_t(a.comp + int(bid.y)) * G * g.arr;
-  T* u = a.u + base;
-  T r = ld_at(a.rhs + (SEL == kVertexTerms ? int64_t(bid.y) * g.arr : base + GRP * g.arr), at.site());
-  const T s = row_sum<S, GRP, SEL>(g, u, at, a.w, std::make_integer_sequence<int, rw.n1 - 1>{});
-  if (VARNU && SEL != kVertexTerms) r *= T(g.eisc[k]);
-  ref_at(u + GRP * g.arr, at.site()) = (r - (VARNU ? s : T(g.h) * s)) * a.inv_diag;
+  const int kb = kByPlane<DISC, T> ? k : 0;          // the plane that offsets count from
+  const Lines<T> at(g, unsigned(i + 1) + unsigned(j + 1) * unsigned(g.sx) + unsigned(k - kb + 1) * unsigned(g.sy));
+  T v[NC];
+#pragma unroll
+  for (int c = 0; c < NC; ++c) {
+    const int64_t base = int64_t(a.comp + int(bid.y) + c) * G * g.arr;
+    T r = ld_at(a.rhs + kb * g.sy + (SEL == kVertexTerms ? int64_t(bid.y) * g.arr : base + GRP * g.arr), at.site());
+    const T s = row_sum<S, GRP, SEL>(g, a.u + base + kb * g.sy, at, a.w, std::make_integer_sequence<int, rw.n1 - 1>{});
+    if (VARNU && SEL != kVertexTerms) r *= T(g.eisc[k]);
+    v[c] = (r - (VARNU ? s : T(g.h) * s)) * a.inv_diag;
+  }
+#pragma unroll
+  for (int c = 0; c < NC; ++c)
+    ref_at(a.u + int64_t(a.comp + int(bid.y) + c) * G * g.arr + kb * g.sy + GRP * g.arr, at.site()) = v[c];
 }
-template <int DISC, int VARNU, int GRP, int SEL, class T>
+template <int DISC, int VARNU, int GRP, int SEL, int NC, class T>
 __global__ void __launch_bounds__(256) k_gs(const __grid_constant__ GsA<T, row_nw<DISC, VARNU, GRP>()> a) {
   pdl_wait();
-  gs_site<DISC, VARNU, GRP, SEL>(blockIdx, a);
+  gs_site<DISC, VARNU, GRP, SEL, NC>(blockIdx, a);
   pdl_trigger();
 }
-template <int DISC, int VARNU, int GRP, int SEL, class T>
+template <int DISC, int VARNU, int GRP, int SEL, int NC, class T>
 __global__ void __launch_bounds__(256) kb_gs(const void* items, int n) {
   uint3 bid, gd;
   const auto& it = batch_item<GsA<T, row_nw<DISC, VARNU, GRP>()>>(items, n, bid, gd);
-  gs_site<DISC, VARNU, GRP, SEL>(bid, it.a);
+  gs_site<DISC, VARNU, GRP, SEL, NC>(bid, it.a);
 }
 
 // t = rhs - (edge terms of the vertex row) at the interior vertices; block: 32
@@ -175,9 +186,15 @@ void launch_phase(const Geo& g, const GsRows<T>& rows, int colour, T* u, const T
   // j from 1 (or 0, odd groups) to ny - 1, k the same
   const int w = GRP == 0 ? (g.nx + 3) / 4 : g.nx, nj = g.ny - (oy ? 0 : 1), nk = g.nz - (oz ? 0 : 1);
   if (nj < 1 || nk < 1) return;
-  launch(reinterpret_cast<const void*>(k_gs<DISC, VARNU, GRP, SEL, T>),
-         reinterpret_cast<const void*>(kb_gs<DISC, VARNU, GRP, SEL, T>),
-         dim3(unsigned((w * nj + threads - 1) / threads), ncomp, nk), threads, true, a, s);
+  // P1-P1: a thread takes the three components of a site
+  constexpr int NC = DISC == 1 ? 3 : 1;
+  const dim3 grd(unsigned((w * nj + threads - 1) / threads), ncomp, nk);
+  if (NC == 3 && ncomp == 3)
+    return launch(reinterpret_cast<const void*>(k_gs<DISC, VARNU, GRP, SEL, NC, T>),
+                  reinterpret_cast<const void*>(kb_gs<DISC, VARNU, GRP, SEL, NC, T>), dim3(grd.x, 1, nk), threads, true,
+                  a, s);
+  launch(reinterpret_cast<const void*>(k_gs<DISC, VARNU, GRP, SEL, 1, T>),
+         reinterpret_cast<const void*>(kb_gs<DISC, VARNU, GRP, SEL, 1, T>), grd, threads, true, a, s);
 }
 
 template <int VARNU, class T>

@@ -218,11 +218,13 @@ __device__ __forceinline__ void pressure_row(const FullA<T>& a, int i, int j, in
 // grid x over the sites of the (i, j) plane (flat), y = plane, z = part: the
 // components (P1: all at once), then the pressure
 template <int DISC, int VARNU, int MODE, class T, class Tab>
-__device__ __forceinline__ void full_body(const uint3 bid, const FullA<T>& a, const Tab& tab) {
-  const Geo& g = a.g;
+__device__ __forceinline__ void full_body(const uint3 bid, const FullA<T>& full, const Tab& tab) {
+  const Geo& g = full.g;
   const int w = g.nx + 1, q = bid.x * blockDim.x + threadIdx.x, j = q / w, i = q - j * w, k = bid.y;
   if (j > g.ny) return;
-  const Lines<T> at(g, unsigned(i + 1) + unsigned(j + 1) * unsigned(g.sx) + unsigned(k + 1) * unsigned(g.sy));
+  const int kb = kByPlane<DISC, T> ? k : 0;          // the plane that offsets count from
+  const FullA<T> a{g, full.x + kb * g.sy, full.b + kb * g.sy, full.y + kb * g.sy, full.tabs};
+  const Lines<T> at(g, unsigned(i + 1) + unsigned(j + 1) * unsigned(g.sx) + unsigned(k - kb + 1) * unsigned(g.sy));
   using SPT = gen::SP<DISC, VARNU, OP_FULL>;
   if constexpr (DISC == 1) {
     if (bid.z == 0)

@@ -22,7 +22,7 @@ LIB = os.path.join(HERE, "libhhg.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 # (source, object, extra flags): stream.cu is compiled once per precision
 SOURCES = [("kernels.cu", "kernels", []), ("transfer.cu", "transfer", []),
-           ("uzrows.cu", "uzrows", []), ("rows.cu", "rows", []), ("march.cu", "march", []),
+           ("uzrows.cu", "uzrows", []), ("rows.cu", "rows", []), ("march.cu", "march", []), ("quad.cu", "quad", []),
            ("gs.cu", "gs", []), ("stream.cu", "stream64", ["-DHHG_STREAM_ONLY=64"]),
            ("stream.cu", "stream32", ["-DHHG_STREAM_ONLY=32"]),
            ("stream.cu", "stream32v2", ["-DHHG_STREAM_ONLY=32", "-DHHG_STREAM_V=2"]),

@@ -21,7 +21,8 @@
 // Measured, both rows and the update of one iteration against the three
 // launches before: P2-P1 FP32 level 5 / 6 / 7: 24 / 49 / 236 us before, 12 / 31
 // / 190 us now; P1-P1 with variable viscosity, 48 tetrahedra, level 6: 81 us
-// before, 73 us (device times).
+// before, 73 us (device times).  Larger P1-P1 levels in FP32 take four aligned
+// sites per thread (quad.cu).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -31,6 +32,7 @@
 #include "at.h"
 #include "batch.h"
 #include "kernels.h"
+#include "quad.h"
 #include "structure.inc"
 #include "uzrows.h"
 
@@ -95,9 +97,9 @@ __device__ __forceinline__ void bt_groups(const BtA<T, NW>& a, const T (&p)[27],
 
 // grid x over the positions of the padded (i, j) plane, y = plane, z = component
 template <int DISC, int VARNU, class T, int NW>
-__device__ __forceinline__ void bt_body(const uint3 bid, const BtA<T, NW>& a) {
+__device__ __forceinline__ void bt_body(const uint3 bid, const BtA<T, NW>& full) {
   constexpr int G = DISC == 2 ? 8 : 1;
-  const Geo& g = a.g;
+  const Geo& g = full.g;
   const int q = bid.x * blockDim.x + threadIdx.x, j = q / g.sx, i = q - j * g.sx, k = bid.y;
   if (i >= g.nx || j >= g.ny) return;
   // groups with an interior DoF in the cell (order of kGroupOff)
@@ -105,7 +107,11 @@ __device__ __forceinline__ void bt_body(const uint3 bid, const BtA<T, NW>& a) {
 #pragma unroll
   for (int gg = 0; gg < G; ++gg)
     if ((i > 0 || (0xB2 >> gg & 1)) && (j > 0 || (0xD4 >> gg & 1)) && (k > 0 || (0xE8 >> gg & 1))) in |= 1 << gg;
-  const Lines<T> at(g, unsigned(i + 1) + unsigned(j + 1) * unsigned(g.sx) + unsigned(k + 1) * unsigned(g.sy));
+  const int kb = kByPlane<DISC, T> ? k : 0;          // the plane that offsets count from
+  const Lines<T> at(g, unsigned(i + 1) + unsigned(j + 1) * unsigned(g.sx) + unsigned(k - kb + 1) * unsigned(g.sy));
+  BtA<T, NW> a = full;
+  a.x += kb * g.sy; a.y += kb * g.sy;
+  if (a.b) a.b += kb * g.sy;
   T p[27];
   bt_load<gen::S<DISC, VARNU, OP_BT>>(a.x + 3 * G * g.arr, at, p, std::make_integer_sequence<int, 27>{});
   const auto groups = std::make_integer_sequence<int, G>{};
@@ -172,11 +178,12 @@ __device__ __forceinline__ void press_body(const uint3 bid, const PressA<T, NW>&
 #pragma unroll 1
   for (int k = bid.y * a.kp; k < k1; ++k) {
     const int64_t idx = int64_t(i + 1) + int64_t(j + 1) * g.sx + int64_t(k + 1) * g.sy;
-    const Lines<T> at(g, unsigned(idx));
+    const int kb = kByPlane<DISC, T> ? k : 0;        // the plane that offsets count from
+    const Lines<T> at(g, unsigned(idx - kb * g.sy));
     const T bv = __ldg(a.b + 3 * G * g.arr + idx);
     const T ml = T(a.s * __ldg(a.inv_ml + idx));
     const T* x = a.x + idx;
-    T v = press_sum<S, rw.t0>(g, a.x, at, a.w, std::make_integer_sequence<int, rw.n0>{});
+    T v = press_sum<S, rw.t0>(g, a.x + kb * g.sy, at, a.w, std::make_integer_sequence<int, rw.n0>{});
     if (!VARNU) v *= T(g.h) * T(g.h);
     if constexpr (rw.n2 > 0) {
       using SPT = gen::SP<DISC, VARNU, OP_BC>;
@@ -186,7 +193,7 @@ __device__ __forceinline__ void press_body(const uint3 bid, const PressA<T, NW>&
                         9 * (k == 0 ? 0 : k == g.nz ? 2 : 1);
         c = press_c<SPT>(g, x + 3 * G * g.arr, a.tabs->wc + cls * SPT::NCB, std::make_integer_sequence<int, SPT::NCB>{});
       } else {
-        c = press_sum<S, rw.t0 + rw.n0>(g, a.x, at, a.w, std::make_integer_sequence<int, rw.n2>{});
+        c = press_sum<S, rw.t0 + rw.n0>(g, a.x + kb * g.sy, at, a.w, std::make_integer_sequence<int, rw.n2>{});
         if (!VARNU) c *= T(g.h) * T(g.h) * T(g.h);
       }
       v += VARNU ? T(g.eisc[k]) * c : c;
@@ -197,11 +204,11 @@ __device__ __forceinline__ void press_body(const uint3 bid, const PressA<T, NW>&
   }
 }
 template <int DISC, int VARNU, class T>
-__global__ void __launch_bounds__(256, DISC == 2 ? 2 : 3) k_pressure(const __grid_constant__ PressA<T, bc_nw<DISC, VARNU>()> a) {
+__global__ void __launch_bounds__(256, DISC == 2 || sizeof(T) == 8 ? 2 : 3) k_pressure(const __grid_constant__ PressA<T, bc_nw<DISC, VARNU>()> a) {
   press_body<DISC, VARNU>(blockIdx, a);
 }
 template <int DISC, int VARNU, class T>
-__global__ void __launch_bounds__(256, DISC == 2 ? 2 : 3) kb_pressure(const void* items, int n) {
+__global__ void __launch_bounds__(256, DISC == 2 || sizeof(T) == 8 ? 2 : 3) kb_pressure(const void* items, int n) {
   uint3 bid, gd;
   const auto& it = batch_item<PressA<T, bc_nw<DISC, VARNU>()>>(items, n, bid, gd);
   press_body<DISC, VARNU>(bid, it.a);
@@ -236,6 +243,9 @@ void launch(const void* kernel, const void* batched, dim3 grd, int threads, cons
 template <int DISC, int VARNU, class T>
 void launch_bt(const Geo& g, int mode, const T* w, const T* x, const T* b, T* y, cudaStream_t s) {
   constexpr int NW = bt_nw<DISC, VARNU>();
+  if constexpr (DISC == 1 && sizeof(T) == 4) {
+    if (quad_bt(VARNU, g, w, x, mode == MODE_RES ? b : nullptr, y, s)) return;
+  }
   BtA<T, NW> a{g, x, mode == MODE_RES ? b : nullptr, y, {}};
   if (NW > 1) std::copy(w, w + NW, a.w);
   const dim3 grd((g.ny * g.sx + 127) / 128, g.nz, DISC == 2 ? 3 : 1);
@@ -252,8 +262,11 @@ void launch_pressure(const Geo& g, const T* w, const ResTabs<T>* tabs, T* x, con
   PressA<T, NW> a{g, x, b, DISC == 2 ? p : tmp + 3 * G * g.arr, inv_mlhat, sc, tabs, kp, {}};
   if (NW > 1) std::copy(w, w + NW, a.w);
   const dim3 grd((g.ny * g.sx + g.nx + 256) / 256, (g.nz + kp) / kp);
-  launch(reinterpret_cast<const void*>(k_pressure<DISC, VARNU, T>),
-         reinterpret_cast<const void*>(kb_pressure<DISC, VARNU, T>), grd, 256, a, s);
+  bool done = false;
+  if constexpr (DISC == 1 && sizeof(T) == 4) done = quad_pressure(VARNU, g, w, tabs, x, b, a.p, inv_mlhat, sc, s);
+  if (!done)
+    launch(reinterpret_cast<const void*>(k_pressure<DISC, VARNU, T>),
+           reinterpret_cast<const void*>(kb_pressure<DISC, VARNU, T>), grd, 256, a, s);
   if (DISC == 1)
     launch(reinterpret_cast<const void*>(k_copy<T>), reinterpret_cast<const void*>(kb_copy<T>),
            dim3(unsigned(std::min<int64_t>((g.arr + 255) / 256, 152 * 8))), 256, CopyA<T>{a.p, p, g.arr}, s);

@@ -54,6 +54,12 @@ template <class T>
 void launch_reduce(int mode, const T* a, const T* b, const double* w, int64_t n, double* partials, int max_blocks,
                    double* out, cudaStream_t s);
 
+// sums of squares of the first n_u and the next n_p elements of x into out[0],
+// out[1]; partials: 2 max_blocks values (not recorded by a batch)
+template <class T>
+void launch_norms(const T* x, int64_t n_u, int64_t n_p, double* partials, int max_blocks, double* out,
+                  cudaStream_t s);
+
 // p -= (*sum) * scale on all pressure nodes
 template <class T>
 void launch_sub_scalar_p(const Geo& g, T* p, const double* sum, double scale, cudaStream_t s);

@@ -474,7 +474,7 @@ extern "C" int hhg_problem_create(const hhg_mesh* mesh, const hhg_problem_desc* 
   }
   pb->o_Z = off; off += align256(size_t(pb->ncoarse) * pb->ncoarse * 8);
   pb->o_idx = off; off += align256(size_t(pb->ncoarse) * 8);
-  pb->o_part = off; off += align256(size_t(pb->max_blocks) * 8);
+  pb->o_part = off; off += align256(2 * size_t(pb->max_blocks) * 8);
   pb->o_scal = off; off += align256(64 * 8);
   if (desc->nn_hidden > 0) {
     if (desc->nn_samples < 2 || desc->nn_batch < 1) return fail(HHG_EINVAL, "nn_samples >= 2 and nn_batch >= 1 needed");
@@ -889,12 +889,10 @@ int norms_of(hhg_problem* pb, Level& lv, int prec, const void* r, double* out2) 
   const int64_t po = p_offset(lv);
   if (prec == HHG_FP64) {
     const double* rr = static_cast<const double*>(r);
-    launch_reduce<double>(RED_SQ, rr, nullptr, nullptr, po, pb->partials, pb->max_blocks, pb->scal + 1, pb->stream);
-    launch_reduce<double>(RED_SQ, rr + po, nullptr, nullptr, lv.g.arr, pb->partials, pb->max_blocks, pb->scal + 2, pb->stream);
+    launch_norms<double>(rr, po, lv.g.arr, pb->partials, pb->max_blocks, pb->scal + 1, pb->stream);
   } else {
     const float* rr = static_cast<const float*>(r);
-    launch_reduce<float>(RED_SQ, rr, nullptr, nullptr, po, pb->partials, pb->max_blocks, pb->scal + 1, pb->stream);
-    launch_reduce<float>(RED_SQ, rr + po, nullptr, nullptr, lv.g.arr, pb->partials, pb->max_blocks, pb->scal + 2, pb->stream);
+    launch_norms<float>(rr, po, lv.g.arr, pb->partials, pb->max_blocks, pb->scal + 1, pb->stream);
   }
   HHG_CHECK_LAUNCH();
   double h[2];

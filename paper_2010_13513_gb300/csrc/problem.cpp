@@ -710,9 +710,12 @@ int set_resident(hhg_problem* pb, Level& lv, int prec, int ctas, int threads = k
 // most 8192 lattice sites each, else none (per-phase kernels)
 int default_resident(hhg_problem* pb, Level& lv, int prec) {
   const int64_t plane = int64_t(lv.g.nx + 1) * (lv.g.ny + 1), nzp = lv.g.nz + 1;
-  for (int C : {1, 2, 4, 8})
-    if (plane * ((nzp + C - 1) / C) <= 8192 && resident_feasible(pb->desc.disc, pb->desc.nu_a != 0.0 ? 1 : 0, prec, lv.g, C))
-      return set_resident(pb, lv, prec, C);
+  const int disc = pb->desc.disc, varnu = pb->desc.nu_a != 0.0 ? 1 : 0;
+  for (bool compact : {false, true})               // the compact layout only where no other fits
+    for (int C : {1, 2, 4, 8})
+      if (plane * ((nzp + C - 1) / C) <= 8192 && resident_compact(disc, varnu, lv.g, C, prec) == compact &&
+          resident_feasible(disc, varnu, prec, lv.g, C))
+        return set_resident(pb, lv, prec, C);
   return set_resident(pb, lv, prec, 0);
 }
 

@@ -77,11 +77,13 @@ struct ResDims {
   int slab, rhs, np, n, n4, ncb, nw;
 };
 __host__ __device__ inline int ncb_of(int disc, int varnu) { return disc == 2 ? 0 : varnu ? 15 : 7; }
-__host__ __device__ inline ResDims res_dims(int disc, int varnu, const Geo& g, int C) {
+// compact: the layout of levels that do not fit the other one.  No odd stride,
+// no tables of the pressure slots, no edge sums, one thread per pressure row.
+__host__ __device__ inline ResDims res_dims(int disc, int varnu, const Geo& g, int C, bool compact) {
   ResDims d;
   d.G = disc == 2 ? 8 : 1;
   d.na = 3 * d.G + 1;
-  d.pad = d.na | 1;
+  d.pad = compact ? d.na : d.na | 1;
   d.planes = d.cells = 0;
   for (int c = 0; c < C; ++c) {
     const int kb = int(int64_t(c) * (g.nz + 1) / C), ke = int(int64_t(c + 1) * (g.nz + 1) / C);
@@ -96,7 +98,8 @@ __host__ __device__ inline ResDims res_dims(int disc, int varnu, const Geo& g, i
   d.n4 = d.cells * g.ny * ((g.nx + 3) / 4);                  // vertex slots: four sites of a row
   // right-hand sides of the owned planes (P2: and the edge sums of the
   // vertices), later the partial sums of the pressure row
-  const int rhs = (3 * d.G + (disc == 2 ? 3 : 0)) * d.cells * sy, parts = (disc == 2 ? 3 : 4) * d.np;
+  const int rhs = (3 * d.G + (disc == 2 && !compact ? 3 : 0)) * d.cells * sy;
+  const int parts = (compact ? 1 : disc == 2 ? 3 : 4) * d.np;
   d.rhs = rhs > parts ? rhs : parts;
   d.ncb = ncb_of(disc, varnu);
   d.nw = varnu ? kResMaxTerms : 0;
@@ -172,25 +175,25 @@ __device__ __forceinline__ void with_comp(int comp, F&& f) {
 
 // the smoother of one cluster (the kernel below, or one work item of a
 // merged launch over several problems' clusters)
-template <int DISC, int VARNU, class T>
+template <int DISC, int VARNU, bool COMPACT, class T>
 __device__ __forceinline__ void uzawa_resident_body(const Geo& g, T* xg, const T* __restrict__ b,
                                                     const double* __restrict__ inv_ml, const SmallArgs& a,
                                                     const ResTabs<T>* __restrict__ tabs) {
   using SA = gen::S<DISC, VARNU, OP_A>;
   using SBT = gen::S<DISC, VARNU, OP_BT>;
   using SBC = gen::S<DISC, VARNU, OP_BC>;
-  constexpr int G = DISC == 2 ? 8 : 1, NA = 3 * G + 1, PAD = NA | 1, NPH = 4 + (G - 1);
+  constexpr int G = DISC == 2 ? 8 : 1, NA = 3 * G + 1, PAD = COMPACT ? NA : NA | 1, NPH = 4 + (G - 1);
   constexpr int WBT = SA::N / 3, WBC = WBT + SBT::N;
   static_assert(WBC + SBC::N <= kResMaxTerms, "weights fit the table");
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ T sdiag[8];
   cg::cluster_group cluster = cg::this_cluster();
   const int C = int(cluster.num_blocks()), c = int(cluster.block_rank());
-  const ResDims dm = res_dims(DISC, VARNU, g, C);
+  const ResDims dm = res_dims(DISC, VARNU, g, C, COMPACT);
   T* xs = reinterpret_cast<T*>(smem_raw);
   T* ts = xs + dm.slab;
-  T* mls = ts + dm.rhs;
-  T* wc = mls + dm.np;
+  T* mls = ts + dm.rhs;                                      // omega M_L^{-1} of the pressure slots
+  T* wc = mls + (COMPACT ? 0 : dm.np);
   T* sw = wc + 27 * dm.ncb;
   int* info = reinterpret_cast<int*>(sw + dm.nw);            // velocity slots: site, groups with an interior DoF
   int* cinfo = info + dm.n;                                  // vertex slots: site of the quad, colour shift
@@ -236,14 +239,20 @@ __device__ __forceinline__ void uzawa_resident_body(const Geo& g, T* xg, const T
     cinfo[s] = (kl < nc && j > 0 && k > 0) ? ((kl + 1) * sy + (j + 1) * sx + 1 + 4 * i4) | ((j + k) & 3) << 16 | i4 << 18
                                            : -1;
   }
-  for (int s = tid; s < dm.np; s += nthr) {
+  auto pslot = [&](int s) {
     const int row = qdiv(s, msx), i = s - row * sx, kl = row / (ny + 1), j = row - kl * (ny + 1), k = kb + kl;
     const int cls = (i == 0 ? 0 : i == nx ? 2 : 1) + 3 * (j == 0 ? 0 : j == ny ? 2 : 1) +
                     9 * (k == 0 ? 0 : k == g.nz ? 2 : 1);
-    const bool in = kl < nk && i <= nx;
-    pinfo[s] = in ? ((kl + 1) * sy + (j + 1) * sx + i + 1) | cls << 16 : -1;
-    mls[s] = in ? T(a.inv_omega_inv * inv_ml[int64_t(k + 1) * sy + (j + 1) * sx + i + 1]) : T(0);
-  }
+    return kl < nk && i <= nx ? ((kl + 1) * sy + (j + 1) * sx + i + 1) | cls << 16 : -1;
+  };
+  // omega M_L^{-1} at a slab site
+  auto site_ml = [&](int il) { return T(a.inv_omega_inv * inv_ml[int64_t(kb) * sy + il]); };
+  if (!COMPACT)
+    for (int s = tid; s < dm.np; s += nthr) {
+      const int f = pslot(s);
+      pinfo[s] = f;
+      mls[s] = f < 0 ? T(0) : site_ml(f & 0xffff);
+    }
   for (int r = tid; r < (nk + 2) * sy; r += nthr) {          // owned planes and the halo planes kb-1, ke
     T v[NA];
 #pragma unroll
@@ -254,7 +263,8 @@ __device__ __forceinline__ void uzawa_resident_body(const Geo& g, T* xg, const T
   bar();                                           // every CTA runs before any remote store
 
   const T hs = T(g.h), hs2 = T(g.h) * T(g.h);
-  const int n = dm.n, n3 = 3 * n, m3 = 3 * dm.n4, np = dm.np, nu = (DISC == 2 ? 3 : 4) * np;
+  const int n = dm.n, n3 = 3 * n, m3 = 3 * dm.n4, np = dm.np, nu = (COMPACT ? 1 : DISC == 2 ? 3 : 4) * np;
+  constexpr bool kSums = DISC == 2 && !COMPACT;    // the vertex colours share the sums of their edge terms
   for (int it = 0; it < a.iterations; ++it) {
     // ---- velocity step: tmp_u = b_u - B^T p at the interior sites of every group
     for (int q = tid; q < n3; q += nthr) {
@@ -287,7 +297,7 @@ __device__ __forceinline__ void uzawa_resident_body(const Geo& g, T* xg, const T
           if (ph < 4) {
             constexpr gen::RowS rw = SA::rows[0];
             constexpr auto terms = std::make_integer_sequence<int, rw.n1 - 1>{};   // the diagonal is the first term
-            if constexpr (DISC == 2) {
+            if constexpr (kSums) {
               if (!sums) {
                 for (int q = tid; q < n3; q += nthr) {
                   const int comp = (q >= n) + (q >= 2 * n), f = info[q - comp * n], il = f & 0xffff;
@@ -307,10 +317,10 @@ __device__ __forceinline__ void uzawa_resident_body(const Geo& g, T* xg, const T
               const int di = (ph - (f >> 16)) & 3, i = 4 * (f >> 18) + di;
               if (f < 0 || i < 1 || i >= nx) continue;
               const int il = (f & 0xffff) + di, kl = qdiv(il, msy) - 1;
-              const T s = row_sum<SA, rw.t0 + 1, 0, VARNU, kVertex, -1, G, PAD>(xs + il * PAD + comp * G, oj, ok, sw,
-                                                                                terms);
-              T t = ts[(DISC == 2 ? 24 + comp : comp) * as + il - t0];
-              if (DISC == 1 && VARNU) t *= T(g.eisc[kb + kl]);
+              const T s = row_sum<SA, rw.t0 + 1, 0, VARNU, kSums ? kVertex : kAll, -1, G, PAD>(
+                  xs + il * PAD + comp * G, oj, ok, sw, terms);
+              T t = ts[(kSums ? 24 + comp : comp * G) * as + il - t0];
+              if (!kSums && VARNU) t *= T(g.eisc[kb + kl]);
               store(il * PAD + comp * G, kl, (t - (VARNU ? s : hs * s)) * sdiag[0]);
             }
           } else if constexpr (DISC == 2) {
@@ -338,9 +348,8 @@ __device__ __forceinline__ void uzawa_resident_body(const Geo& g, T* xg, const T
     // ---- pressure step: tmp_p = g - (B u - C p) at every pressure site, its
     // parts (per velocity component, C) by different threads, then
     // p -= omega M_L^{-1} tmp_p
-    for (int q = tid; q < nu; q += nthr) {
-      const int part = (q >= np) + (q >= 2 * np) + (q >= 3 * np), f = pinfo[q - part * np], il = f & 0xffff;
-      if (f < 0) continue;
+    auto press_part = [&](int part, int f) {
+      const int il = f & 0xffff;
       const T* p = xs + il * PAD;
       T s = T(0);
       if (DISC == 1 && part == 3) {
@@ -358,17 +367,31 @@ __device__ __forceinline__ void uzawa_resident_body(const Geo& g, T* xg, const T
         });
         if (!VARNU) s *= hs2;
       }
-      ts[q] = s;
+      return s;
+    };
+    for (int q = tid; q < nu; q += nthr) {
+      const int part = COMPACT ? 0 : (q >= np) + (q >= 2 * np) + (q >= 3 * np);
+      const int f = COMPACT ? pslot(q) : pinfo[q - part * np];
+      if (f < 0) continue;
+      if (COMPACT) {
+        T v = T(0);
+#pragma unroll 1
+        for (int c_ = 0; c_ < (DISC == 2 ? 3 : 4); ++c_) v += press_part(c_, f);
+        ts[q] = v;
+      } else {
+        ts[q] = press_part(part, f);
+      }
     }
     if (DISC == 1) bar();                          // the neighbours have read the old halo pressures
     else __syncthreads();
     for (int s = tid; s < np; s += nthr) {
-      const int f = pinfo[s], il = f & 0xffff;
+      const int f = COMPACT ? pslot(s) : pinfo[s], il = f & 0xffff;
       if (f < 0) continue;
-      T v = ts[s] + ts[s + np] + ts[s + 2 * np];
-      if (DISC == 1) v += ts[s + 3 * np];
+      T v = ts[s];
+      if (!COMPACT) v = v + ts[s + np] + ts[s + 2 * np];
+      if (DISC == 1 && !COMPACT) v += ts[s + 3 * np];
       const T r = __ldg(b + 3 * G * g.arr + int64_t(kb) * sy + il) - v;
-      store(il * PAD + 3 * G, qdiv(il, msy) - 1, xs[il * PAD + 3 * G] - mls[s] * r);
+      store(il * PAD + 3 * G, qdiv(il, msy) - 1, xs[il * PAD + 3 * G] - (COMPACT ? site_ml(il) : mls[s]) * r);
     }
     bar();
   }
@@ -382,29 +405,30 @@ __device__ __forceinline__ void uzawa_resident_body(const Geo& g, T* xg, const T
 template <class T>
 struct ResA { Geo g; T* xg; const T* b; const double* inv_ml; SmallArgs a; const ResTabs<T>* tabs; };
 
-template <int DISC, int VARNU, class T>
+template <int DISC, int VARNU, bool COMPACT, class T>
 __global__ void __launch_bounds__(kResidentThreads, 1) k_uzawa_resident(const __grid_constant__ ResA<T> r) {
-  uzawa_resident_body<DISC, VARNU, T>(r.g, r.xg, r.b, r.inv_ml, r.a, r.tabs);
+  uzawa_resident_body<DISC, VARNU, COMPACT, T>(r.g, r.xg, r.b, r.inv_ml, r.a, r.tabs);
 }
 // every cluster of the merged grid belongs to one item (items start at
 // multiples of the cluster size)
-template <int DISC, int VARNU, class T>
+template <int DISC, int VARNU, bool COMPACT, class T>
 __global__ void __launch_bounds__(kResidentThreads, 1) kb_uzawa_resident(const void* items, int n) {
   uint3 bid, gd;
   const auto& it = batch_item<ResA<T>>(items, n, bid, gd);
   const ResA<T>& r = it.a;
-  uzawa_resident_body<DISC, VARNU, T>(r.g, r.xg, r.b, r.inv_ml, r.a, r.tabs);
+  uzawa_resident_body<DISC, VARNU, COMPACT, T>(r.g, r.xg, r.b, r.inv_ml, r.a, r.tabs);
 }
 
 template <class T> constexpr int prec_of() { return sizeof(T) == 8 ? HHG_FP64 : HHG_FP32; }
 
 template <class T>
-const void* kernel_of(int disc, int varnu, bool batched) {
-#define HHG_K(D, V)                                                                          \
-  if (disc == D && varnu == V)                                                               \
-    return batched ? reinterpret_cast<const void*>(kb_uzawa_resident<D, V, T>)               \
-                   : reinterpret_cast<const void*>(k_uzawa_resident<D, V, T>);
-  HHG_K(1, 0) HHG_K(1, 1) HHG_K(2, 0) HHG_K(2, 1)
+const void* kernel_of(int disc, int varnu, bool compact, bool batched) {
+#define HHG_K(D, V, M)                                                                       \
+  if (disc == D && varnu == V && compact == M)                                               \
+    return batched ? reinterpret_cast<const void*>(kb_uzawa_resident<D, V, M, T>)            \
+                   : reinterpret_cast<const void*>(k_uzawa_resident<D, V, M, T>);
+  HHG_K(1, 0, false) HHG_K(1, 1, false) HHG_K(2, 0, false) HHG_K(2, 1, false)
+  HHG_K(1, 0, true) HHG_K(1, 1, true) HHG_K(2, 0, true) HHG_K(2, 1, true)
 #undef HHG_K
   return nullptr;
 }
@@ -426,10 +450,20 @@ void fill_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr, int C, int 
 
 }  // namespace
 
-size_t resident_smem(int disc, int varnu, const Geo& g, int ctas, int prec) {
+namespace {
+size_t layout_smem(int disc, int varnu, const Geo& g, int ctas, int prec, bool compact) {
   const size_t es = prec == HHG_FP64 ? 8 : 4;
-  const ResDims d = res_dims(disc, varnu, g, ctas);
-  return (size_t(d.slab) + d.rhs + d.np + 27 * d.ncb + d.nw) * es + (size_t(d.n) + d.n4 + d.np) * 4;
+  const ResDims d = res_dims(disc, varnu, g, ctas, compact);
+  const size_t np = compact ? 0 : d.np;
+  return (size_t(d.slab) + d.rhs + np + 27 * d.ncb + d.nw) * es + (size_t(d.n) + d.n4 + np) * 4;
+}
+}  // namespace
+
+bool resident_compact(int disc, int varnu, const Geo& g, int ctas, int prec) {
+  return layout_smem(disc, varnu, g, ctas, prec, false) > kResidentSmemMax;
+}
+size_t resident_smem(int disc, int varnu, const Geo& g, int ctas, int prec) {
+  return layout_smem(disc, varnu, g, ctas, prec, resident_compact(disc, varnu, g, ctas, prec));
 }
 
 bool resident_feasible(int disc, int varnu, int prec, const Geo& g, int ctas) {
@@ -439,7 +473,9 @@ bool resident_feasible(int disc, int varnu, int prec, const Geo& g, int ctas) {
   if (planes * g.sy >= 65536 || g.nx >= 4 * 8192) return false;
   const size_t smem = resident_smem(disc, varnu, g, ctas, prec);
   if (smem > kResidentSmemMax) return false;
-  const void* fn = prec == HHG_FP64 ? kernel_of<double>(disc, varnu, false) : kernel_of<float>(disc, varnu, false);
+  const bool compact = resident_compact(disc, varnu, g, ctas, prec);
+  const void* fn = prec == HHG_FP64 ? kernel_of<double>(disc, varnu, compact, false)
+                                    : kernel_of<float>(disc, varnu, compact, false);
   if (!fn || cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kResidentSmemMax)) != cudaSuccess ||
       cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
     cudaGetLastError();
@@ -464,13 +500,14 @@ int uzawa_resident(int disc, int varnu, const Geo& g, int ctas, int threads, T* 
   cudaLaunchAttribute attr[1];
   fill_config(cfg, attr, ctas, threads, resident_smem(disc, varnu, g, ctas, prec_of<T>()), s);
   ResA<T> r{g, x, b, inv_ml, a, tabs};
+  const bool compact = resident_compact(disc, varnu, g, ctas, prec_of<T>());
   if (g_rec) {
-    g_rec->add(kernel_of<T>(disc, varnu, true), dim3(ctas), dim3(threads), cfg.dynamicSmemBytes, ctas, r);
+    g_rec->add(kernel_of<T>(disc, varnu, compact, true), dim3(ctas), dim3(threads), cfg.dynamicSmemBytes, ctas, r);
     return 0;
   }
   ++g_launches;
   void* args[] = {&r};
-  return cudaLaunchKernelExC(&cfg, kernel_of<T>(disc, varnu, false), args) == cudaSuccess ? 0 : -1;
+  return cudaLaunchKernelExC(&cfg, kernel_of<T>(disc, varnu, compact, false), args) == cudaSuccess ? 0 : -1;
 }
 
 template int uzawa_resident<double>(int, int, const Geo&, int, int, double*, const double*, const double*,

@@ -37,7 +37,9 @@ constexpr size_t kResidentSmemMax = 225 * 1024;   // dynamic shared memory per C
 // shared memory per CTA (bytes) of a cluster of `ctas` CTAs on the level: CTA
 // c owns the k planes [c (nz+1) / C, (c+1) (nz+1) / C) of every array and
 // keeps them, with one halo plane below and above, next to its right-hand
-// sides and site tables
+// sides and site tables (a compact layout without the tables where that does
+// not fit: resident_compact)
+bool resident_compact(int disc, int varnu, const Geo& g, int ctas, int prec);
 size_t resident_smem(int disc, int varnu, const Geo& g, int ctas, int prec);
 // true if `ctas` CTAs can hold the level (every CTA owns a plane, the slab
 // fits the shared memory, the cluster can be scheduled).  Sets the kernel's

@@ -22,12 +22,31 @@ CASES = [
     ("P2P1", (2, 1, 1), 2, 0.0, 4, 256),
     ("P2P1", (1, 1, 1), 3, 0.0, 8, 1024),
 ]
+# levels that fit the compact layout only
+COMPACT = [
+    ("P1P1", (2, 3, 1), 4, 0.0, 16, 1024, "fp32"),
+    ("P1P1", (1, 2, 3), 3, 1.7, 1, 256, "fp32"),
+    ("P1P1", (1, 3, 1), 4, 0.0, 9, 512, "fp64"),
+    ("P1P1", (3, 1, 1), 4, 1.2, 16, 1024, "fp64"),
+    ("P2P1", (2, 2, 1), 3, 0.0, 5, 1024, "fp32"),
+    ("P2P1", (1, 1, 1), 4, 0.9, 9, 512, "fp32"),
+]
 
 
 @pytest.mark.parametrize("ahat,xi", [("f", 3), ("s", 2)])
 @pytest.mark.parametrize("prec", ["fp64", "fp32"])
 @pytest.mark.parametrize("disc,box,L,nu_a,ctas,threads", CASES)
 def test_resident_smoother(disc, box, L, nu_a, ctas, threads, prec, ahat, xi):
+    check(disc, box, L, nu_a, ctas, threads, prec, ahat, xi)
+
+
+@pytest.mark.parametrize("ahat,xi", [("f", 2), ("s", 1)])
+@pytest.mark.parametrize("disc,box,L,nu_a,ctas,threads,prec", COMPACT)
+def test_compact_layout(disc, box, L, nu_a, ctas, threads, prec, ahat, xi):
+    check(disc, box, L, nu_a, ctas, threads, prec, ahat, xi)
+
+
+def check(disc, box, L, nu_a, ctas, threads, prec, ahat, xi):
     from oracle.stokes import Params
     from paper_2010_13513_gb300 import hhg
     lc = 0 if disc == "P1P1" else 1

@@ -200,12 +200,13 @@ def apply_roofline(pb, steps=20):
 
 
 def kernel_source_hash():
-    """sha256 of the sources of the streaming stencil-row kernel (the apply
-    kernel of the roofline line): its source and header, and the generator
-    and stencil builder that produce its compile-time row structure."""
+    """sha256 of the sources of the large levels' stencil-row kernels (the apply
+    kernel of the roofline line: marching for P2-P1, streaming for P1-P1):
+    their sources and headers, and the generator and stencil builder that
+    produce their compile-time row structure."""
     import hashlib
     h = hashlib.sha256()
-    for f in ("stream.cu", "stream.h", "gen_structure.cpp", "stencils.cpp"):
+    for f in ("march.cu", "march.h", "stream.cu", "stream.h", "at.h", "gen_structure.cpp", "stencils.cpp"):
         path = os.path.join(ROOT, "paper_2010_13513_gb300", "csrc", f)
         if os.path.exists(path):
             with open(path, "rb") as fh:

@@ -164,7 +164,7 @@ int hhg_problem_create(const hhg_mesh* mesh, const hhg_problem_desc* desc, hhg_p
 int hhg_problem_workspace_bytes(const hhg_problem* pb, size_t* bytes);
 /* Binds a device workspace (>= hhg_problem_workspace_bytes, 256-byte aligned)
  * and the CUDA stream (cudaStream_t, 0 = legacy default stream); uploads the
- * stencil and transfer tables, assembles and inverts the bordered coarse
+ * stencil tables, assembles and inverts the bordered coarse
  * system.  Synchronises the stream. */
 int hhg_problem_bind(hhg_problem* pb, void* workspace, size_t bytes, void* stream);
 int hhg_problem_destroy(hhg_problem* pb);
@@ -248,8 +248,8 @@ int hhg_vcycle(hhg_problem* pb, int level, const hhg_params* prm, int prec, void
  * x_out (device, may be NULL to keep it only in the workspace).  stats may be
  * NULL; if given, residual norms are computed (synchronises). */
 int hhg_fmg_solve(hhg_problem* pb, const hhg_params* prm, void* x_out, hhg_stats* stats);
-/* Per-level autotuner of the launch shapes (threads per block and k planes
- * per thread of the stencil-row kernels, threads per block of the
+/* Per-level autotuner of the launch shapes (threads per block of the streaming
+ * kernels of the full operator or none, threads per block and order of the
  * Gauss-Seidel kernels, and the smoother's resident CTA count of
  * hhg_set_level_smoother): every candidate is timed `reps` times with CUDA
  * events on the problem's stream in the precision of the V-cycles, the
@@ -257,36 +257,28 @@ int hhg_fmg_solve(hhg_problem* pb, const hhg_params* prm, void* x_out, hhg_stats
  * are dropped.  shapes_out (optional) receives 16 ints per level (coarse ..
  * L): row threads, row k planes, Gauss-Seidel threads (edge groups), resident CTAs,
  * resident threads per CTA, the threads per block of the streaming kernel
- * of the full operator (0 = the plain kernels), the row kernels' sites per
- * thread, the
- * lanes per Gauss-Seidel site of the edge groups and of the vertex colours
- * (tuned apart), and the threads, k planes and sites per thread of the
- * smoother's B^T rows and of its (B, -C) rows (tuned apart from the full
- * operator's), and the Gauss-Seidel threads of the vertex colours.
- * Synchronises. */
+ * of the full operator (0 = the plain kernels), the sites per thread of
+ * hhg_set_launch_shape, the lanes per Gauss-Seidel site of the edge groups and
+ * of the vertex colours (1), the threads, k planes and sites per thread of the
+ * smoother's B^T rows and of its (B, -C) rows, and the Gauss-Seidel threads of
+ * the vertex colours.  Slots of kernels that have one shape keep their place
+ * and a fixed value.  Synchronises. */
 int hhg_autotune(hhg_problem* pb, int reps, int* shapes_out);
 /* Not in the paper (GPU launch choices): the launch shape of the stencil
- * kernels of one level -- threads per block of the row kernels (64/128/256),
- * k planes per thread (1..64), threads per block of the Gauss-Seidel kernels
+ * kernels of one level -- threads per block of the row kernels (64/128/256)
+ * and k planes per thread (1..64), both reported back only, since these
+ * kernels have one shape; threads per block of the Gauss-Seidel kernels
  * (64/128/256), and row_tile = 64, 128 or 256 (1 = 128) to evaluate the
- * rows of the full operator (apply, residual) and of the smoother's B^T and
- * (B, -C) residuals, in both precisions, by the streaming kernels with that
- * many threads per block (a block owns 4 x threads positions of the (i, j)
+ * rows of the full operator (apply, residual; in both precisions, P2-P1 in
+ * FP64 only) by the streaming kernels with that many threads per block (a block owns 4 x threads positions of the (i, j)
  * plane, stages the planes of its input arrays in shared memory as it marches
  * along k, and loads each line of a thread's stencil footprint once per
  * plane; the grid is one wave of blocks with equal runs of planes; only on
  * levels with nx >= 64, whose pitch sx is a multiple of four; four sites per
- * thread, or two for FP32 with row_sites = 2; 0 = the plain kernels), and
- * row_sites = 1 or 4 sites per thread of the
- * row kernels (4: each warp evaluates four runs of 32 consecutive
- * positions of the padded (i, j) plane, sharing each term's address
- * between the runs; row_tile != 0 takes precedence; sets the FP32
- * and FP64 rows, which hhg_autotune chooses separately), and gs_lanes = 1, 2
- * or 4 lanes per Gauss-Seidel site (the lanes take every gs_lanes-th term
- * of the site's rows and add their sums by shuffles; sets the vertex colours
- * and the edge groups, which hhg_autotune chooses apart; the B^T and
- * (B, -C) rows take this shape too until hhg_autotune gives them their own).  Results agree up to
- * rounding.  Drops cached graphs.  hhg_get_launch_shape writes the six
+ * thread, or two for FP32 with row_sites = 2; 0 = the plain kernels; sets the
+ * FP32 and FP64 rows, which hhg_autotune chooses separately), row_sites = 1, 2
+ * or 4 and gs_lanes = 1, 2 or 4 (otherwise reported back only: a
+ * Gauss-Seidel site has one lane).  Results agree up to rounding.  Drops cached graphs.  hhg_get_launch_shape writes the six
  * values to shape6 in the same order; its row_sites slot reads 2 when the
  * level's streaming rows (first velocity pass) take 2 sites per thread. */
 int hhg_set_launch_shape(hhg_problem* pb, int level, int row_threads, int row_kplanes, int gs_threads, int row_tile,

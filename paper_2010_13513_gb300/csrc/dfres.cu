@@ -238,7 +238,7 @@ __device__ __forceinline__ void df_store(const Geo& g, const OpDev& op, int R, i
 }
 
 // row R = (OUT, OG, ALL, T0, N0, N1, N2) on the sites of the block: the
-// indexing of the vector row kernels (four runs of 32 positions per warp; a
+// indexing in the file's header (V runs of 32 positions per warp; a
 // warp whose last run passes the group's last site takes its sites one by one)
 template <int V, int VARNU, int OUT, int OG, int ALL, int T0, int N0, int N1, int N2, class Tab>
 __device__ __forceinline__ void df_rows(const uint3 bid, const Geo& g, int R, const float* __restrict__ xh,

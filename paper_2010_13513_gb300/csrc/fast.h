@@ -1,5 +1,5 @@
-// Specialised stencil kernels (fast.cu): compile-time row structure,
-// weights and linear offsets passed as __grid_constant__ parameters.
+// Tables and launch shapes of the specialised stencil kernels (rows.cu,
+// march.cu, stream.cu, gs.cu): their row structure is known at compile time.
 #pragma once
 
 #include <cuda_runtime.h>

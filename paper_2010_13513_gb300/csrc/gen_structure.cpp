@@ -1,7 +1,7 @@
 // Build-time generator: prints the per-row term counts of the hot stencil
 // operators (FULL, A, BT, BC) for P1-P1 / P2-P1 and constant / variable
-// viscosity, as compile-time tables for the specialised kernels in fast.cu,
-// and the pass/line plan of the streaming kernels in stream.cu.  The counts
+// viscosity, as compile-time tables for the specialised kernels, and the
+// pass/line plan of the kernels that read each line once.  The counts
 // come from the same builder that produces the run-time weights, so the two
 // always agree.
 #include <algorithm>

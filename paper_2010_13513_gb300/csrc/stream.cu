@@ -1,5 +1,7 @@
 // Streaming stencil rows: y = calA x and r = b - calA x over all rows of the
-// operator (Eq. stokes-discrete), on levels large enough to fill the GPU.
+// operator (Eq. stokes-discrete), on levels large enough to fill the GPU: P1-P1
+// in both precisions and P2-P1 in FP64 (P2-P1 in FP32 marches in registers,
+// march.cu).
 //
 // Data reuse.  In the Kuhn-lattice layout an input value x(a, site) is read
 // by the rows of every DoF group at about 27 neighbouring sites, so a kernel

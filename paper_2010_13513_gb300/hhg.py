@@ -433,7 +433,8 @@ class Problem:
         stream_threads, row_sites, gs_lanes, gs_lanes_vertex, bt_threads,
         bt_kplanes, bt_sites, bc_threads, bc_kplanes, bc_sites,
         gs_threads_vertex)}; stream_threads is the block size of the
-        streaming kernel of the full operator (0: the plain kernels)."""
+        streaming kernel of the full operator (0: the plain kernels); the
+        slots of kernels that have one shape hold a fixed value."""
         n = self.L - self.lc + 1
         out = (C.c_int * (16 * n))()
         _check(load().hhg_autotune(self.h, reps, out), "hhg_autotune")
@@ -441,8 +442,9 @@ class Problem:
 
     def set_launch_shape(self, level, row_threads, row_kplanes, gs_threads, row_tile=0, row_sites=1, gs_lanes=1):
         """row_tile: 0 = plain row kernels; 64/128/256 = the streaming kernels
-        with that many threads per block (levels with nx >= 64), of 4 sites
-        per thread, or 2 (FP32) with row_sites = 2."""
+        with that many threads per block (levels with nx >= 64; P1-P1, and
+        P2-P1 in FP64), of 4 sites per thread, or 2 (FP32) with row_sites =
+        2; row_threads, row_kplanes and gs_lanes are only reported back."""
         _check(load().hhg_set_launch_shape(self.h, level, row_threads, row_kplanes, gs_threads, int(row_tile),
                                            int(row_sites), int(gs_lanes)), "hhg_set_launch_shape")
 

@@ -25,7 +25,7 @@
 // sweep of P2-P1: FP32 level 5 / 6 / 7 28.8 / 59.5 / 543 us before, 23.8 / 59.9
 // / 439 us now (level 7 with the shared edge sums); FP64 level 4 44 us before,
 // 31 us; P1-P1 at 2.1 / 17 million sites, constant viscosity, 47.7 / 378 us
-// before, 34.4 / 367 us, variable viscosity 64.9 / 443 us before, 53.9 / 426 us.
+// before, 34.1 / 368 us, variable viscosity 64.9 / 443 us before, 53.4 / 426 us.
 // Programmatic launches pay at every size: limited to one wave of
 // blocks, the level-6 sweep takes 78 us.
 #include <cuda_runtime.h>
@@ -98,18 +98,33 @@ __device__ __forceinline__ void gs_site(const uint3 bid, const GsA<T, NW>& a) {
   if (j >= g.ny || i >= g.nx || (!ox && i == 0)) return;
   const int kb = kByPlane<DISC, T> ? k : 0;          // the plane that offsets count from
   const Lines<T> at(g, unsigned(i + 1) + unsigned(j + 1) * unsigned(g.sx) + unsigned(k - kb + 1) * unsigned(g.sy));
-  T v[NC];
-#pragma unroll
-  for (int c = 0; c < NC; ++c) {
-    const int64_t base = int64_t(a.comp + int(bid.y) + c) * G * g.arr;
-    T r = ld_at(a.rhs + kb * g.sy + (SEL == kVertexTerms ? int64_t(bid.y) * g.arr : base + GRP * g.arr), at.site());
-    const T s = row_sum<S, GRP, SEL>(g, a.u + base + kb * g.sy, at, a.w, std::make_integer_sequence<int, rw.n1 - 1>{});
-    if (VARNU && SEL != kVertexTerms) r *= T(g.eisc[k]);
-    v[c] = (r - (VARNU ? s : T(g.h) * s)) * a.inv_diag;
+  const int64_t base = int64_t(a.comp + int(bid.y)) * G * g.arr;
+  T* u = a.u + base;
+  const T* rhs = a.rhs + (SEL == kVertexTerms ? int64_t(bid.y) * g.arr : base + GRP * g.arr);
+  if constexpr (kByPlane<DISC, T>) {
+    u += kb * g.sy;
+    rhs += kb * g.sy;
   }
+  if constexpr (NC == 1) {
+    T r = ld_at(rhs, at.site());
+    const T s = row_sum<S, GRP, SEL>(g, u, at, a.w, std::make_integer_sequence<int, rw.n1 - 1>{});
+    if (VARNU && SEL != kVertexTerms) r *= T(g.eisc[k]);
+    ref_at(u + GRP * g.arr, at.site()) = (r - (VARNU ? s : T(g.h) * s)) * a.inv_diag;
+  } else {
+    static_assert(DISC == 1 && SEL == kAllTerms && GRP == 0, "one array per component");
+    T v[NC];
 #pragma unroll
-  for (int c = 0; c < NC; ++c)
-    ref_at(a.u + int64_t(a.comp + int(bid.y) + c) * G * g.arr + kb * g.sy + GRP * g.arr, at.site()) = v[c];
+    for (int c = 0; c < NC; ++c) {
+      const int64_t bc = int64_t(a.comp + int(bid.y) + c) * G * g.arr;
+      T r = ld_at(a.rhs + kb * g.sy + (SEL == kVertexTerms ? int64_t(bid.y) * g.arr : bc + GRP * g.arr), at.site());
+      const T s = row_sum<S, GRP, SEL>(g, a.u + bc + kb * g.sy, at, a.w, std::make_integer_sequence<int, rw.n1 - 1>{});
+      if (VARNU && SEL != kVertexTerms) r *= T(g.eisc[k]);
+      v[c] = (r - (VARNU ? s : T(g.h) * s)) * a.inv_diag;
+    }
+#pragma unroll
+    for (int c = 0; c < NC; ++c)
+      ref_at(a.u + int64_t(a.comp + int(bid.y) + c) * G * g.arr + kb * g.sy + GRP * g.arr, at.site()) = v[c];
+  }
 }
 template <int DISC, int VARNU, int GRP, int SEL, int NC, class T>
 __global__ void __launch_bounds__(256) k_gs(const __grid_constant__ GsA<T, row_nw<DISC, VARNU, GRP>()> a) {

@@ -34,11 +34,13 @@
 namespace hhg {
 namespace {
 
-// weight of the coarse node at doubled position (nx, ny, nz) (0..2) of a cell
-// at the point with coordinates (px, py, pz) / 4 of the cell, quadratic
-// interpolation on the Kuhn tetrahedron that holds the point: the tetrahedron
-// 0 -> e_a -> e_a + e_b -> (1, 1, 1) of the coordinates in descending order
-constexpr double p2_weight(int px, int py, int pz, int nx, int ny, int nz) {
+// local node I (the vertices, then the edges 01 02 03 12 13 23) of the Kuhn
+// tetrahedron that holds the point with coordinates (px, py, pz) / 4 of a cell:
+// its doubled position (0..2) in the cell and its weight at the point, quadratic
+// interpolation.  The tetrahedron is 0 -> e_a -> e_a + e_b -> (1, 1, 1) of the
+// coordinates in descending order.
+struct P2Node { int x, y, z; double w; };
+constexpr P2Node p2_node(int px, int py, int pz, int I) {
   const int p[3] = {px, py, pz};
   int o[3] = {0, 1, 2};
   for (int r = 0; r < 2; ++r)                      // stable sort, descending
@@ -52,10 +54,16 @@ constexpr double p2_weight(int px, int py, int pz, int nx, int ny, int nz) {
   int v[4][3] = {};
   for (int s = 0; s < 3; ++s)
     for (int d = 0; d < 3; ++d) v[s + 1][d] = v[s][d] + (d == o[s] ? 1 : 0);
-  for (int a = 0; a < 4; ++a)
-    for (int b = a; b < 4; ++b)
-      if (v[a][0] + v[b][0] == nx && v[a][1] + v[b][1] == ny && v[a][2] + v[b][2] == nz)
-        return a == b ? lam[a] * (2 * lam[a] - 1) : 4 * lam[a] * lam[b];
+  const int a = I < 4 ? I : I < 7 ? 0 : I < 9 ? 1 : 2, b = I < 4 ? I : I < 7 ? I - 3 : I < 9 ? I - 5 : 3;
+  return P2Node{v[a][0] + v[b][0], v[a][1] + v[b][1], v[a][2] + v[b][2],
+                a == b ? lam[a] * (2 * lam[a] - 1) : 4 * lam[a] * lam[b]};
+}
+// weight of the coarse node at doubled position (nx, ny, nz) of a cell at the point
+constexpr double p2_weight(int px, int py, int pz, int nx, int ny, int nz) {
+  for (int I = 0; I < 10; ++I) {
+    const P2Node n = p2_node(px, py, pz, I);
+    if (n.x == nx && n.y == ny && n.z == nz) return n.w;
+  }
   return 0.0;
 }
 // group of a parity offset (order of kGroupOff)
@@ -69,15 +77,18 @@ __device__ __forceinline__ int64_t xsite(const Geo& g, int i, int j, int k) {
 }
 
 // ------------------------------------------------------------- prolongation
-template <int PX, int PY, int PZ, int NZ, class T, int... N>
-__device__ __forceinline__ T p2_point(const T (&c)[NZ * 9], std::integer_sequence<int, N...>) {
+// the value at point (PX, PY, PZ) from the loaded nodes c, NX of them in x of
+// which the cell's start at X0; the small vertex terms before the edge terms
+template <int PX, int PY, int PZ, int NX, int X0, int NC, class T, int... I>
+__device__ __forceinline__ T p2_point(const T (&c)[NC], std::integer_sequence<int, I...>) {
   T a = T(0);
   ([&] {
-    constexpr double w = p2_weight(PX, PY, PZ, N % 3, N / 3 % 3, N / 9);
-    if constexpr (w != 0.0) a = fma(T(w), c[N], a);
+    constexpr P2Node n = p2_node(PX, PY, PZ, I);
+    if constexpr (n.w != 0.0) a = fma(T(n.w), c[X0 + n.x + NX * (n.y + 3 * n.z)], a);
   }(), ...);
   return a;
 }
+constexpr auto kP2Nodes = std::make_integer_sequence<int, 10>{};
 
 // xf += v, or xf = v (SET)
 template <bool SET, class T>
@@ -111,7 +122,7 @@ __device__ __forceinline__ void prolong_p2(const Geo& gf, const Geo& gc, int ax,
     if (Px > 2 * gf.nx || Py > 2 * gf.ny) return;
     const bool in = inz && Px >= lo && Px <= 2 * gf.nx - lo && Py >= lo && Py <= 2 * gf.ny - lo;
     T* f = f0 + group_at(PX & 1, PY & 1, PZ & 1) * gf.arr + (PX >> 1) + (PY >> 1) * gf.sx + (PZ >> 1) * gf.sy;
-    const T v = p2_point<PX, PY, PZ, NZ>(c, std::make_integer_sequence<int, NZ * 9>{});
+    const T v = p2_point<PX, PY, PZ, 3, 0>(c, kP2Nodes);
     if (in) put<SET>(f, v);
     else if (SET) *f = T(0);                       // Dirichlet row
   };
@@ -156,22 +167,11 @@ __device__ __forceinline__ void put_pair(T* f, bool in0, bool in1, T v0, T v1) {
   if (in1) p.y += v1;
   *reinterpret_cast<P*>(f) = p;
 }
-// point (PX, PY, PZ) of the cell whose first x node is number X0 of the five loaded
-template <int PX, int PY, int PZ, int NZ, int X0, class T, int... N>
-__device__ __forceinline__ T p2_point5(const T (&c)[NZ * 15], std::integer_sequence<int, N...>) {
-  T a = T(0);
-  ([&] {
-    constexpr double w = p2_weight(PX, PY, PZ, N % 3, N / 3 % 3, N / 9);
-    if constexpr (w != 0.0) a = fma(T(w), c[X0 + N % 3 + 5 * (N / 3)], a);
-  }(), ...);
-  return a;
-}
 template <int PZ, bool SET, class T, int... Q>
 __device__ __forceinline__ void prolong_p2_pair(const Geo& gf, const Geo& gc, int ax, int ay, int az,
                                                 bool interior_only, const T* __restrict__ xc, T* __restrict__ xf,
                                                 std::integer_sequence<int, Q...>) {
   constexpr int NZ = PZ == 0 ? 1 : 3;
-  constexpr auto nodes = std::make_integer_sequence<int, NZ * 9>{};
   T c[NZ * 15];
   const T* x0 = xc + xsite(gc, ax - 1, ay, az);
 #pragma unroll
@@ -192,7 +192,7 @@ __device__ __forceinline__ void prolong_p2_pair(const Geo& gf, const Geo& gc, in
     if (!SET && !in) return;
     T* f = f0 + group_at(ODD, PY & 1, PZ & 1) * gf.arr + (PY >> 1) * gf.sx + (PZ >> 1) * gf.sy;
     put_pair<SET>(f, in && Px - 2 >= lo && Px - 2 <= 2 * gf.nx - lo, in && Px >= lo && Px <= 2 * gf.nx - lo,
-                  p2_point5<2 + ODD, PY, PZ, NZ, 0>(c, nodes), p2_point5<ODD, PY, PZ, NZ, 2>(c, nodes));
+                  p2_point<2 + ODD, PY, PZ, 5, 0>(c, kP2Nodes), p2_point<ODD, PY, PZ, 5, 2>(c, kP2Nodes));
   };
   (at(std::integral_constant<int, Q>{}), ...);
 }
@@ -273,33 +273,55 @@ constexpr double p2_restrict_weight(int ox, int oy, int oz, int ex, int ey, int 
                    oz - 2 * bz);
 }
 
+// the fine nodes around coarse node (2 a + o) with a weight: group and site
+// relative to the fine vertex at the node's cell (doubled fine position 4 a), by
+// group and offset (x slowest)
+struct RTerm { int grp, dx, dy, dz; double w; };
+struct RTerms { int n; RTerm t[125]; };
+template <int OX, int OY, int OZ>
+constexpr RTerms p2_restrict_terms() {
+  RTerms r{};
+  for (int g = 0; g < 8; ++g)
+    for (int dx = -2; dx <= 2; ++dx)
+      for (int dy = -2; dy <= 2; ++dy)
+        for (int dz = -2; dz <= 2; ++dz) {
+          const int ex = 2 * dx + kGroupOff[g][0] - 2 * OX, ey = 2 * dy + kGroupOff[g][1] - 2 * OY,
+                    ez = 2 * dz + kGroupOff[g][2] - 2 * OZ;
+          if (ex < -3 || ex > 3 || ey < -3 || ey > 3 || ez < -3 || ez > 3) continue;
+          const double w = p2_restrict_weight(OX, OY, OZ, ex, ey, ez);
+          if (w != 0.0) r.t[r.n++] = RTerm{g, dx, dy, dz, w};
+        }
+  return r;
+}
+template <int OX, int OY, int OZ>
+struct Restrict { static constexpr RTerms r = p2_restrict_terms<OX, OY, OZ>(); };
+
 // sum over the fine nodes around coarse node (2 a + o); f0: the fine vertex at
-// the node's cell, i.e. doubled fine position 4 a
+// the node's cell.  Eight chains of equal length: short sums (with chains that
+// differ by the zero weights left out the FP32 error is a tenth larger) and
+// independent latencies.
 template <int OX, int OY, int OZ, class T, int... E>
 __device__ __forceinline__ T restrict_p2(const Geo& gf, const T* __restrict__ f0, std::integer_sequence<int, E...>) {
-  T s[8] = {};                                     // eight chains: short sums, independent latencies
+  T s[8] = {};
   ([&] {
-    constexpr int ex = E % 7 - 3, ey = E / 7 % 7 - 3, ez = E / 49 - 3;
-    constexpr double w = p2_restrict_weight(OX, OY, OZ, ex, ey, ez);
-    if constexpr (w != 0.0) {
-      // doubled fine position relative to 4 a; arithmetic shift = floor
-      constexpr int rx = 2 * OX + ex, ry = 2 * OY + ey, rz = 2 * OZ + ez;
-      constexpr int grp = group_at(rx & 1, ry & 1, rz & 1);
-      s[E & 7] = fma(T(w), __ldg(f0 + grp * gf.arr + (rx >> 1) + (ry >> 1) * gf.sx + (rz >> 1) * gf.sy), s[E & 7]);
-    }
+    constexpr RTerm t = Restrict<OX, OY, OZ>::r.t[E];
+    s[E & 7] = fma(T(t.w), __ldg(f0 + t.grp * gf.arr + t.dx + t.dy * gf.sx + t.dz * gf.sy), s[E & 7]);
   }(), ...);
-  return ((s[0] + s[1]) + (s[2] + s[3])) + ((s[4] + s[5]) + (s[6] + s[7]));
+  return ((s[0] + s[4]) + (s[2] + s[6])) + ((s[1] + s[5]) + (s[3] + s[7]));
 }
 
+// a P1 field: two chains over the 15 fine nodes in the order of their offsets
 template <class T>
 __device__ __forceinline__ T restrict_p1(const Geo& gf, const T* __restrict__ f) {
-  T s = T(0);
+  T s[2] = {T(0), T(0)};
 #pragma unroll
-  for (int q = 1; q < 8; ++q) {
-    const int d = (q & 1) + (q >> 1 & 1) * gf.sx + (q >> 2) * int(gf.sy);
-    s += __ldg(f + d) + __ldg(f - d);
+  for (int q = 0; q < 15; ++q) {
+    // 7 - q: the offsets (x, y, z) in binary below the node, its own, and above it
+    const int b = q < 7 ? 7 - q : q - 7;
+    const int d = (b >> 2 & 1) + (b >> 1 & 1) * gf.sx + (b & 1) * int(gf.sy);
+    s[q & 1] = fma(q == 7 ? T(1) : T(0.5), __ldg(q < 7 ? f - d : f + d), s[q & 1]);
   }
-  return fma(T(0.5), s, __ldg(f));
+  return s[0] + s[1];
 }
 
 template <int GRP, class T>
@@ -310,7 +332,8 @@ __device__ __forceinline__ void restrict_group(const Geo& gf, const Geo& gc, int
   const bool inside = Px > 0 && Py > 0 && Pz > 0 && Px < 2 * gc.nx && Py < 2 * gc.ny && Pz < 2 * gc.nz;
   T v = T(0);
   if (inside)
-    v = restrict_p2<ox, oy, oz>(gf, rf + xsite(gf, 2 * i, 2 * j, 2 * k), std::make_integer_sequence<int, 343>{});
+    v = restrict_p2<ox, oy, oz>(gf, rf + xsite(gf, 2 * i, 2 * j, 2 * k),
+                                std::make_integer_sequence<int, Restrict<ox, oy, oz>::r.n>{});
   rc[GRP * gc.arr + xsite(gc, i, j, k)] = v;
 }
 

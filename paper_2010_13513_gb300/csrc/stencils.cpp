@@ -233,6 +233,22 @@ void accumulate_block(BlockAcc& acc, int out_order, int og, int in_order, int in
         }
 }
 
+// With a constant viscosity the weights of A are multiples of h / 360, those of
+// B and B^T of h^2 / 360 (P2 gradients and P1 functions integrated over Kuhn
+// tetrahedra).  They are rounded to these multiples, since the quadrature leaves
+// errors of up to 4e-15 that depend on how this file is compiled (contracted
+// multiply-adds): the generator of the unrolled rows and the library are two
+// compilations of it, and the weights of h = 1 that the one prints are used
+// beside the diagonals and tables of the other.
+void round_weights(BlockAcc& acc, double scale) {
+  auto round = [&](double& w) {
+    const double n = std::round(w / scale * 360.0);
+    if (std::fabs(w / scale * 360.0 - n) < 1e-9) w = n * scale / 360.0;
+  };
+  for (auto& kv : acc.merged) round(kv.second);
+  for (auto& kv : acc.cube) round(kv.second);
+}
+
 // Terms that cancel exactly for a constant viscosity (e.g. the diagonal
 // directions of the P1 Laplacian) are dropped; with a variable viscosity every
 // structural term is kept, so the term list never depends on the values.
@@ -297,6 +313,10 @@ StencilSet build_stencils(int disc, double h, double nu_a, bool pspg_rhs) {
       accumulate_block(aA, ov, g, ov, c * G, +1, nu_ah, 1.0, K);
       accumulate_block(aBT, ov, g, 1, parr, 0, nu_ah, 1.0,
                        [&](int s, int a, int k) { return E[s].D[c][k * nv + a]; });
+      if (nu_a == 0.0) {
+        round_weights(aA, h);
+        round_weights(aBT, h * h);
+      }
       accumulate_block(aM, ov, g, ov, c * G, 0, nu_ah, 1.0, Mv);
       HRow rA{out, g, false, {}, {}};
       flush_block(aA, rA, 1, true, c * G + g, false);
@@ -324,6 +344,7 @@ StencilSet build_stencils(int disc, double h, double nu_a, bool pspg_rhs) {
         accumulate_block(aL, 1, 0, ov, c * G, -1, nu_ah, 1.0,
                          [&](int s, int k, int j) { return E[s].L[c][k * nv + j]; });
     }
+    if (nu_a == 0.0) round_weights(aB, h * h);
     if (ov == 1) accumulate_block(aC, 1, 0, 1, parr, -1, nu_ah, 1.0, Cq);
     accumulate_block(aMq, 1, 0, 1, parr, 0, nu_ah, 1.0, Mq);
     accumulate_block(aMLh, 1, 0, 1, parr, -1, nu_ah, 1.0, MLq);

@@ -21,6 +21,22 @@ __device__ __forceinline__ const T& ref_at(const T* base, unsigned off) {
   return *reinterpret_cast<const T*>(reinterpret_cast<const char*>(base) + off);
 }
 
+// A row of n terms summed by m chains of consecutive terms.  Terms whose weights
+// cancel on smooth fields are neighbours in the generated order and stay in one
+// chain (the pressure row of P2-P1 starts -w -w -w -3w +w +w +w): dealt out in
+// turn, every chain would sum values that cancel only at the end.
+// The chain of term i:
+constexpr int chain_of(int i, int n, int m) { return i * m / n; }
+// The term evaluated in step j of chain_steps where the chains take turns (-1:
+// none): for long rows in kernels of few warps (P2-P1 level 7 with variable
+// viscosity, one smoothing step with its pressure row chain after chain 2.04 ms,
+// in turns 1.83 ms).
+constexpr int chain_term(int j, int n, int m) {
+  const int q = j % m, e = (q * n + m - 1) / m + j / m;
+  return e < ((q + 1) * n + m - 1) / m ? e : -1;
+}
+constexpr int chain_steps(int n, int m) { return (n + m - 1) / m * m; }
+
 // FP64 P1-P1 arrays may exceed the 4 GB (up to 715 million sites are
 // accepted): its kernels count offsets from the site's plane instead
 template <int DISC, class T>

@@ -124,17 +124,22 @@ __device__ __forceinline__ T c_class(const Geo& g, const T* __restrict__ p, cons
   ((a = fma(__ldg(wc + O), __ldg(p + SPT::cbo[O].di + SPT::cbo[O].dj * g.sx + SPT::cbo[O].dk * g.sy), a)), ...);
   return a;
 }
-// terms [T0, T0 + n) of the pressure row: four chains of sums
-template <class S, int T0, class SPT, class T, class Tab, int... I>
+// terms [T0, T0 + n) of the pressure row: eight (P1-P1: three, a component each)
+// chains of consecutive terms (FP32 error of the apply's pressure, P2-P1 level 6:
+// 1.9e-7 in one chain, 4.8e-7 with the terms dealt out to four in turn, 1.0e-7
+// now; see chain_of)
+template <int DISC, class S, int T0, class SPT, class T, class Tab, int... I>
 __device__ __forceinline__ T b_terms(const Geo& g, const T* __restrict__ x, const Lines<T>& at, const Tab& tab,
                                      std::integer_sequence<int, I...>) {
-  T a[4] = {};
+  constexpr int M = DISC == 2 ? 8 : 3;
+  T a[M] = {};
   ([&] {
     constexpr gen::OffT o = S::off[T0 + I];
-    a[I & 3] = fma(fweight<SPT, T0 + I, T>(tab), at.template ld<o.di, o.dj, o.dk>(x + o.arr * g.arr),
-                   a[I & 3]);
+    constexpr int q = chain_of(I, sizeof...(I), M);
+    a[q] = fma(fweight<SPT, T0 + I, T>(tab), at.template ld<o.di, o.dj, o.dk>(x + o.arr * g.arr), a[q]);
   }(), ...);
-  return (a[0] + a[1]) + (a[2] + a[3]);
+  if constexpr (M == 3) return (a[0] + a[1]) + a[2];
+  else return ((a[0] + a[1]) + (a[2] + a[3])) + ((a[4] + a[5]) + (a[6] + a[7]));
 }
 
 template <int MODE, class T>
@@ -196,7 +201,7 @@ __device__ __forceinline__ void pressure_row(const FullA<T>& a, int i, int j, in
   constexpr gen::RowS rw = S::rows[PARR];
   static_assert(rw.out == PARR && rw.n1 == 0, "the last row is the pressure's; B is unscaled");
   const Geo& g = a.g;
-  T v = b_terms<S, rw.t0, SPT>(g, a.x, at, tab, std::make_integer_sequence<int, rw.n0>{});
+  T v = b_terms<DISC, S, rw.t0, SPT>(g, a.x, at, tab, std::make_integer_sequence<int, rw.n0>{});
   if (!kTabled<DISC, VARNU, T>) v *= T(g.h) * T(g.h);
   if constexpr (rw.n2 > 0) {
     T c;
@@ -215,8 +220,9 @@ __device__ __forceinline__ void pressure_row(const FullA<T>& a, int i, int j, in
   put<MODE>(a, PARR, at.site(), true, v);
 }
 
-// grid x over the sites of the (i, j) plane (flat), y = plane, z = part: the
-// components (P1: all at once), then the pressure
+// grid x over the sites of the (i, j) plane (flat), y = plane, z = part: P1-P1 the
+// components, all at once, then the pressure; P2-P1 the pressure, whose row is
+// the longest chain of sums, then the components
 template <int DISC, int VARNU, int MODE, class T, class Tab>
 __device__ __forceinline__ void full_body(const uint3 bid, const FullA<T>& full, const Tab& tab) {
   const Geo& g = full.g;
@@ -232,11 +238,11 @@ __device__ __forceinline__ void full_body(const uint3 bid, const FullA<T>& full,
     else
       pressure_row<1, VARNU, MODE>(a, i, j, k, at, tab);
   } else {
-    if (bid.z == 0)
+    if (bid.z == 1)
       velocity_rows<2, VARNU, MODE, 0>(a, i, j, k, at, tab, std::make_integer_sequence<int, SPT::passes[0].np>{});
-    else if (bid.z == 1)
-      velocity_rows<2, VARNU, MODE, 1>(a, i, j, k, at, tab, std::make_integer_sequence<int, SPT::passes[1].np>{});
     else if (bid.z == 2)
+      velocity_rows<2, VARNU, MODE, 1>(a, i, j, k, at, tab, std::make_integer_sequence<int, SPT::passes[1].np>{});
+    else if (bid.z == 3)
       velocity_rows<2, VARNU, MODE, 2>(a, i, j, k, at, tab, std::make_integer_sequence<int, SPT::passes[2].np>{});
     else
       pressure_row<2, VARNU, MODE>(a, i, j, k, at, tab);

@@ -144,16 +144,22 @@ struct PressA { Geo g; const T* x; const T* b; T* p; const double* inv_ml; doubl
 template <int DISC, int VARNU>
 constexpr int bc_nw() { return VARNU ? gen::S<DISC, VARNU, OP_BC>::N : 1; }
 
-// terms [T0, T0 + n) of the pressure row: four chains of sums
-template <class S, int T0, int NW, class T, int... I>
+// terms [T0, T0 + N) of the pressure row: three chains, one per component, the
+// few C terms (whose diagonal stands in the middle) one chain
+template <bool CT> constexpr int kChains = CT ? 1 : 3;
+template <class S, int T0, int N, bool CT, int NW, class T, int... J>
 __device__ __forceinline__ T press_sum(const Geo& g, const T* __restrict__ x, const Lines<T>& at, const T (&w)[NW],
-                                       std::integer_sequence<int, I...>) {
-  T a[4] = {};
+                                       std::integer_sequence<int, J...>) {
+  constexpr int M = kChains<CT>;
+  T a[3] = {};
   ([&] {
-    constexpr gen::OffT o = S::off[T0 + I];
-    a[I & 3] = fma(rweight<S, T0 + I>(w), at.template ld<o.di, o.dj, o.dk>(x + o.arr * g.arr), a[I & 3]);
+    constexpr int e = chain_term(J, N, M);
+    if constexpr (e >= 0) {
+      constexpr gen::OffT o = S::off[T0 + e];
+      a[J % M] = fma(rweight<S, T0 + e>(w), at.template ld<o.di, o.dj, o.dk>(x + o.arr * g.arr), a[J % M]);
+    }
   }(), ...);
-  return (a[0] + a[1]) + (a[2] + a[3]);
+  return (a[0] + a[1]) + a[2];
 }
 // the C terms of a boundary row: the stencil of its class
 template <class SPT, class T, int... O>
@@ -183,7 +189,8 @@ __device__ __forceinline__ void press_body(const uint3 bid, const PressA<T, NW>&
     const T bv = __ldg(a.b + 3 * G * g.arr + idx);
     const T ml = T(a.s * __ldg(a.inv_ml + idx));
     const T* x = a.x + idx;
-    T v = press_sum<S, rw.t0>(g, a.x + kb * g.sy, at, a.w, std::make_integer_sequence<int, rw.n0>{});
+    T v = press_sum<S, rw.t0, rw.n0, false>(g, a.x + kb * g.sy, at, a.w,
+                                             std::make_integer_sequence<int, chain_steps(rw.n0, kChains<false>)>{});
     if (!VARNU) v *= T(g.h) * T(g.h);
     if constexpr (rw.n2 > 0) {
       using SPT = gen::SP<DISC, VARNU, OP_BC>;
@@ -193,7 +200,8 @@ __device__ __forceinline__ void press_body(const uint3 bid, const PressA<T, NW>&
                         9 * (k == 0 ? 0 : k == g.nz ? 2 : 1);
         c = press_c<SPT>(g, x + 3 * G * g.arr, a.tabs->wc + cls * SPT::NCB, std::make_integer_sequence<int, SPT::NCB>{});
       } else {
-        c = press_sum<S, rw.t0 + rw.n0>(g, a.x + kb * g.sy, at, a.w, std::make_integer_sequence<int, rw.n2>{});
+        c = press_sum<S, rw.t0 + rw.n0, rw.n2, true>(g, a.x + kb * g.sy, at, a.w,
+                                                        std::make_integer_sequence<int, rw.n2>{});
         if (!VARNU) c *= T(g.h) * T(g.h) * T(g.h);
       }
       v += VARNU ? T(g.eisc[k]) * c : c;

@@ -74,3 +74,81 @@ def test_restriction(disc, box, L):
         lib, plain = np.concatenate(lib), np.concatenate(plain)
         print(f"{disc} {name}: {rms(lib):.3e}, plain {rms(plain):.3e}, ratio {rms(lib) / rms(plain):.3f}")
         assert rms(lib) <= allowed(lib.size) * rms(plain)
+
+
+def sine_velocity(shape, seed=1):
+    """Canonical velocity lattice (z, y, x) of sine modes that vanish on the
+    boundary, with a tenth of noise: what a smoother meets."""
+    rng = np.random.default_rng(seed)
+    X = [np.linspace(0, 1, m) for m in shape]
+    u = np.zeros((3,) + shape)
+    for c in range(3):
+        for _ in range(4):
+            s = [np.sin(np.pi * rng.integers(1, 4) * x) for x in X]
+            u[c] += rng.standard_normal() * s[0][:, None, None] * s[1][:, None] * s[2]
+    u[:, 1:-1, 1:-1, 1:-1] += 0.1 * rng.standard_normal((3,) + tuple(m - 2 for m in shape))
+    u[:, [0, -1]] = u[:, :, [0, -1]] = u[:, :, :, [0, -1]] = 0
+    return f32(u)
+
+
+def divergence_terms(disc):
+    """An interior row of B at h = 1: (component, lattice offset x, y, z, weight)
+    by component, group of the parity offset and cell offset (x slowest), and the
+    row's lumped mass."""
+    q = 2 if disc == "P2P1" else 1
+    L, lc = 2, 0 if disc == "P1P1" else 1
+    lev = oracle_hierarchy((1, 1, 1), L, disc, lc=lc).lv[L]
+    n, h = 4, 0.25
+    m, group = q * n + 1, {(0, 0, 0): 0, (1, 0, 0): 1, (0, 1, 0): 2, (0, 0, 1): 3, (1, 1, 0): 4, (1, 0, 1): 5,
+                           (0, 1, 1): 6, (1, 1, 1): 7}
+    row = (n // 2) * (1 + (n + 1) * (1 + (n + 1)))
+    terms = []
+    for c in range(3):
+        B = lev.B[c].tocsr()
+        for col, w in zip(B.indices[B.indptr[row]:B.indptr[row + 1]], B.data[B.indptr[row]:B.indptr[row + 1]]):
+            d = np.array([col % m, col // m % m, col // (m * m)]) - q * n // 2
+            if abs(w) > 1e-13 * abs(B.data).max():
+                terms.append((c, group[tuple(d % q)], *(d // q), d, w / h ** 2))
+    terms.sort(key=lambda t: t[:5])
+    return [(t[0], *t[5], t[6]) for t in terms], lev.ML_hat[row] / h ** 3
+
+
+@pytest.mark.parametrize("disc,L,path", [("P1P1", 5, "residual"), ("P1P1", 5, "separate"), ("P1P1", 5, "resident"),
+                                         ("P2P1", 5, "residual"), ("P2P1", 5, "separate"), ("P2P1", 4, "resident")])
+def test_pressure_row(disc, L, path):
+    """B u of a smooth velocity, whose terms cancel: at most the error of one
+    chain over the row.  In the smoother the row meets the velocity it has just
+    written, and the factor omega M_L^-1 adds two roundings to both sides."""
+    from paper_2010_13513_gb300 import hhg
+    pb = lib_problem((1, 1, 1), L, disc, lc=0 if disc == "P1P1" else 1, solve="mixed")
+    q, n = 2 if disc == "P2P1" else 1, 2 ** L
+    vshape, npress = (q * n + 1,) * 3, (n + 1) ** 3
+    nv = 3 * (q * n + 1) ** 3
+    u = sine_velocity(vshape)
+    xd = pb.to_device(L, np.concatenate([u.ravel(), np.zeros(npress)]), hhg.FP32)
+    zero = pb.new_vector(L, hhg.FP32)
+    terms, mass = divergence_terms(disc)
+    h, om = 1.0 / n, OMEGA_INV[disc]
+    if path == "residual":
+        y = pb.new_vector(L, hhg.FP32)
+        pb.residual(L, xd, zero, y)
+        factor, out = -1.0, pb.to_host(L, y)
+    else:
+        pb.set_level_smoother(L, 0 if path == "separate" else 16, prec=hhg.FP32)
+        pb.smooth(L, hhg.Params.make(1, 1, 0, 1, "f", 1, om), 1, xd, zero)
+        out = pb.to_host(L, xd)
+        factor = 1.0 / (om * mass * h ** 3)
+        u = out[:nv].reshape((3,) + vshape)
+
+    def at(c, dx, dy, dz):                         # the DoF at an offset from every interior pressure node
+        s = [slice(q + d, q * (n - 1) + d + 1, q) for d in (dz, dy, dx)]
+        return u[(c, *s)].ravel()
+
+    X = np.stack([at(*t[:4]) for t in terms], axis=1)
+    W = np.broadcast_to(np.array([t[4] for t in terms]) * h ** 2, X.shape)
+    exact = (W * X).sum(1) * factor
+    lib = out[nv:].reshape((n + 1,) * 3)[1:-1, 1:-1, 1:-1].ravel() - exact
+    plain = f32(plain_sum(W, X) * f32(factor)) - exact
+    print(f"{disc} {path}: {rms(lib) / rms(exact):.3e}, one chain {rms(plain) / rms(exact):.3e}, "
+          f"ratio {rms(lib) / rms(plain):.3f}")
+    assert rms(lib) <= rms(plain)

@@ -45,6 +45,7 @@
 
 #include "batch.h"
 #include "kernels.h"
+#include "weights.h"
 #include "structure.inc"
 
 namespace hhg {
@@ -349,13 +350,6 @@ __global__ void __launch_bounds__(128) k_res_df(Geo g, const float* __restrict__
 // 20 instructions per term and site.  P2-P1 level 7, with the split of x: 1.75
 // ms before, 1.15 ms now; level 6: 259 us before, 171 us.  Bound: instruction
 // issue.
-template <int DISC> constexpr double kScaleA = DISC == 2 ? 15.0 : 1.0;
-template <int DISC> constexpr double kScaleB = DISC == 2 ? 60.0 : 12.0;
-constexpr double rounded(double v) { return v < 0 ? -double(int64_t(0.5 - v)) : double(int64_t(v + 0.5)); }
-constexpr bool near_integer(double v) {
-  const double d = v - rounded(v);
-  return d < 1e-9 && d > -1e-9;
-}
 constexpr bool power_of_two(double v) {
   if (v < 0) v = -v;
   for (double p = 1.0; p <= 64.0; p *= 2.0)

@@ -6,8 +6,8 @@
 // the index arithmetic: a sweep with constant viscosity at 2.1 million sites 55
 // us with a component per thread, 34 us).  The row is unrolled from the
 // generated structure; with a constant viscosity its weights are immediates
-// (those of h = 1, the sum scaled by h), with a variable one the group's row
-// is a kernel parameter.  Offsets are formed from the array stride and the
+// (the sum scaled by the inverse diagonal: weights.h), with a variable
+// one the group's row is a kernel parameter.  Offsets are formed from the array stride and the
 // pitches, uniform for the launch, and added to a 32-bit site index, so that
 // a term is little more than its load and its FMA.  (The kernels these
 // replace passed weights and linear offsets of all groups as a 4.5 KB
@@ -39,6 +39,7 @@
 #include "gs.h"
 #include "kernels.h"
 #include "structure.inc"
+#include "weights.h"
 
 namespace hhg {
 namespace {
@@ -51,8 +52,8 @@ template <int DISC, int VARNU, int GRP>
 constexpr int row_nw() { return VARNU ? gen::S<DISC, VARNU, OP_A>::rows[GRP].n1 : 1; }
 
 // the terms of row GRP behind the diagonal that pass the filter, at the site
-// of 32-bit index i; w: the row's weights (NW = 1: immediates)
-template <class S, int GRP, int SEL, int NW, class T, int... I>
+// of 32-bit index i; w: the row's weights (NW = 1: immediates, weights.h)
+template <int DISC, class S, int GRP, int SEL, int NW, class T, int... I>
 __device__ __forceinline__ T row_sum(const Geo& g, const T* u, const Lines<T>& at, const T (&w)[NW],
                                      std::integer_sequence<int, I...>) {
   T a[3] = {};
@@ -64,13 +65,28 @@ __device__ __forceinline__ T row_sum(const Geo& g, const T* u, const Lines<T>& a
       if constexpr (NW > 1) {
         wt = w[1 + I];
       } else {
-        constexpr double r = S::wref[e];
+        constexpr double r = row_weight<S, e, T>(kScaleA<DISC>);
         wt = T(r);
       }
       a[I % 3] = fma(wt, at.template get<o.di, o.dj, o.dk>(u + o.arr * g.arr), a[I % 3]);
     }
   }(), ...);
   return (a[0] + a[1]) + a[2];
+}
+// (r - s) / diagonal: a row's new value from its right-hand side and its other
+// terms.  Constant viscosity: s in the scale of the row's weights, and with
+// vertex terms only r comes divided (edge_sums)
+template <int DISC, int VARNU, int GRP, int SEL, class T>
+__device__ __forceinline__ T new_value(T r, T s, T inv_diag) {
+  if constexpr (VARNU != 0) {
+    return (r - s) * inv_diag;
+  } else {
+    using S = gen::S<DISC, VARNU, OP_A>;
+    constexpr gen::RowS rw = S::rows[GRP];
+    static_assert(int_weights<S>(rw.t0, rw.n1, kScaleA<DISC>), "the scaled weights are small integers");
+    constexpr Factor<T> f = make_factor<T>(1.0 / row_weight<S, rw.t0, T>(kScaleA<DISC>));
+    return minus_scaled(SEL == kVertexTerms ? r : r * inv_diag, f, s);
+  }
 }
 
 // Programmatic dependent launch: a phase may start while its predecessor in
@@ -107,19 +123,19 @@ __device__ __forceinline__ void gs_site(const uint3 bid, const GsA<T, NW>& a) {
   }
   if constexpr (NC == 1) {
     T r = ld_at(rhs, at.site());
-    const T s = row_sum<S, GRP, SEL>(g, u, at, a.w, std::make_integer_sequence<int, rw.n1 - 1>{});
+    const T s = row_sum<DISC, S, GRP, SEL>(g, u, at, a.w, std::make_integer_sequence<int, rw.n1 - 1>{});
     if (VARNU && SEL != kVertexTerms) r *= T(g.eisc[k]);
-    ref_at(u + GRP * g.arr, at.site()) = (r - (VARNU ? s : T(g.h) * s)) * a.inv_diag;
+    ref_at(u + GRP * g.arr, at.site()) = new_value<DISC, VARNU, GRP, SEL>(r, s, a.inv_diag);
   } else {
     static_assert(DISC == 1 && SEL == kAllTerms && GRP == 0, "one array per component");
     T v[NC];
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
       const int64_t bc = int64_t(a.comp + int(bid.y) + c) * G * g.arr;
-      T r = ld_at(a.rhs + kb * g.sy + (SEL == kVertexTerms ? int64_t(bid.y) * g.arr : bc + GRP * g.arr), at.site());
-      const T s = row_sum<S, GRP, SEL>(g, a.u + bc + kb * g.sy, at, a.w, std::make_integer_sequence<int, rw.n1 - 1>{});
-      if (VARNU && SEL != kVertexTerms) r *= T(g.eisc[k]);
-      v[c] = (r - (VARNU ? s : T(g.h) * s)) * a.inv_diag;
+      T r = ld_at(a.rhs + kb * g.sy + bc + GRP * g.arr, at.site());
+      const T s = row_sum<DISC, S, GRP, SEL>(g, a.u + bc + kb * g.sy, at, a.w, std::make_integer_sequence<int, rw.n1 - 1>{});
+      if (VARNU) r *= T(g.eisc[k]);
+      v[c] = new_value<DISC, VARNU, GRP, SEL>(r, s, a.inv_diag);
     }
 #pragma unroll
     for (int c = 0; c < NC; ++c)
@@ -139,11 +155,12 @@ __global__ void __launch_bounds__(256) kb_gs(const void* items, int n) {
   gs_site<DISC, VARNU, GRP, SEL, NC>(bid, it.a);
 }
 
-// t = rhs - (edge terms of the vertex row) at the interior vertices; block: 32
-// x 8 sites of the plane, a few planes per block on levels that fill the GPU
-// (their lines then meet in L1)
+// t = rhs - (edge terms of the vertex row) at the interior vertices (constant
+// viscosity: divided by the diagonal, the scale of u); block: 32 x 8 sites of the
+// plane, a few planes per block on levels that fill the GPU (their lines then
+// meet in L1)
 template <class T, int NW>
-struct EdgeA { Geo g; const T* u; const T* rhs; T* t; int kp; T w[NW]; };
+struct EdgeA { Geo g; const T* u; const T* rhs; T* t; T inv_diag; int kp; T w[NW]; };
 template <int VARNU, class T, int NW>
 __device__ __forceinline__ void edge_sums(const uint3 bid, const EdgeA<T, NW>& a) {
   using S = gen::S<2, VARNU, OP_A>;
@@ -157,10 +174,10 @@ __device__ __forceinline__ void edge_sums(const uint3 bid, const EdgeA<T, NW>& a
 #pragma unroll 1
   for (int k = k0; k < min(k0 + a.kp, g.nz); ++k) {
     const Lines<T> at(g, unsigned(i + 1) + unsigned(j + 1) * unsigned(g.sx) + unsigned(k + 1) * unsigned(g.sy));
-    const T s = row_sum<S, 0, kEdgeTerms>(g, u, at, a.w, std::make_integer_sequence<int, S::rows[0].n1 - 1>{});
+    const T s = row_sum<2, S, 0, kEdgeTerms>(g, u, at, a.w, std::make_integer_sequence<int, S::rows[0].n1 - 1>{});
     T r = ld_at(rhs, at.site());
     if (VARNU) r *= T(g.eisc[k]);
-    ref_at(t, at.site()) = r - (VARNU ? s : T(g.h) * s);
+    ref_at(t, at.site()) = VARNU ? r - s : new_value<2, VARNU, 0, kEdgeTerms>(r, s, a.inv_diag);
   }
 }
 template <int VARNU, class T>
@@ -217,7 +234,7 @@ void launch_vertex(const Geo& g, const GsRows<T>& rows, bool reverse, T* u, cons
                    cudaStream_t s) {
   constexpr int NW = row_nw<2, VARNU, 0>();
   const int kp = int64_t(g.nx + 1) * (g.ny + 1) * (g.nz + 1) > 1000000 ? 4 : 1;
-  EdgeA<T, NW> a{g, u, rhs, t, kp, {}};
+  EdgeA<T, NW> a{g, u, rhs, t, rows.inv_diag[0], kp, {}};
   if (NW > 1) std::copy(rows.w[0], rows.w[0] + NW, a.w);
   if (g.nx < 2 || g.ny < 2 || g.nz < 2) return;    // no interior vertex
   const dim3 grd((g.nx - 1 + 31) / 32, (g.ny - 1 + 7) / 8, 3 * ((g.nz - 1 + kp - 1) / kp));

@@ -28,6 +28,7 @@
 #include "fast.h"
 #include "rows.h"
 #include "structure.inc"
+#include "weights.h"
 
 namespace hhg {
 namespace {
@@ -41,8 +42,25 @@ struct NoTab {};
 template <int DISC, int VARNU, class T>
 using RowTab = std::conditional_t<kTabled<DISC, VARNU, T>, FastTab<T, gen::S<DISC, VARNU, OP_FULL>::N>, NoTab>;
 
+// h and h^2 in T.  FP32: where they are not exact, in two parts (weights.h; a
+// rounded factor would be a relative error of up to 6e-8 common to all rows).
 template <class T>
-struct FullA { Geo g; const T* x; const T* b; T* y; const ResTabs<T>* tabs; };
+struct Powers { Factor<T> h, h2; bool inexact; };
+template <class T>
+Powers<T> make_powers(double h) {
+  if (sizeof(T) == 8 || (T(h) == h && T(h * h) == h * h)) return {{T(h), T(0)}, {T(h * h), T(0)}, false};
+  return {make_factor<T>(h), make_factor<T>(h * h), true};
+}
+// h^2 times a sum of B^T plus h times one of A
+template <class T>
+__device__ __forceinline__ T combine(const Powers<T>& h, T bt, T a) {
+  if constexpr (sizeof(T) == 8) return fma(h.h.hi, a, h.h2.hi * bt);
+  const T low = h.inexact ? fma(h.h2.lo, bt, h.h.lo * a) : T(0);
+  return fma(h.h.hi, a, fma(h.h2.hi, bt, low));
+}
+
+template <class T>
+struct FullA { Geo g; const T* x; const T* b; T* y; const ResTabs<T>* tabs; Powers<T> h; };
 
 template <class SPT, int T0, class T, class Tab>
 __device__ __forceinline__ T fweight(const Tab& tab) {
@@ -106,14 +124,20 @@ __device__ __forceinline__ T c_terms(const Geo& g, const T* __restrict__ x, cons
   }(), ...);
   return a;
 }
-// terms [T0, T0 + n) of a row in table order: one chain
-template <class S, int T0, class SPT, class T, class Tab, int... I>
+// place in the table of the I-th of n terms of an FP32 row of A: the diagonal,
+// first in the table, comes in the middle, where it meets half of the terms that
+// cancel it (error of a 7-term row on smooth fields 2.3e-7, in table order up to
+// 4.1e-7)
+constexpr int diag_middle(int I, int n) { return I < n / 2 ? I + 1 : I == n / 2 ? 0 : I; }
+// terms [T0, T0 + n) of a row: one chain
+template <class S, int T0, int SEG, class SPT, class T, class Tab, int... I>
 __device__ __forceinline__ T chain(const Geo& g, const T* __restrict__ x, const Lines<T>& at, const Tab& tab,
                                    std::integer_sequence<int, I...>) {
   T a = T(0);
   ([&] {
-    constexpr gen::OffT o = S::off[T0 + I];
-    a = fma(fweight<SPT, T0 + I, T>(tab), at.template ld<o.di, o.dj, o.dk>(x + o.arr * g.arr), a);
+    constexpr int e = T0 + (SEG == 1 && sizeof(T) == 4 ? diag_middle(I, sizeof...(I)) : I);
+    constexpr gen::OffT o = S::off[e];
+    a = fma(fweight<SPT, e, T>(tab), at.template ld<o.di, o.dj, o.dk>(x + o.arr * g.arr), a);
   }(), ...);
   return a;
 }
@@ -160,21 +184,21 @@ __device__ __forceinline__ void velocity_rows(const FullA<T>& a, int i, int j, i
   all_lines<SPT, Q, true>(g, a.x, at, acc, tab, std::make_integer_sequence<int, ps.nl>{});
   // the segments' scales: B^T unscaled (weights at h = 1: h^2), A exp(nu_a h k) (h)
   constexpr bool tabled = kTabled<DISC, VARNU, T>;
-  const T es = VARNU ? T(g.esc[k]) : tabled ? T(1) : T(g.h), e0 = tabled ? T(1) : T(g.h) * T(g.h);
+  const T es = VARNU ? T(g.esc[k]) : T(1);
   ([&] {
     constexpr gen::PartT pt = SPT::parts[ps.p0 + P];
     if constexpr (!pt.all) {
       constexpr int ox = (0xB2 >> pt.og) & 1, oy = (0xD4 >> pt.og) & 1, oz = (0xE8 >> pt.og) & 1;
       if (i <= g.nx - ox && j <= g.ny - oy && k <= g.nz - oz) {
         const bool inside = (ox || (i > 0 && i < g.nx)) && (oy || (j > 0 && j < g.ny)) && (oz || (k > 0 && k < g.nz));
-        put<MODE>(a, pt.out, at.site(), inside, e0 * acc[2 * P] + es * acc[2 * P + 1]);
+        put<MODE>(a, pt.out, at.site(), inside,
+                  tabled ? acc[2 * P] + es * acc[2 * P + 1] : combine(a.h, acc[2 * P], acc[2 * P + 1]));
       }
     }
   }(), ...);
 }
 
-// P1-P1: the velocity rows, row by row in table order (a row's B^T and A
-// segments one chain each; the components' pressure loads are the same)
+// P1-P1: the velocity rows, row by row (a row's B^T and A segments one chain each; the components' pressure loads are the same)
 template <int VARNU, int MODE, class T, class Tab, int... R>
 __device__ __forceinline__ void velocity_rows_p1(const FullA<T>& a, int i, int j, int k, const Lines<T>& at,
                                                  const Tab& tab, std::integer_sequence<int, R...>) {
@@ -182,14 +206,14 @@ __device__ __forceinline__ void velocity_rows_p1(const FullA<T>& a, int i, int j
   using SPT = gen::SP<1, VARNU, OP_FULL>;
   const Geo& g = a.g;
   constexpr bool tabled = kTabled<1, VARNU, T>;
-  const T es = VARNU ? T(g.esc[k]) : tabled ? T(1) : T(g.h), e0 = tabled ? T(1) : T(g.h) * T(g.h);
+  const T es = VARNU ? T(g.esc[k]) : T(1);
   const bool inside = i > 0 && i < g.nx && j > 0 && j < g.ny && k > 0 && k < g.nz;
   ([&] {
     constexpr gen::RowS rw = S::rows[R];
     static_assert(rw.n2 == 0, "no C terms in a velocity row");
-    const T a0 = chain<S, rw.t0, SPT>(g, a.x, at, tab, std::make_integer_sequence<int, rw.n0>{});
-    const T a1 = chain<S, rw.t0 + rw.n0, SPT>(g, a.x, at, tab, std::make_integer_sequence<int, rw.n1>{});
-    put<MODE>(a, rw.out, at.site(), inside, e0 * a0 + es * a1);
+    const T a0 = chain<S, rw.t0, 0, SPT>(g, a.x, at, tab, std::make_integer_sequence<int, rw.n0>{});
+    const T a1 = chain<S, rw.t0 + rw.n0, 1, SPT>(g, a.x, at, tab, std::make_integer_sequence<int, rw.n1>{});
+    put<MODE>(a, rw.out, at.site(), inside, tabled ? a0 + es * a1 : combine(a.h, a0, a1));
   }(), ...);
 }
 
@@ -202,7 +226,7 @@ __device__ __forceinline__ void pressure_row(const FullA<T>& a, int i, int j, in
   static_assert(rw.out == PARR && rw.n1 == 0, "the last row is the pressure's; B is unscaled");
   const Geo& g = a.g;
   T v = b_terms<DISC, S, rw.t0, SPT>(g, a.x, at, tab, std::make_integer_sequence<int, rw.n0>{});
-  if (!kTabled<DISC, VARNU, T>) v *= T(g.h) * T(g.h);
+  if (!kTabled<DISC, VARNU, T>) v = a.h.inexact ? scaled(a.h.h2, v) : a.h.h2.hi * v;
   if constexpr (rw.n2 > 0) {
     T c;
     if (i == 0 || j == 0 || k == 0 || i == g.nx || j == g.ny || k == g.nz) {
@@ -229,7 +253,7 @@ __device__ __forceinline__ void full_body(const uint3 bid, const FullA<T>& full,
   const int w = g.nx + 1, q = bid.x * blockDim.x + threadIdx.x, j = q / w, i = q - j * w, k = bid.y;
   if (j > g.ny) return;
   const int kb = kByPlane<DISC, T> ? k : 0;          // the plane that offsets count from
-  const FullA<T> a{g, full.x + kb * g.sy, full.b + kb * g.sy, full.y + kb * g.sy, full.tabs};
+  const FullA<T> a{g, full.x + kb * g.sy, full.b + kb * g.sy, full.y + kb * g.sy, full.tabs, full.h};
   const Lines<T> at(g, unsigned(i + 1) + unsigned(j + 1) * unsigned(g.sx) + unsigned(k - kb + 1) * unsigned(g.sy));
   using SPT = gen::SP<DISC, VARNU, OP_FULL>;
   if constexpr (DISC == 1) {
@@ -296,7 +320,7 @@ int fast_terms(int disc, int varnu, int op) {
 template <class T>
 void full_rows(int disc, int varnu, int mode, const Geo& g, const void* tab, const ResTabs<T>* tabs, const T* x,
                const T* b, T* y, cudaStream_t s) {
-  const FullA<T> a{g, x, b, y, tabs};
+  const FullA<T> a{g, x, b, y, tabs, make_powers<T>(g.h)};
 #define HHG_F(D, V)                                                           \
   if (disc == D && varnu == V)                                                \
     return mode == MODE_RES ? launch_full<D, V, MODE_RES, T>(a, tab, s)       \

@@ -18,8 +18,8 @@
 //    boundary plane is also stored into the neighbour's halo plane
 //    (distributed shared memory), and a cluster barrier ends the phase;
 //  * rows are unrolled from the generated structure: with a constant
-//    viscosity the weights are immediates too (those of h = 1, the row scaled
-//    by h at the end), with a variable one they are read from a shared table;
+//    viscosity the weights are immediates too (the row scaled at the end:
+//    weights.h), with a variable one they are read from a shared table;
 //  * the right-hand sides tmp_u = b_u - B^T p stay in shared memory.
 //
 // The vertex group takes its four colours in two steps: the part of its row
@@ -55,6 +55,7 @@
 #include "kernels.h"
 #include "small.h"
 #include "structure.inc"
+#include "weights.h"
 
 namespace cg = cooperative_groups;
 
@@ -108,13 +109,15 @@ __host__ __device__ inline ResDims res_dims(int disc, int varnu, const Geo& g, i
 
 // ------------------------------------------------------------- row sums
 enum { kAll = 0, kVertex = 1, kEdges = 2 };
-// weight of term E of operator table S (index W0 + E in the run-time table)
-template <class S, int E, int W0, int VARNU, class T>
+// weight of term E of operator table S (index W0 + E in the run-time table;
+// constant viscosity: weights.h; W0 = 0: the rows of A)
+template <int DISC, class S, int E, int W0, int VARNU, class T>
 __device__ __forceinline__ T weight(const T* sw) {
   if constexpr (VARNU) {
     return sw[W0 + E];
   } else {
-    constexpr double w = S::wref[E];
+    constexpr double K = W0 == 0 ? kScaleA<DISC> : kScaleB<DISC>, w = row_weight<S, E, T>(K);
+    static_assert(int_weights<S>(E, 1, K), "the scaled weights are small integers");
     return T(w);
   }
 }
@@ -128,20 +131,22 @@ __device__ __forceinline__ T row_sum(const T* p, int oj, int ok, const T* sw, st
     constexpr gen::OffT o = S::off[E0 + I];
     constexpr bool vertex = o.arr % G == 0;
     if constexpr ((SEL == kAll || (SEL == kVertex) == vertex) && (COMP < 0 || (o.arr < 3 * G && o.arr / G == COMP)))
-      a[I % 3] = fma(weight<S, E0 + I, W0, VARNU, T>(sw), p[o.arr + PAD * o.di + o.dj * oj + o.dk * ok], a[I % 3]);
+      a[I % 3] = fma(weight<G == 8 ? 2 : 1, S, E0 + I, W0, VARNU, T>(sw),
+                     p[o.arr + PAD * o.di + o.dj * oj + o.dk * ok], a[I % 3]);
   }(), ...);
   return a[0] + a[1] + a[2];
 }
 
-// r[g] -= scale times row R0 + g, all of component R0 / G (B^T rows)
+// r[g] -= row R0 + g, all of component R0 / G (B^T rows)
 template <class S, int R0, int W0, int VARNU, int G, int PAD, class T, int... GG>
-__device__ __forceinline__ void bt_rows(T (&r)[G], const T* p, int oj, int ok, const T* sw, T scale,
+__device__ __forceinline__ void bt_rows(T (&r)[G], const T* p, int oj, int ok, const T* sw, const Factor<T>& sb,
                                         std::integer_sequence<int, GG...>) {
   ([&] {
     constexpr gen::RowS rw = S::rows[R0 + GG];
     static_assert(rw.n1 == 0 && rw.n2 == 0, "B^T is unscaled");
-    r[GG] -= scale * row_sum<S, rw.t0, W0, VARNU, kAll, -1, G, PAD>(p, oj, ok, sw,
-                                                                    std::make_integer_sequence<int, rw.n0>{});
+    const T s = row_sum<S, rw.t0, W0, VARNU, kAll, -1, G, PAD>(p, oj, ok, sw, std::make_integer_sequence<int, rw.n0>{});
+    if constexpr (VARNU != 0) r[GG] -= s;
+    else r[GG] = minus_scaled(r[GG], sb, s);
   }(), ...);
 }
 // the C terms of a pressure row, w: the weights of its boundary class
@@ -178,7 +183,7 @@ __device__ __forceinline__ void with_comp(int comp, F&& f) {
 template <int DISC, int VARNU, bool COMPACT, class T>
 __device__ __forceinline__ void uzawa_resident_body(const Geo& g, T* xg, const T* __restrict__ b,
                                                     const double* __restrict__ inv_ml, const SmallArgs& a,
-                                                    const ResTabs<T>* __restrict__ tabs) {
+                                                    const ResTabs<T>* __restrict__ tabs, const Factor<T>& sb) {
   using SA = gen::S<DISC, VARNU, OP_A>;
   using SBT = gen::S<DISC, VARNU, OP_BT>;
   using SBC = gen::S<DISC, VARNU, OP_BC>;
@@ -262,7 +267,18 @@ __device__ __forceinline__ void uzawa_resident_body(const Geo& g, T* xg, const T
   }
   bar();                                           // every CTA runs before any remote store
 
-  const T hs = T(g.h), hs2 = T(g.h) * T(g.h);
+  // (r - s) / diagonal of group row g; constant viscosity: s in the scale of the
+  // row's weights, r divided already
+  auto over_diag = [&](auto gc, T r, T s) {
+    constexpr int GRP = decltype(gc)::value;
+    if constexpr (VARNU != 0) {
+      return (r - s) * sdiag[GRP];
+    } else {
+      constexpr Factor<T> f = make_factor<T>(1.0 / row_weight<SA, SA::rows[GRP].t0, T>(kScaleA<DISC>));
+      return minus_scaled(r, f, s);
+    }
+  };
+  constexpr std::integral_constant<int, 0> vertex{};
   const int n = dm.n, n3 = 3 * n, m3 = 3 * dm.n4, np = dm.np, nu = (COMPACT ? 1 : DISC == 2 ? 3 : 4) * np;
   constexpr bool kSums = DISC == 2 && !COMPACT;    // the vertex colours share the sums of their edge terms
   for (int it = 0; it < a.iterations; ++it) {
@@ -277,7 +293,7 @@ __device__ __forceinline__ void uzawa_resident_body(const Geo& g, T* xg, const T
       for (int gg = 0; gg < G; ++gg) r[gg] = __ldg(bg + gg * g.arr);
       with_comp(comp, [&](auto cc) {
         constexpr int CO = decltype(cc)::value;
-        bt_rows<SBT, CO * G, WBT, VARNU, G, PAD>(r, p, oj, ok, sw, VARNU ? T(1) : hs2,
+        bt_rows<SBT, CO * G, WBT, VARNU, G, PAD>(r, p, oj, ok, sw, sb,
                                                  std::make_integer_sequence<int, G>{});
       });
       T* t = ts + comp * G * as + il - t0;
@@ -304,9 +320,8 @@ __device__ __forceinline__ void uzawa_resident_body(const Geo& g, T* xg, const T
                   if (!(f >> 16 & 1)) continue;
                   const T s = row_sum<SA, rw.t0 + 1, 0, VARNU, kEdges, -1, G, PAD>(xs + il * PAD + comp * G, oj, ok, sw,
                                                                                    terms);
-                  T einv = T(1);
-                  if (VARNU) einv = T(g.eisc[kb + qdiv(il, msy) - 1]);
-                  ts[(24 + comp) * as + il - t0] = ts[comp * G * as + il - t0] * einv - (VARNU ? s : hs * s);
+                  const T r = ts[comp * G * as + il - t0] * (VARNU ? T(g.eisc[kb + qdiv(il, msy) - 1]) : sdiag[0]);
+                  ts[(24 + comp) * as + il - t0] = VARNU ? r - s : over_diag(vertex, r, s);
                 }
                 __syncthreads();
                 sums = true;
@@ -320,8 +335,8 @@ __device__ __forceinline__ void uzawa_resident_body(const Geo& g, T* xg, const T
               const T s = row_sum<SA, rw.t0 + 1, 0, VARNU, kSums ? kVertex : kAll, -1, G, PAD>(
                   xs + il * PAD + comp * G, oj, ok, sw, terms);
               T t = ts[(kSums ? 24 + comp : comp * G) * as + il - t0];
-              if (!kSums && VARNU) t *= T(g.eisc[kb + kl]);
-              store(il * PAD + comp * G, kl, (t - (VARNU ? s : hs * s)) * sdiag[0]);
+              if (!kSums) t *= VARNU ? T(g.eisc[kb + kl]) : sdiag[0];
+              store(il * PAD + comp * G, kl, over_diag(vertex, t, s));
             }
           } else if constexpr (DISC == 2) {
             sums = false;
@@ -336,8 +351,8 @@ __device__ __forceinline__ void uzawa_resident_body(const Geo& g, T* xg, const T
                 const T t = ts[(comp * G + GRP) * as + il - t0];
                 const T s = row_sum<SA, rw.t0 + 1, 0, VARNU, kAll, -1, G, PAD>(
                     xs + il * PAD + comp * G, oj, ok, sw, std::make_integer_sequence<int, rw.n1 - 1>{});
-                const T v = VARNU ? t * T(g.eisc[kb + kl]) - s : t - hs * s;
-                store(il * PAD + comp * G + GRP, kl, v * inv_diag);
+                store(il * PAD + comp * G + GRP, kl,
+                      over_diag(gc, t * (VARNU ? T(g.eisc[kb + kl]) : inv_diag), s));
               }
             });
           }
@@ -365,7 +380,7 @@ __device__ __forceinline__ void uzawa_resident_body(const Geo& g, T* xg, const T
           s = row_sum<SBC, rw.t0, WBC, VARNU, kAll, decltype(cc)::value, G, PAD>(
               p, oj, ok, sw, std::make_integer_sequence<int, rw.n0>{});
         });
-        if (!VARNU) s *= hs2;
+        if (!VARNU) s = scaled(sb, s);
       }
       return s;
     };
@@ -403,11 +418,11 @@ __device__ __forceinline__ void uzawa_resident_body(const Geo& g, T* xg, const T
 }
 
 template <class T>
-struct ResA { Geo g; T* xg; const T* b; const double* inv_ml; SmallArgs a; const ResTabs<T>* tabs; };
+struct ResA { Geo g; T* xg; const T* b; const double* inv_ml; SmallArgs a; const ResTabs<T>* tabs; Factor<T> sb; };   // sb: h^2 / K
 
 template <int DISC, int VARNU, bool COMPACT, class T>
 __global__ void __launch_bounds__(kResidentThreads, 1) k_uzawa_resident(const __grid_constant__ ResA<T> r) {
-  uzawa_resident_body<DISC, VARNU, COMPACT, T>(r.g, r.xg, r.b, r.inv_ml, r.a, r.tabs);
+  uzawa_resident_body<DISC, VARNU, COMPACT, T>(r.g, r.xg, r.b, r.inv_ml, r.a, r.tabs, r.sb);
 }
 // every cluster of the merged grid belongs to one item (items start at
 // multiples of the cluster size)
@@ -416,7 +431,7 @@ __global__ void __launch_bounds__(kResidentThreads, 1) kb_uzawa_resident(const v
   uint3 bid, gd;
   const auto& it = batch_item<ResA<T>>(items, n, bid, gd);
   const ResA<T>& r = it.a;
-  uzawa_resident_body<DISC, VARNU, COMPACT, T>(r.g, r.xg, r.b, r.inv_ml, r.a, r.tabs);
+  uzawa_resident_body<DISC, VARNU, COMPACT, T>(r.g, r.xg, r.b, r.inv_ml, r.a, r.tabs, r.sb);
 }
 
 template <class T> constexpr int prec_of() { return sizeof(T) == 8 ? HHG_FP64 : HHG_FP32; }
@@ -499,7 +514,7 @@ int uzawa_resident(int disc, int varnu, const Geo& g, int ctas, int threads, T* 
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute attr[1];
   fill_config(cfg, attr, ctas, threads, resident_smem(disc, varnu, g, ctas, prec_of<T>()), s);
-  ResA<T> r{g, x, b, inv_ml, a, tabs};
+  ResA<T> r{g, x, b, inv_ml, a, tabs, make_factor<T>(g.h * g.h / row_scale<T>(disc == 2 ? kScaleB<2> : kScaleB<1>))};
   const bool compact = resident_compact(disc, varnu, g, ctas, prec_of<T>());
   if (g_rec) {
     g_rec->add(kernel_of<T>(disc, varnu, compact, true), dim3(ctas), dim3(threads), cfg.dynamicSmemBytes, ctas, r);

@@ -11,7 +11,7 @@
 //    update is in place; the P1-P1 row does, so that the new pressures go to
 //    the scratch vector and are copied back.
 // All rows are unrolled from the generated structure; with a constant
-// viscosity the weights are immediates (those of h = 1).  Boundary pressure
+// viscosity the weights are immediates (weights.h).  Boundary pressure
 // rows keep the merged B terms (exact for inputs with zero Dirichlet
 // velocities) and take the C stencil of their boundary class.
 //
@@ -35,33 +35,48 @@
 #include "quad.h"
 #include "structure.inc"
 #include "uzrows.h"
+#include "weights.h"
 
 namespace hhg {
 namespace {
 
-template <class S, int E, class T, int NW>
+// 1 / the unit of the C terms of P1-P1
+template <int VARNU>
+constexpr double inv_unit_c() {
+  if constexpr (VARNU) {
+    return 1.0;
+  } else {
+    using S = gen::S<1, 0, OP_BC>;
+    constexpr gen::RowS rw = S::rows[0];
+    return 1.0 / c_unit<S>(rw.t0 + rw.n0, rw.n2);
+  }
+}
+
+// weight of term E, of C (CT) or of B or B^T; constant viscosity (NW = 1): weights.h
+template <int DISC, class S, int E, bool CT, class T, int NW>
 __device__ __forceinline__ T rweight(const T (&w)[NW]) {
   if constexpr (NW > 1) {
     return w[E];
   } else {
-    constexpr double r = S::wref[E];
+    constexpr double K = CT ? inv_unit_c<0>() : kScaleB<DISC>, r = row_weight<S, E, T>(K);
+    static_assert(int_weights<S>(E, 1, K), "the scaled weights are small integers");
     return T(r);
   }
 }
 
 // ------------------------------------------------------------------- B^T
 template <class T, int NW>
-struct BtA { Geo g; const T* x; const T* b; T* y; T w[NW]; };   // b = null: y = B^T p
+struct BtA { Geo g; const T* x; const T* b; T* y; Factor<T> sb; T w[NW]; };   // b = null: y = B^T p; sb: h^2 / K
 template <int DISC, int VARNU>
 constexpr int bt_nw() { return VARNU ? gen::S<DISC, VARNU, OP_BT>::N : 1; }
 
-template <class S, int R, int NW, class T, int... I>
+template <int DISC, class S, int R, int NW, class T, int... I>
 __device__ __forceinline__ T bt_row(const T (&p)[27], const T (&w)[NW], std::integer_sequence<int, I...>) {
   T a = T(0);
   ([&] {
     constexpr int e = S::rows[R].t0 + I;
     constexpr gen::OffT o = S::off[e];
-    a = fma(rweight<S, e>(w), p[(o.di + 1) + 3 * (o.dj + 1) + 9 * (o.dk + 1)], a);
+    a = fma(rweight<DISC, S, e, false>(w), p[(o.di + 1) + 3 * (o.dj + 1) + 9 * (o.dk + 1)], a);
   }(), ...);
   return a;
 }
@@ -84,14 +99,17 @@ __device__ __forceinline__ void bt_groups(const BtA<T, NW>& a, const T (&p)[27],
                                         std::integer_sequence<int, GG...>) {
   using S = gen::S<DISC, VARNU, OP_BT>;
   const Geo& g = a.g;
-  const T hs = VARNU ? T(1) : T(g.h) * T(g.h);
   T bv[sizeof...(GG)];
   ((bv[GG] = a.b && (in >> GG & 1) ? ld_at(a.b + (R0 + GG) * g.arr, at) : T(0)), ...);
   ([&] {
     constexpr gen::RowS rw = S::rows[R0 + GG];
     static_assert(rw.n1 == 0 && rw.n2 == 0, "B^T is unscaled");
-    const T v = bt_row<S, R0 + GG>(p, a.w, std::make_integer_sequence<int, rw.n0>{});
-    if (in >> GG & 1) ref_at(a.y + (R0 + GG) * g.arr, at) = a.b ? bv[GG] - hs * v : hs * v;
+    const T v = bt_row<DISC, S, R0 + GG>(p, a.w, std::make_integer_sequence<int, rw.n0>{});
+    if (in >> GG & 1) {
+      T& y = ref_at(a.y + (R0 + GG) * g.arr, at);
+      if constexpr (VARNU != 0) y = a.b ? bv[GG] - v : v;
+      else y = a.b ? minus_scaled(bv[GG], a.sb, v) : scaled(a.sb, v);
+    }
   }(), ...);
 }
 
@@ -140,14 +158,18 @@ __global__ void __launch_bounds__(128) kb_bt(const void* items, int n) {
 
 // ---------------------------------------------------------- pressure step
 template <class T, int NW>
-struct PressA { Geo g; const T* x; const T* b; T* p; const double* inv_ml; double s; const ResTabs<T>* tabs; int kp; T w[NW]; };
+struct PressA {
+  Geo g; const T* x; const T* b; T* p; const double* inv_ml; double s; const ResTabs<T>* tabs; int kp;
+  Factor<T> sb, sc;                                  // h^2 / K of B, h^3 times the unit of C
+  T w[NW];
+};
 template <int DISC, int VARNU>
 constexpr int bc_nw() { return VARNU ? gen::S<DISC, VARNU, OP_BC>::N : 1; }
 
 // terms [T0, T0 + N) of the pressure row: three chains, one per component, the
 // few C terms (whose diagonal stands in the middle) one chain
 template <bool CT> constexpr int kChains = CT ? 1 : 3;
-template <class S, int T0, int N, bool CT, int NW, class T, int... J>
+template <int DISC, class S, int T0, int N, bool CT, int NW, class T, int... J>
 __device__ __forceinline__ T press_sum(const Geo& g, const T* __restrict__ x, const Lines<T>& at, const T (&w)[NW],
                                        std::integer_sequence<int, J...>) {
   constexpr int M = kChains<CT>;
@@ -156,7 +178,7 @@ __device__ __forceinline__ T press_sum(const Geo& g, const T* __restrict__ x, co
     constexpr int e = chain_term(J, N, M);
     if constexpr (e >= 0) {
       constexpr gen::OffT o = S::off[T0 + e];
-      a[J % M] = fma(rweight<S, T0 + e>(w), at.template ld<o.di, o.dj, o.dk>(x + o.arr * g.arr), a[J % M]);
+      a[J % M] = fma(rweight<DISC, S, T0 + e, CT>(w), at.template ld<o.di, o.dj, o.dk>(x + o.arr * g.arr), a[J % M]);
     }
   }(), ...);
   return (a[0] + a[1]) + a[2];
@@ -189,9 +211,9 @@ __device__ __forceinline__ void press_body(const uint3 bid, const PressA<T, NW>&
     const T bv = __ldg(a.b + 3 * G * g.arr + idx);
     const T ml = T(a.s * __ldg(a.inv_ml + idx));
     const T* x = a.x + idx;
-    T v = press_sum<S, rw.t0, rw.n0, false>(g, a.x + kb * g.sy, at, a.w,
+    T v = press_sum<DISC, S, rw.t0, rw.n0, false>(g, a.x + kb * g.sy, at, a.w,
                                              std::make_integer_sequence<int, chain_steps(rw.n0, kChains<false>)>{});
-    if (!VARNU) v *= T(g.h) * T(g.h);
+    if (!VARNU) v = scaled(a.sb, v);
     if constexpr (rw.n2 > 0) {
       using SPT = gen::SP<DISC, VARNU, OP_BC>;
       T c;
@@ -200,9 +222,9 @@ __device__ __forceinline__ void press_body(const uint3 bid, const PressA<T, NW>&
                         9 * (k == 0 ? 0 : k == g.nz ? 2 : 1);
         c = press_c<SPT>(g, x + 3 * G * g.arr, a.tabs->wc + cls * SPT::NCB, std::make_integer_sequence<int, SPT::NCB>{});
       } else {
-        c = press_sum<S, rw.t0 + rw.n0, rw.n2, true>(g, a.x + kb * g.sy, at, a.w,
+        c = press_sum<DISC, S, rw.t0 + rw.n0, rw.n2, true>(g, a.x + kb * g.sy, at, a.w,
                                                         std::make_integer_sequence<int, rw.n2>{});
-        if (!VARNU) c *= T(g.h) * T(g.h) * T(g.h);
+        if (!VARNU) c = scaled(a.sc, c);
       }
       v += VARNU ? T(g.eisc[k]) * c : c;
       a.p[idx] = __ldg(x + 3 * G * g.arr) - ml * (bv - v);
@@ -254,7 +276,7 @@ void launch_bt(const Geo& g, int mode, const T* w, const T* x, const T* b, T* y,
   if constexpr (DISC == 1 && sizeof(T) == 4) {
     if (quad_bt(VARNU, g, w, x, mode == MODE_RES ? b : nullptr, y, s)) return;
   }
-  BtA<T, NW> a{g, x, mode == MODE_RES ? b : nullptr, y, {}};
+  BtA<T, NW> a{g, x, mode == MODE_RES ? b : nullptr, y, make_factor<T>(g.h * g.h / row_scale<T>(kScaleB<DISC>)), {}};
   if (NW > 1) std::copy(w, w + NW, a.w);
   const dim3 grd((g.ny * g.sx + 127) / 128, g.nz, DISC == 2 ? 3 : 1);
   launch(reinterpret_cast<const void*>(k_bt<DISC, VARNU, T>), reinterpret_cast<const void*>(kb_bt<DISC, VARNU, T>), grd,
@@ -267,7 +289,9 @@ void launch_pressure(const Geo& g, const T* w, const ResTabs<T>* tabs, T* x, con
   T* p = x + 3 * G * g.arr;
   // planes of a block: several where the level fills the GPU anyway
   const int kp = int64_t(g.nx + 1) * (g.ny + 1) * (g.nz + 1) > 1000000 ? 4 : 1;
-  PressA<T, NW> a{g, x, b, DISC == 2 ? p : tmp + 3 * G * g.arr, inv_mlhat, sc, tabs, kp, {}};
+  PressA<T, NW> a{g, x, b, DISC == 2 ? p : tmp + 3 * G * g.arr, inv_mlhat, sc, tabs, kp,
+                   make_factor<T>(g.h * g.h / row_scale<T>(kScaleB<DISC>)),
+                   make_factor<T>(g.h * g.h * g.h / row_scale<T>(inv_unit_c<VARNU>())), {}};
   if (NW > 1) std::copy(w, w + NW, a.w);
   const dim3 grd((g.ny * g.sx + g.nx + 256) / 256, (g.nz + kp) / kp);
   bool done = false;

@@ -152,3 +152,47 @@ def test_pressure_row(disc, L, path):
     print(f"{disc} {path}: {rms(lib) / rms(exact):.3e}, one chain {rms(plain) / rms(exact):.3e}, "
           f"ratio {rms(lib) / rms(plain):.3f}")
     assert rms(lib) <= rms(plain)
+
+
+@pytest.mark.parametrize("disc,box,L", [("P1P1", (3, 1, 2), 3), ("P1P1", (5, 1, 1), 3), ("P2P1", (3, 1, 2), 3),
+                                        ("P2P1", (1, 1, 5), 3)])
+def test_no_common_factor(disc, box, L):
+    """Mesh widths that are no power of two: no error of the factor that scales a
+    row.  With integers as input the terms of these rows are integers times a unit
+    of the row and add up exactly, so that a row is its sum times a factor, rounded
+    once: half a unit in the last place, and a hundredth of it for the factor (in
+    two parts: 2^-46).  A factor rounded to FP32 is off by up to as much again, and
+    all rows with it."""
+    from paper_2010_13513_gb300 import hhg
+    lc = 0 if disc == "P1P1" else 1
+    pb = lib_problem(box, L, disc, lc=lc, solve="mixed")
+    lev = oracle_hierarchy(box, L, disc, lc=lc).lv[L]
+    x = np.random.default_rng(5).integers(1, 1000, size=lev.size).astype(np.float64)
+    x[:3 * lev.nv] *= np.tile(lev.vint, 3)
+    inner = np.concatenate([lev.vint] * 3)
+    u, p = lev.split(x)
+    only_u, only_p = lev.join(u, 0 * p), lev.join([0 * c for c in u], p)
+
+    def check(name, out, exact):
+        s = np.abs(exact) > 1e-6 * np.abs(exact).max()               # (exact zeros are not, in the oracle)
+        e = np.abs(out[s] - exact[s]) / np.spacing(np.abs(exact[s]).astype(F))
+        print(f"{disc} {box} {name}: {e.max():.3f} units in the last place, {s.sum()} rows")
+        assert s.sum() > 1000 and e.max() <= 0.51
+
+    y = pb.new_vector(L, hhg.FP32)
+    pb.apply(L, "BT", pb.to_device(L, only_p, hhg.FP32), y)
+    check("B^T p", pb.to_host(L, y)[:3 * lev.nv][inner],
+          np.concatenate([(lev.B[c].T @ p) * lev.vint for c in range(3)])[inner])
+    if disc == "P1P1":
+        pb.apply(L, "FULL", pb.to_device(L, only_u, hhg.FP32), y)
+        check("full operator", pb.to_host(L, y)[:3 * lev.nv][inner], np.concatenate([lev.A @ c for c in u])[inner])
+    # the vertex colour that a sweep updates first: - (the rest of the row) / diagonal
+    first = lev.phases[0]
+    exact = np.concatenate([(lev.Adiag * c - lev.A @ c)[first] / lev.Adiag[first] for c in u])
+    # (the resident smoother of P2-P1 rounds the edge terms' sum on the way)
+    for ctas in (0, 4) if disc == "P1P1" else (0,):
+        pb.set_level_smoother(L, ctas, prec=hhg.FP32)
+        xd = pb.to_device(L, only_u, hhg.FP32)
+        pb.smooth(L, hhg.Params.make(1, 1, 0, 1, "f", 1, OMEGA_INV[disc]), 1, xd, pb.new_vector(L, hhg.FP32))
+        out = lev.split(pb.to_host(L, xd))[0]
+        check(f"first colour, {ctas} CTAs", np.concatenate([c[first] for c in out]), exact)

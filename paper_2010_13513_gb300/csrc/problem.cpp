@@ -2355,8 +2355,8 @@ extern "C" int hhg_estimate_omega(hhg_problem* pb, int level, int iters, const d
     for (auto r = phases.rbegin(); r != phases.rend(); ++r)
       launch_gs<double>(g, lv.op[OP_A], r->first, r->second, lv.inv_diag[r->first], V2, V1, pb->stream);
     launch_axpy<double>(-1.0, V1 + po, V2 + po, g.arr, pb->stream);                // V2_p = -v
-    HHG_TRY(apply_op<double>(pb, lv, OP_BC, MODE_SET, V2, nullptr, Wv));           // w = B y + C v
-    launch_xpby<double>(Wv + po, 0.0, Wv + po, Wv + po, g.arr, pb->stream);
+    bc_rows(pb->desc.disc, pb->desc.nu_a != 0.0 ? 1 : 0, g, static_cast<const double*>(ftab<double>(lv, OP_BC)),
+            rtab<double>(lv), V2, Wv, pb->stream);                                 // w = B y + C v
     // w <- M_L(1/nu)^{-1} w : multiply by inv_mlhat through the pressure update
     // kernel applied to a zero vector: 0 - (w * inv_ml) * (-1)
     HHG_CUDA(cudaMemsetAsync(V1 + po, 0, size_t(g.arr) * 8, pb->stream));

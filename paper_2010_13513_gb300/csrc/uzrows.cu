@@ -192,8 +192,9 @@ __device__ __forceinline__ T press_c(const Geo& g, const T* __restrict__ p, cons
   return a;
 }
 
-// grid x over the positions of the padded (i, j) plane, y = groups of kp planes
-template <int DISC, int VARNU, class T, int NW>
+// grid x over the positions of the padded (i, j) plane, y = groups of kp planes;
+// ROW: the row itself into p, no update
+template <int DISC, int VARNU, bool ROW, class T, int NW>
 __device__ __forceinline__ void press_body(const uint3 bid, const PressA<T, NW>& a) {
   using S = gen::S<DISC, VARNU, OP_BC>;
   constexpr gen::RowS rw = S::rows[0];
@@ -208,8 +209,11 @@ __device__ __forceinline__ void press_body(const uint3 bid, const PressA<T, NW>&
     const int64_t idx = int64_t(i + 1) + int64_t(j + 1) * g.sx + int64_t(k + 1) * g.sy;
     const int kb = kByPlane<DISC, T> ? k : 0;        // the plane that offsets count from
     const Lines<T> at(g, unsigned(idx - kb * g.sy));
-    const T bv = __ldg(a.b + 3 * G * g.arr + idx);
-    const T ml = T(a.s * __ldg(a.inv_ml + idx));
+    T bv = T(0), ml = T(0);
+    if constexpr (!ROW) {
+      bv = __ldg(a.b + 3 * G * g.arr + idx);
+      ml = T(a.s * __ldg(a.inv_ml + idx));
+    }
     const T* x = a.x + idx;
     T v = press_sum<DISC, S, rw.t0, rw.n0, false>(g, a.x + kb * g.sy, at, a.w,
                                              std::make_integer_sequence<int, chain_steps(rw.n0, kChains<false>)>{});
@@ -227,21 +231,26 @@ __device__ __forceinline__ void press_body(const uint3 bid, const PressA<T, NW>&
         if (!VARNU) c = scaled(a.sc, c);
       }
       v += VARNU ? T(g.eisc[k]) * c : c;
-      a.p[idx] = __ldg(x + 3 * G * g.arr) - ml * (bv - v);
-    } else {
-      a.p[idx] -= ml * (bv - v);
     }
+    if constexpr (ROW) a.p[idx] = v;
+    else if constexpr (rw.n2 > 0) a.p[idx] = __ldg(x + 3 * G * g.arr) - ml * (bv - v);
+    else a.p[idx] -= ml * (bv - v);
   }
 }
 template <int DISC, int VARNU, class T>
 __global__ void __launch_bounds__(256, DISC == 2 || sizeof(T) == 8 ? 2 : 3) k_pressure(const __grid_constant__ PressA<T, bc_nw<DISC, VARNU>()> a) {
-  press_body<DISC, VARNU>(blockIdx, a);
+  press_body<DISC, VARNU, false>(blockIdx, a);
 }
 template <int DISC, int VARNU, class T>
 __global__ void __launch_bounds__(256, DISC == 2 || sizeof(T) == 8 ? 2 : 3) kb_pressure(const void* items, int n) {
   uint3 bid, gd;
   const auto& it = batch_item<PressA<T, bc_nw<DISC, VARNU>()>>(items, n, bid, gd);
-  press_body<DISC, VARNU>(bid, it.a);
+  press_body<DISC, VARNU, false>(bid, it.a);
+}
+
+template <int DISC, int VARNU>
+__global__ void __launch_bounds__(256, 2) k_bc(const __grid_constant__ PressA<double, bc_nw<DISC, VARNU>()> a) {
+  press_body<DISC, VARNU, true>(blockIdx, a);
 }
 
 // P1-P1: the new pressures back into the iterate
@@ -282,13 +291,14 @@ void launch_bt(const Geo& g, int mode, const T* w, const T* x, const T* b, T* y,
   launch(reinterpret_cast<const void*>(k_bt<DISC, VARNU, T>), reinterpret_cast<const void*>(kb_bt<DISC, VARNU, T>), grd,
          128, a, s);
 }
+// planes of a block: several where the level fills the GPU anyway
+int press_planes(const Geo& g) { return int64_t(g.nx + 1) * (g.ny + 1) * (g.nz + 1) > 1000000 ? 4 : 1; }
 template <int DISC, int VARNU, class T>
 void launch_pressure(const Geo& g, const T* w, const ResTabs<T>* tabs, T* x, const T* b, T* tmp,
                      const double* inv_mlhat, double sc, cudaStream_t s) {
   constexpr int NW = bc_nw<DISC, VARNU>(), G = DISC == 2 ? 8 : 1;
   T* p = x + 3 * G * g.arr;
-  // planes of a block: several where the level fills the GPU anyway
-  const int kp = int64_t(g.nx + 1) * (g.ny + 1) * (g.nz + 1) > 1000000 ? 4 : 1;
+  const int kp = press_planes(g);
   PressA<T, NW> a{g, x, b, DISC == 2 ? p : tmp + 3 * G * g.arr, inv_mlhat, sc, tabs, kp,
                    make_factor<T>(g.h * g.h / row_scale<T>(kScaleB<DISC>)),
                    make_factor<T>(g.h * g.h * g.h / row_scale<T>(inv_unit_c<VARNU>())), {}};
@@ -304,7 +314,27 @@ void launch_pressure(const Geo& g, const T* w, const ResTabs<T>* tabs, T* x, con
            dim3(unsigned(std::min<int64_t>((g.arr + 255) / 256, 152 * 8))), 256, CopyA<T>{a.p, p, g.arr}, s);
 }
 
+template <int DISC, int VARNU>
+void launch_bc(const Geo& g, const double* w, const ResTabs<double>* tabs, const double* x, double* y, cudaStream_t s) {
+  constexpr int NW = bc_nw<DISC, VARNU>(), G = DISC == 2 ? 8 : 1;
+  PressA<double, NW> a{g, x, nullptr, y + 3 * G * g.arr, nullptr, 0.0, tabs, press_planes(g),
+                       make_factor<double>(g.h * g.h / row_scale<double>(kScaleB<DISC>)),
+                       make_factor<double>(g.h * g.h * g.h / row_scale<double>(inv_unit_c<VARNU>())), {}};
+  if (NW > 1) std::copy(w, w + NW, a.w);
+  const dim3 grd((g.ny * g.sx + g.nx + 256) / 256, (g.nz + a.kp) / a.kp);
+  ++g_launches;
+  k_bc<DISC, VARNU><<<grd, 256, 0, s>>>(a);
+}
+
 }  // namespace
+
+void bc_rows(int disc, int varnu, const Geo& g, const double* w, const ResTabs<double>* tabs, const double* x,
+             double* y, cudaStream_t s) {
+  if (disc == 1 && !varnu) launch_bc<1, 0>(g, w, tabs, x, y, s);
+  else if (disc == 1) launch_bc<1, 1>(g, w, tabs, x, y, s);
+  else if (!varnu) launch_bc<2, 0>(g, w, tabs, x, y, s);
+  else launch_bc<2, 1>(g, w, tabs, x, y, s);
+}
 
 template <class T>
 void bt_rows(int disc, int varnu, int mode, const Geo& g, const T* w, const T* x, const T* b, T* y, cudaStream_t s) {

@@ -22,4 +22,9 @@ template <class T>
 void uzawa_pressure(int disc, int varnu, const Geo& g, const T* w, const ResTabs<T>* tabs, T* x, const T* b, T* tmp,
                     const double* inv_mlhat, double s, cudaStream_t st);
 
+// y_p = B u - C p, FP64 (the power iteration of the spectral estimate); w, tabs
+// as above
+void bc_rows(int disc, int varnu, const Geo& g, const double* w, const ResTabs<double>* tabs, const double* x,
+             double* y, cudaStream_t s);
+
 }  // namespace hhg

@@ -1,5 +1,7 @@
-// Element access by 32-bit byte offset.
+// Element access by 32-bit byte offset, and pieces that the unrolled rows share.
 #pragma once
+
+#include <utility>
 
 #include "internal.h"
 
@@ -36,6 +38,15 @@ constexpr int chain_term(int j, int n, int m) {
   return e < ((q + 1) * n + m - 1) / m ? e : -1;
 }
 constexpr int chain_steps(int n, int m) { return (n + m - 1) / m * m; }
+
+// the C terms of a boundary pressure row at p: the stencil wc of its class
+template <class SPT, class T, int... O>
+__device__ __forceinline__ T c_class(const Geo& g, const T* __restrict__ p, const T* __restrict__ wc,
+                                     std::integer_sequence<int, O...>) {
+  T a = T(0);
+  ((a = fma(__ldg(wc + O), __ldg(p + SPT::cbo[O].di + SPT::cbo[O].dj * g.sx + SPT::cbo[O].dk * g.sy), a)), ...);
+  return a;
+}
 
 // FP64 P1-P1 arrays may exceed the 4 GB (up to 715 million sites are
 // accepted): its kernels count offsets from the site's plane instead

@@ -43,7 +43,7 @@ template <int DISC, int VARNU, class T>
 using RowTab = std::conditional_t<VARNU != 0, FastTab<T, gen::S<DISC, VARNU, OP_FULL>::N>, NoTab>;
 
 template <class T>
-struct MarchA { Geo g; const T* x; const T* b; T* y; const ResTabs<T>* tabs; int kc; };
+struct MarchA { Geo g; const T* x; const T* b; T* y; int kc; };
 
 // columns of a pass: array slot, i and j offset, the planes lo .. hi read, and
 // the first of the column's registers
@@ -128,14 +128,14 @@ __device__ __forceinline__ void shift(T (&w)[NR], std::integer_sequence<int, C..
   }(), ...);
 }
 
-// acc[3 part + segment] (constant viscosity: segments 0 and 1 share one)
+// acc[2 part + segment] (constant viscosity: the segments B^T and A share one)
 template <class SPT, int Q, int L, int VARNU, class T, class Tab, int NR, int NA, int... I>
 __device__ __forceinline__ void line_terms(const T (&w)[NR], T (&acc)[NA], const Tab& tab,
                                            std::integer_sequence<int, I...>) {
   ([&] {
     constexpr gen::LineT ln = SPT::lines[L];
     constexpr gen::TermE te = SPT::terms[ln.e0 + I];
-    constexpr int a = 3 * te.part + (VARNU || te.seg == 2 ? te.seg : 0), r = Cols<SPT, Q>::reg(ln.slot, ln.dj, te.di, ln.dk);
+    constexpr int a = 2 * te.part + (VARNU ? te.seg : 0), r = Cols<SPT, Q>::reg(ln.slot, ln.dj, te.di, ln.dk);
     acc[a] = fma(mweight<SPT, te.t, VARNU, T>(tab), w[r], acc[a]);
   }(), ...);
 }
@@ -144,23 +144,6 @@ __device__ __forceinline__ void all_terms(const T (&w)[NR], T (&acc)[NA], const 
                                           std::integer_sequence<int, L...>) {
   (line_terms<SPT, Q, SPT::passes[Q].l0 + L, VARNU>(
        w, acc, tab, std::make_integer_sequence<int, SPT::lines[SPT::passes[Q].l0 + L].ne>{}), ...);
-}
-
-// whether part P of pass Q has C terms (segment 2)
-template <class SPT, int Q, int P>
-constexpr bool has_c() {
-  constexpr gen::PassT ps = SPT::passes[Q];
-  for (int l = ps.l0; l < ps.l0 + ps.nl; ++l)
-    for (int e = SPT::lines[l].e0; e < SPT::lines[l].e0 + SPT::lines[l].ne; ++e)
-      if (SPT::terms[e].part == P && SPT::terms[e].seg == 2) return true;
-  return false;
-}
-template <class SPT, class T, int... O>
-__device__ __forceinline__ T c_class(const Geo& g, const T* __restrict__ p, const T* __restrict__ wc,
-                                     std::integer_sequence<int, O...>) {
-  T a = T(0);
-  ((a = fma(__ldg(wc + O), __ldg(p + SPT::cbo[O].di + SPT::cbo[O].dj * g.sx + SPT::cbo[O].dk * g.sy), a)), ...);
-  return a;
 }
 
 // what the rows of a step are combined with -- the right-hand side (MODE_RES),
@@ -192,26 +175,15 @@ template <int DISC, int VARNU, int MODE, int Q, class T, int NA, int NP, int... 
 __device__ __forceinline__ void store_rows(const MarchA<T>& a, int i, int j, int k, unsigned at, const T (&acc)[NA],
                                            const T (&old)[NP], std::integer_sequence<int, P...>) {
   using SPT = gen::SP<DISC, VARNU, OP_FULL>;
-  constexpr int PARR = DISC == 2 ? 24 : 3;
+  static_assert(gen::S<DISC, VARNU, OP_FULL>::rows[24].n2 == 0, "P2-P1: no C terms");
   const Geo& g = a.g;
-  const T es = VARNU ? T(__ldg(g.esc + k)) : T(1), eis = VARNU ? T(__ldg(g.eisc + k)) : T(1);
+  const T es = VARNU ? T(__ldg(g.esc + k)) : T(1);
   ([&] {
     constexpr gen::PartT pt = SPT::parts[SPT::passes[Q].p0 + P];
     constexpr int ox = (0xB2 >> pt.og) & 1, oy = (0xD4 >> pt.og) & 1, oz = (0xE8 >> pt.og) & 1;
     if (i <= g.nx - ox && j <= g.ny - oy && k <= g.nz - oz) {
       const bool inside = (ox || (i > 0 && i < g.nx)) && (oy || (j > 0 && j < g.ny)) && (oz || (k > 0 && k < g.nz));
-      T v = VARNU ? acc[3 * P] + es * acc[3 * P + 1] : (pt.all ? T(g.h) * T(g.h) : T(g.h)) * acc[3 * P];
-      if constexpr (has_c<SPT, Q, P>()) {
-        T c = acc[3 * P + 2];                      // (constant viscosity: the pressures entered scaled by h)
-        if (!VARNU) c *= T(g.h) * T(g.h);
-        if (!inside) {
-          const int cls = (i == 0 ? 0 : i == g.nx ? 2 : 1) + 3 * (j == 0 ? 0 : j == g.ny ? 2 : 1) +
-                          9 * (k == 0 ? 0 : k == g.nz ? 2 : 1);
-          c = c_class<SPT>(g, a.x + PARR * g.arr + at / unsigned(sizeof(T)), a.tabs->wc + cls * SPT::NCB,
-                           std::make_integer_sequence<int, SPT::NCB>{});
-        }
-        v += eis * c;
-      }
+      const T v = VARNU ? acc[2 * P] + es * acc[2 * P + 1] : (pt.all ? T(g.h) * T(g.h) : T(g.h)) * acc[2 * P];
       T& y = ref_at(a.y + pt.out * g.arr, at);
       if (!pt.all && !inside) {
         y = T(0);                              // Dirichlet velocity row
@@ -232,7 +204,7 @@ __device__ __forceinline__ void march_body(const uint3 bid, const MarchA<T>& a, 
   using SPT = gen::SP<DISC, VARNU, OP_FULL>;
   constexpr gen::PassT ps = SPT::passes[Q];
   constexpr auto cols = std::make_integer_sequence<int, Cols<SPT, Q>::t.n>{};
-  constexpr int PARR = DISC == 2 ? 24 : 3;
+  constexpr int PARR = 24;
   const Geo& g = a.g;
   const int q = bid.x * blockDim.x + threadIdx.x, j = q / g.sx, i = q - j * g.sx;
   if (i > g.nx || j > g.ny) return;
@@ -247,7 +219,7 @@ __device__ __forceinline__ void march_body(const uint3 bid, const MarchA<T>& a, 
     const Lines<T> lines(g, site);
     const unsigned at = lines.site();
     step_loads<SPT, Q, PARR, VARNU>(g, a.x, lines, hs, w, cols);
-    T old[ps.np], acc[3 * ps.np] = {};
+    T old[ps.np], acc[2 * ps.np] = {};
     old_values<DISC, VARNU, MODE, Q>(a, at, old, std::make_integer_sequence<int, ps.np>{});
     if ((threadIdx.x & 7) == 0 && k + kAhead < k1)  // one thread per 32-byte sector
       prefetch_planes<DISC, VARNU, MODE, Q>(a, at + kAhead * plane * unsigned(sizeof(T)), std::make_integer_sequence<int, ps.na>{});
@@ -298,19 +270,17 @@ void launch_march(MarchA<T>& a, const void* tab, cudaStream_t s, std::integer_se
 }  // namespace
 
 template <class T>
-void march_rows(int disc, int varnu, int mode, const Geo& g, const void* tab, const ResTabs<T>* tabs, const T* x,
-                const T* b, T* y, cudaStream_t s) {
-  MarchA<T> a{g, x, b, y, tabs, 1};
-#define HHG_M(D, V)                                                                                          \
-  if (disc == D && varnu == V) {                                                                             \
-    using Passes = std::make_integer_sequence<int, gen::SP<D, V, OP_FULL>::NP>;                              \
-    return mode == MODE_RES ? launch_march<D, V, MODE_RES, T>(a, tab, s, Passes{})                           \
-                            : launch_march<D, V, MODE_SET, T>(a, tab, s, Passes{});                          \
-  }
-  HHG_M(2, 0) HHG_M(2, 1)
-#undef HHG_M
+void march_rows(int varnu, int mode, const Geo& g, const void* tab, const T* x, const T* b, T* y, cudaStream_t s) {
+  MarchA<T> a{g, x, b, y, 1};
+  auto launch = [&](auto v) {
+    constexpr int V = decltype(v)::value;
+    using Passes = std::make_integer_sequence<int, gen::SP<2, V, OP_FULL>::NP>;
+    if (mode == MODE_RES) launch_march<2, V, MODE_RES, T>(a, tab, s, Passes{});
+    else launch_march<2, V, MODE_SET, T>(a, tab, s, Passes{});
+  };
+  if (varnu) launch(std::integral_constant<int, 1>{});
+  else launch(std::integral_constant<int, 0>{});
 }
-template void march_rows<float>(int, int, int, const Geo&, const void*, const ResTabs<float>*, const float*,
-                                const float*, float*, cudaStream_t);
+template void march_rows<float>(int, int, const Geo&, const void*, const float*, const float*, float*, cudaStream_t);
 
 }  // namespace hhg

@@ -5,16 +5,14 @@
 
 #include "internal.h"
 #include "kernels.h"
-#include "small.h"
 
 namespace hhg {
 
 // y = calA x (MODE_SET) or y = b - calA x (MODE_RES) over all rows of a level
 // (Dirichlet velocity rows 0); inputs with zero Dirichlet velocity entries.
 // tab: host FastTab of the full operator (read with a variable viscosity
-// only), tabs: device table with the C stencil per boundary class
+// only)
 template <class T>
-void march_rows(int disc, int varnu, int mode, const Geo& g, const void* tab, const ResTabs<T>* tabs, const T* x,
-                const T* b, T* y, cudaStream_t s);
+void march_rows(int varnu, int mode, const Geo& g, const void* tab, const T* x, const T* b, T* y, cudaStream_t s);
 
 }  // namespace hhg

@@ -360,8 +360,8 @@ extern "C" int hhg_problem_create(const hhg_mesh* mesh, const hhg_problem_desc* 
     for (int o = 0; o < OP_COUNT; ++o) {
       OpHost h = serialise(lv.st.op[o], lv.g);
       const int N = fast_terms(desc->disc, varnu, o);
-      if (N >= 0) {
-        if (N != int(h.terms.size())) return fail(HHG_EINVAL, "internal: specialised kernel structure mismatch");
+      if (N >= 0 && N != int(h.terms.size())) return fail(HHG_EINVAL, "internal: specialised kernel structure mismatch");
+      if (N >= 0 && o != OP_A) {                   // (the rows of A: GsRows, ResTabs)
         auto image = [&](auto zero, std::vector<char>& out) {
           using T = decltype(zero);
           const size_t bytes = (size_t(N) * (sizeof(T) + 4) + 7) / 8 * 8;
@@ -649,13 +649,13 @@ template <class T> const ResTabs<T>* rtab(const Level& lv);
 template <> const ResTabs<double>* rtab<double>(const Level& lv) { return lv.rtab64; }
 template <> const ResTabs<float>* rtab<float>(const Level& lv) { return lv.rtab32; }
 
-// the streaming kernels of the full operator if the level's shape selects them (true if launched)
 // P2-P1 in FP32 has two ways, by size: above a million sites the marching
 // kernels (level 7 of one cube: 206 us against 290 us), below the unstaged
 // rows (level 6: 29 us against 41 us)
 bool marched(const hhg_problem* pb, const Level& lv) {
   return pb->ov == 2 && int64_t(lv.g.nx + 1) * (lv.g.ny + 1) * (lv.g.nz + 1) > 1000000;
 }
+// the streaming kernels of the full operator if the level's shape selects them (true if launched)
 template <class T>
 bool stream_op(hhg_problem* pb, Level& lv, const Shape& sh, int mode, const T* x, const T* b, T* y) {
   const int nt = sizeof(T) == 8 ? sh.st64_threads : sh.st_threads;
@@ -670,7 +670,7 @@ int apply_op(hhg_problem* pb, Level& lv, int op, int mode, const T* x, const T* 
   if (op == OP_FULL && mode != MODE_ADD) {
     if constexpr (sizeof(T) == 4) {
       if (marched(pb, lv)) {
-        march_rows(disc, varnu, mode, lv.g, ftab<T>(lv, OP_FULL), rtab<T>(lv), x, b, y, pb->stream);
+        march_rows(varnu, mode, lv.g, ftab<T>(lv, OP_FULL), x, b, y, pb->stream);
         HHG_CHECK_LAUNCH();
         return HHG_OK;
       }
@@ -1945,7 +1945,7 @@ int tune_level(hhg_problem* pb, Level& lv, int reps, T* xa, T* xb) {
     tune_rows(xa, xb, bestS.st64_threads, nullptr);
     bestS.st_threads = bestS.st64_threads;
   } else {
-    tune_rows(xa, xb, bestS.st_threads, &bestS.st_sites);
+    if (!marched(pb, lv)) tune_rows(xa, xb, bestS.st_threads, &bestS.st_sites);
     tune_rows(lv.tmp64, lv.bw64, bestS.st64_threads, nullptr);
   }
   // Gauss-Seidel phases: threads per block, the vertex colours and the edge

@@ -80,15 +80,6 @@ __device__ __forceinline__ void quad_lines(const Geo& g, const float* __restrict
   (quad_line<SPT, L>(g, x, at, lo, hi, tab, acc, std::make_integer_sequence<int, SPT::lines[L].ne>{}), ...);
 }
 
-// the C terms of a boundary row: the stencil of its class
-template <class SPT, int... O>
-__device__ __forceinline__ float quad_class(const Geo& g, const float* __restrict__ p, const float* __restrict__ wc,
-                                            std::integer_sequence<int, O...>) {
-  float a = 0.0f;
-  ((a = fmaf(__ldg(wc + O), __ldg(p + SPT::cbo[O].di + SPT::cbo[O].dj * g.sx + SPT::cbo[O].dk * g.sy), a)), ...);
-  return a;
-}
-
 // v at the sites of mask m
 __device__ __forceinline__ void quad_store(float* base, unsigned off, int m, const float (&v)[4]) {
   if (m == 15) {
@@ -148,7 +139,7 @@ __device__ __forceinline__ void quad_body(const uint3 bid, const QuadA& a, const
 #pragma unroll
         for (int s = 0; s < 4; ++s)
           if (bnd >> s & 1)
-            acc[P][1][s] = quad_class<SPT>(
+            acc[P][1][s] = c_class<SPT>(
                 g, p + s, a.tabs->wc + (cjk + (i + s == 0 ? 0 : i + s == g.nx ? 2 : 1)) * SPT::NCB,
                 std::make_integer_sequence<int, SPT::NCB>{});
       }

@@ -141,13 +141,6 @@ __device__ __forceinline__ T chain(const Geo& g, const T* __restrict__ x, const 
   }(), ...);
   return a;
 }
-template <class SPT, class T, int... O>
-__device__ __forceinline__ T c_class(const Geo& g, const T* __restrict__ p, const T* __restrict__ wc,
-                                     std::integer_sequence<int, O...>) {
-  T a = T(0);
-  ((a = fma(__ldg(wc + O), __ldg(p + SPT::cbo[O].di + SPT::cbo[O].dj * g.sx + SPT::cbo[O].dk * g.sy), a)), ...);
-  return a;
-}
 // terms [T0, T0 + n) of the pressure row: eight (P1-P1: three, a component each)
 // chains of consecutive terms (FP32 error of the apply's pressure, P2-P1 level 6:
 // 1.9e-7 in one chain, 4.8e-7 with the terms dealt out to four in turn, 1.0e-7

@@ -20,8 +20,9 @@ constexpr int kResMaxTerms = 640;   // component-0 rows of A, the rows of B^T, t
 constexpr int kResMaxC = 15;        // lattice offsets of the C stencil
 
 // run-time weights of one level: the rows of A of component 0, of B^T and of
-// (B, -C) in the order of the generated structure (read with a variable
-// viscosity only), and the C stencil of the pressure row clipped to the
+// (B, -C) in the order of the generated structure (the smoother reads them with a
+// variable viscosity only, the full operator's rows (rows.cu) the interior C
+// terms of P1-P1 with a constant one too), and the C stencil of the pressure row clipped to the
 // domain per boundary class (27 x the stencil's offsets, class
 // ci + 3 cj + 9 ck with c = 0 on the low face, 1 inside, 2 on the high face)
 template <class T>

@@ -183,14 +183,6 @@ __device__ __forceinline__ T press_sum(const Geo& g, const T* __restrict__ x, co
   }(), ...);
   return (a[0] + a[1]) + a[2];
 }
-// the C terms of a boundary row: the stencil of its class
-template <class SPT, class T, int... O>
-__device__ __forceinline__ T press_c(const Geo& g, const T* __restrict__ p, const T* __restrict__ wc,
-                                     std::integer_sequence<int, O...>) {
-  T a = T(0);
-  ((a = fma(__ldg(wc + O), __ldg(p + SPT::cbo[O].di + SPT::cbo[O].dj * g.sx + SPT::cbo[O].dk * g.sy), a)), ...);
-  return a;
-}
 
 // grid x over the positions of the padded (i, j) plane, y = groups of kp planes;
 // ROW: the row itself into p, no update
@@ -224,7 +216,7 @@ __device__ __forceinline__ void press_body(const uint3 bid, const PressA<T, NW>&
       if (i == 0 || j == 0 || k == 0 || i == g.nx || j == g.ny || k == g.nz) {
         const int cls = (i == 0 ? 0 : i == g.nx ? 2 : 1) + 3 * (j == 0 ? 0 : j == g.ny ? 2 : 1) +
                         9 * (k == 0 ? 0 : k == g.nz ? 2 : 1);
-        c = press_c<SPT>(g, x + 3 * G * g.arr, a.tabs->wc + cls * SPT::NCB, std::make_integer_sequence<int, SPT::NCB>{});
+        c = c_class<SPT>(g, x + 3 * G * g.arr, a.tabs->wc + cls * SPT::NCB, std::make_integer_sequence<int, SPT::NCB>{});
       } else {
         c = press_sum<DISC, S, rw.t0 + rw.n0, rw.n2, true>(g, a.x + kb * g.sy, at, a.w,
                                                         std::make_integer_sequence<int, rw.n2>{});

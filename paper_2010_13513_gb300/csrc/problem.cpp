@@ -2043,9 +2043,10 @@ extern "C" int hhg_autotune(hhg_problem* pb, int reps, int* shapes_out) {
       o[5] = lv.shape.st_threads;
       o[6] = lv.shape.row_sites;
       o[7] = o[8] = 1;                             // lanes per Gauss-Seidel site
-      // (the smoother's B^T and (B, -C) rows have one launch shape, uzrows.cu)
-      o[9] = 128; o[10] = 1; o[11] = 1;
-      o[12] = 256; o[13] = 1; o[14] = 1;
+      // (the smoother's B^T and (B, -C) rows: a fixed shape by size, uzrows.cu)
+      const RowsShape bt = bt_shape(pb->desc.disc, mixed, lv.g), bc = pressure_shape(pb->desc.disc, mixed, lv.g);
+      o[9] = bt.threads; o[10] = bt.planes; o[11] = bt.sites;
+      o[12] = bc.threads; o[13] = bc.planes; o[14] = bc.sites;
       o[15] = lv.shape.gs_threads0 ? lv.shape.gs_threads0 : lv.shape.gs_threads;
     }
   }

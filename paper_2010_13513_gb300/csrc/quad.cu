@@ -161,7 +161,7 @@ __device__ __forceinline__ void quad_body(const uint3 bid, const QuadA& a, const
   }
 }
 template <int VARNU, int OP>
-__global__ void __launch_bounds__(256, 3) k_quad(const __grid_constant__ QuadA a,
+__global__ void __launch_bounds__(kQuadThreads, 3) k_quad(const __grid_constant__ QuadA a,
                                                  const __grid_constant__ QuadTab<VARNU, OP> tab) {
   quad_body<VARNU, OP>(blockIdx, a, tab);
 }
@@ -169,7 +169,7 @@ __global__ void __launch_bounds__(256, 3) k_quad(const __grid_constant__ QuadA a
 template <int VARNU, int OP>
 struct QuadB { QuadA a; const QuadTab<VARNU, OP>* tab; };
 template <int VARNU, int OP>
-__global__ void __launch_bounds__(256, 3) kb_quad(const void* items, int n) {
+__global__ void __launch_bounds__(kQuadThreads, 3) kb_quad(const void* items, int n) {
   uint3 bid, gd;
   const auto& it = batch_item<QuadB<VARNU, OP>>(items, n, bid, gd);
   quad_body<VARNU, OP>(bid, it.a.a, *it.a.tab);
@@ -180,19 +180,23 @@ __global__ void __launch_bounds__(256, 3) kb_quad(const void* items, int n) {
 // / 410 us with a site per thread (uzrows.cu); at 2.1 million, 70 / 64 us and
 // 72 / 64 us, and four planes a block are too few blocks (82 / 75 us)
 constexpr int64_t kQuadSites = 4000000;
-
+}  // namespace
+bool quad_level(const Geo& g) {
+  return int64_t(g.nx + 1) * (g.ny + 1) * (g.nz + 1) > kQuadSites && g.sx % 4 == 0;
+}
+namespace {
 bool aligned(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
 
 template <int VARNU, int OP>
 bool launch_quad(const QuadA& q, const float* w, cudaStream_t s) {
   const Geo& g = q.g;
-  if (int64_t(g.nx + 1) * (g.ny + 1) * (g.nz + 1) <= kQuadSites || g.sx % 4 || !aligned(q.x) || !aligned(q.b) || !aligned(q.y) || !aligned(q.inv_ml)) return false;
+  if (!quad_level(g) || !aligned(q.x) || !aligned(q.b) || !aligned(q.y) || !aligned(q.inv_ml)) return false;
   QuadA a = q;
-  a.kp = 4;
-  const dim3 grd(((g.ny + 1) * (g.sx / 4) + 255) / 256, (g.nz + a.kp) / a.kp);
+  a.kp = kQuadPlanes;
+  const dim3 grd(((g.ny + 1) * (g.sx / 4) + kQuadThreads - 1) / kQuadThreads, (g.nz + a.kp) / a.kp);
   using Tab = QuadTab<VARNU, OP>;
   if (g_rec) {
-    g_rec->add(reinterpret_cast<const void*>(kb_quad<VARNU, OP>), grd, dim3(256), 0, 1,
+    g_rec->add(reinterpret_cast<const void*>(kb_quad<VARNU, OP>), grd, dim3(kQuadThreads), 0, 1,
                QuadB<VARNU, OP>{a, static_cast<const Tab*>(g_rec->table(w, sizeof(Tab)))});
     return true;
   }
@@ -200,7 +204,7 @@ bool launch_quad(const QuadA& q, const float* w, cudaStream_t s) {
   std::copy(w, w + sizeof(tab.w) / 4, tab.w);
   ++g_launches;
   void* args[] = {&a, &tab};
-  cudaLaunchKernel(reinterpret_cast<const void*>(k_quad<VARNU, OP>), grd, dim3(256), args, 0, s);
+  cudaLaunchKernel(reinterpret_cast<const void*>(k_quad<VARNU, OP>), grd, dim3(kQuadThreads), args, 0, s);
   return true;
 }
 

@@ -9,9 +9,12 @@
 
 namespace hhg {
 
+// whether the level is large enough, and its pitch a multiple of four
+bool quad_level(const Geo& g);
+constexpr int kQuadThreads = 256, kQuadPlanes = 4;
+
 // Each launches its rows and returns true, or returns false with nothing
-// launched: a level that is too small or whose pitch is not a multiple of
-// four, a vector that is not 16-byte aligned.  w: the level's weights of the operator (the FastTab
+// launched: another level, a vector that is not 16-byte aligned.  w: the level's weights of the operator (the FastTab
 // image), tabs: device table with the C stencil per boundary class.
 
 // y = B^T p (b = null) or y = b - B^T p at the interior sites; p the pressures of x

@@ -113,6 +113,8 @@ __device__ __forceinline__ void bt_groups(const BtA<T, NW>& a, const T (&p)[27],
   }(), ...);
 }
 
+constexpr int kBtThreads = 128, kPressThreads = 256;
+
 // grid x over the positions of the padded (i, j) plane, y = plane, z = component
 template <int DISC, int VARNU, class T, int NW>
 __device__ __forceinline__ void bt_body(const uint3 bid, const BtA<T, NW>& full) {
@@ -146,11 +148,11 @@ __device__ __forceinline__ void bt_body(const uint3 bid, const BtA<T, NW>& full)
   }
 }
 template <int DISC, int VARNU, class T>
-__global__ void __launch_bounds__(128) k_bt(const __grid_constant__ BtA<T, bt_nw<DISC, VARNU>()> a) {
+__global__ void __launch_bounds__(kBtThreads) k_bt(const __grid_constant__ BtA<T, bt_nw<DISC, VARNU>()> a) {
   bt_body<DISC, VARNU>(blockIdx, a);
 }
 template <int DISC, int VARNU, class T>
-__global__ void __launch_bounds__(128) kb_bt(const void* items, int n) {
+__global__ void __launch_bounds__(kBtThreads) kb_bt(const void* items, int n) {
   uint3 bid, gd;
   const auto& it = batch_item<BtA<T, bt_nw<DISC, VARNU>()>>(items, n, bid, gd);
   bt_body<DISC, VARNU>(bid, it.a);
@@ -230,18 +232,18 @@ __device__ __forceinline__ void press_body(const uint3 bid, const PressA<T, NW>&
   }
 }
 template <int DISC, int VARNU, class T>
-__global__ void __launch_bounds__(256, DISC == 2 || sizeof(T) == 8 ? 2 : 3) k_pressure(const __grid_constant__ PressA<T, bc_nw<DISC, VARNU>()> a) {
+__global__ void __launch_bounds__(kPressThreads, DISC == 2 || sizeof(T) == 8 ? 2 : 3) k_pressure(const __grid_constant__ PressA<T, bc_nw<DISC, VARNU>()> a) {
   press_body<DISC, VARNU, false>(blockIdx, a);
 }
 template <int DISC, int VARNU, class T>
-__global__ void __launch_bounds__(256, DISC == 2 || sizeof(T) == 8 ? 2 : 3) kb_pressure(const void* items, int n) {
+__global__ void __launch_bounds__(kPressThreads, DISC == 2 || sizeof(T) == 8 ? 2 : 3) kb_pressure(const void* items, int n) {
   uint3 bid, gd;
   const auto& it = batch_item<PressA<T, bc_nw<DISC, VARNU>()>>(items, n, bid, gd);
   press_body<DISC, VARNU, false>(bid, it.a);
 }
 
 template <int DISC, int VARNU>
-__global__ void __launch_bounds__(256, 2) k_bc(const __grid_constant__ PressA<double, bc_nw<DISC, VARNU>()> a) {
+__global__ void __launch_bounds__(kPressThreads, 2) k_bc(const __grid_constant__ PressA<double, bc_nw<DISC, VARNU>()> a) {
   press_body<DISC, VARNU, true>(blockIdx, a);
 }
 
@@ -279,9 +281,9 @@ void launch_bt(const Geo& g, int mode, const T* w, const T* x, const T* b, T* y,
   }
   BtA<T, NW> a{g, x, mode == MODE_RES ? b : nullptr, y, make_factor<T>(g.h * g.h / row_scale<T>(kScaleB<DISC>)), {}};
   if (NW > 1) std::copy(w, w + NW, a.w);
-  const dim3 grd((g.ny * g.sx + 127) / 128, g.nz, DISC == 2 ? 3 : 1);
+  const dim3 grd((g.ny * g.sx + kBtThreads - 1) / kBtThreads, g.nz, DISC == 2 ? 3 : 1);
   launch(reinterpret_cast<const void*>(k_bt<DISC, VARNU, T>), reinterpret_cast<const void*>(kb_bt<DISC, VARNU, T>), grd,
-         128, a, s);
+         kBtThreads, a, s);
 }
 // planes of a block: several where the level fills the GPU anyway
 int press_planes(const Geo& g) { return int64_t(g.nx + 1) * (g.ny + 1) * (g.nz + 1) > 1000000 ? 4 : 1; }
@@ -295,12 +297,12 @@ void launch_pressure(const Geo& g, const T* w, const ResTabs<T>* tabs, T* x, con
                    make_factor<T>(g.h * g.h / row_scale<T>(kScaleB<DISC>)),
                    make_factor<T>(g.h * g.h * g.h / row_scale<T>(inv_unit_c<VARNU>())), {}};
   if (NW > 1) std::copy(w, w + NW, a.w);
-  const dim3 grd((g.ny * g.sx + g.nx + 256) / 256, (g.nz + kp) / kp);
+  const dim3 grd((g.ny * g.sx + g.nx + kPressThreads) / kPressThreads, (g.nz + kp) / kp);
   bool done = false;
   if constexpr (DISC == 1 && sizeof(T) == 4) done = quad_pressure(VARNU, g, w, tabs, x, b, a.p, inv_mlhat, sc, s);
   if (!done)
     launch(reinterpret_cast<const void*>(k_pressure<DISC, VARNU, T>),
-           reinterpret_cast<const void*>(kb_pressure<DISC, VARNU, T>), grd, 256, a, s);
+           reinterpret_cast<const void*>(kb_pressure<DISC, VARNU, T>), grd, kPressThreads, a, s);
   if (DISC == 1)
     launch(reinterpret_cast<const void*>(k_copy<T>), reinterpret_cast<const void*>(kb_copy<T>),
            dim3(unsigned(std::min<int64_t>((g.arr + 255) / 256, 152 * 8))), 256, CopyA<T>{a.p, p, g.arr}, s);
@@ -313,12 +315,21 @@ void launch_bc(const Geo& g, const double* w, const ResTabs<double>* tabs, const
                        make_factor<double>(g.h * g.h / row_scale<double>(kScaleB<DISC>)),
                        make_factor<double>(g.h * g.h * g.h / row_scale<double>(inv_unit_c<VARNU>())), {}};
   if (NW > 1) std::copy(w, w + NW, a.w);
-  const dim3 grd((g.ny * g.sx + g.nx + 256) / 256, (g.nz + a.kp) / a.kp);
+  const dim3 grd((g.ny * g.sx + g.nx + kPressThreads) / kPressThreads, (g.nz + a.kp) / a.kp);
   ++g_launches;
-  k_bc<DISC, VARNU><<<grd, 256, 0, s>>>(a);
+  k_bc<DISC, VARNU><<<grd, kPressThreads, 0, s>>>(a);
 }
 
 }  // namespace
+
+RowsShape bt_shape(int disc, bool fp32, const Geo& g) {
+  if (disc == 1 && fp32 && quad_level(g)) return {kQuadThreads, kQuadPlanes, 4};
+  return {kBtThreads, 1, 1};
+}
+RowsShape pressure_shape(int disc, bool fp32, const Geo& g) {
+  if (disc == 1 && fp32 && quad_level(g)) return {kQuadThreads, kQuadPlanes, 4};
+  return {kPressThreads, press_planes(g), 1};
+}
 
 void bc_rows(int disc, int varnu, const Geo& g, const double* w, const ResTabs<double>* tabs, const double* x,
              double* y, cudaStream_t s) {

@@ -22,6 +22,11 @@ template <class T>
 void uzawa_pressure(int disc, int varnu, const Geo& g, const T* w, const ResTabs<T>* tabs, T* x, const T* b, T* tmp,
                     const double* inv_mlhat, double s, cudaStream_t st);
 
+// launch shapes of the two on a level (fp32: the precision), for reports
+struct RowsShape { int threads, planes, sites; };
+RowsShape bt_shape(int disc, bool fp32, const Geo& g);
+RowsShape pressure_shape(int disc, bool fp32, const Geo& g);
+
 // y_p = B u - C p, FP64 (the power iteration of the spectral estimate); w, tabs
 // as above
 void bc_rows(int disc, int varnu, const Geo& g, const double* w, const ResTabs<double>* tabs, const double* x,

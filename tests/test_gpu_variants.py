@@ -102,7 +102,7 @@ def test_marching_rows_with_variable_viscosity():
     from oracle.sampled import sample_rows
     from paper_2010_13513_gb300 import hhg
     box, H, L, nu_a = (2, 2, 1), 0.5, 6, 1.3
-    pb = hhg.Problem(hhg.Mesh.box(*box, H), disc="P2P1", L=L, coarse_level=2, solve="mixed", nu_a=nu_a)
+    pb = hhg.Problem(hhg.Mesh.box(*box, H), disc="P2P1", L=L, coarse_level=1, solve="mixed", nu_a=nu_a)
     info = pb.layout(L)
     nv = info.n_velocity_nodes
     rng = np.random.default_rng(11)

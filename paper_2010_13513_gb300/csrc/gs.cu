@@ -6,10 +6,10 @@
 // the index arithmetic: a sweep with constant viscosity at 2.1 million sites 55
 // us with a component per thread, 34 us).  The row is unrolled from the
 // generated structure; with a constant viscosity its weights are immediates
-// (the sum scaled by the inverse diagonal: weights.h), with a variable
-// one the group's row is a kernel parameter.  Offsets are formed from the array stride and the
-// pitches, uniform for the launch, and added to a 32-bit site index, so that
-// a term is little more than its load and its FMA.  (The kernels these
+// (the sum scaled by the inverse diagonal: weights.h), with a variable one the
+// group's row is a kernel parameter.  Offsets are formed from the array stride
+// and the pitches, uniform for the launch, and added to a 32-bit site index, so
+// that a term is little more than its load and its FMA.  (The kernels these
 // replace passed weights and linear offsets of all groups as a 4.5 KB
 // parameter table, one thread or up to four lanes per site for all three
 // components, about six instructions per term.)
@@ -18,7 +18,10 @@
 // gs_vertex_phases sums these terms once for all four colours, with
 // consecutive sites in consecutive lanes; a launch per colour, whose lanes lie
 // four sites apart (four times the sectors per access), then reads the six
-// vertex neighbours only.
+// vertex neighbours only.  One smoothing step (three sweeps, FP32) with full rows on
+// all components / component by component / on shared edge sums: level 6 211 / 324
+// / 213 us, 1.1 million sites (2x2x1 cubes) 894 / 842 / 796 us, level 7 1,725 /
+// 1,577 / 1,503 us; with variable viscosity at 1.1 million 1,019 / 1,001 / 963 us.
 //
 // Bound: launch latency on level 5, L1/L2 loads on level 6, HBM on level 7 (an
 // edge phase reads the whole velocity, 217 MB in FP32).  Measured, one forward

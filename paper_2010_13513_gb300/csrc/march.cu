@@ -18,9 +18,10 @@
 // Bound: instruction issue (about 690 instructions per site and pass, 290 of
 // them FMAs) and the latency of a step's loads at 16 warps per SM.  Measured,
 // level 7, 6-tetrahedron cube: apply 206 us (four sites staged in shared
-// memory, the kernel this replaces: 271 us), residual 241 us (461 us).  On
-// level 6 the rows without marching (rows.cu) are faster (29 against 41 us):
-// the runs of planes are too short to fill the GPU.  P1-P1, with 28 columns
+// memory, the kernel this replaces: 271 us), residual 241 us (461 us), with a
+// variable viscosity 245 us (314 us).  On level 6 the rows
+// without marching (rows.cu) are faster (29 against 41 us): the runs of planes
+// are too short to fill the GPU.  P1-P1, with 28 columns
 // and 112 or 150 terms, is slower this way than staged (one component's loads
 // in flight are too few): it keeps the streaming kernels.
 #include <cuda_runtime.h>

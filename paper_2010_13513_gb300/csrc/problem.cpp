@@ -424,7 +424,7 @@ extern "C" int hhg_problem_create(const hhg_mesh* mesh, const hhg_problem_desc* 
       lv.grows32.inv_diag[gg] = float(lv.inv_diag[gg]);
     }
     // (until hhg_autotune times it: above a million sites the vertex phases
-    // are worth the separate pass over the edges)
+    // are worth the separate pass over the edges, gs.cu)
     lv.shape.gs_edge_sums = pb->G == 8 && int64_t(lv.g.nx + 1) * (lv.g.ny + 1) * (lv.g.nz + 1) > 1000000 ? 1 : 0;
     HHG_TRY(put_res_tabs<double>(B, lv, c_class, lv.o_rtab64));
     HHG_TRY(put_res_tabs<float>(B, lv, c_class, lv.o_rtab32));
@@ -649,11 +649,16 @@ template <class T> const ResTabs<T>* rtab(const Level& lv);
 template <> const ResTabs<double>* rtab<double>(const Level& lv) { return lv.rtab64; }
 template <> const ResTabs<float>* rtab<float>(const Level& lv) { return lv.rtab32; }
 
-// P2-P1 in FP32 has two ways, by size: above a million sites the marching
-// kernels (level 7 of one cube: 206 us against 290 us), below the unstaged
-// rows (level 6: 29 us against 41 us)
+// P2-P1 in FP32 has two ways, by size: above half a million sites the marching
+// kernels, below the unstaged rows, whose blocks fill the GPU earlier.  Apply /
+// residual in us, marching against unstaged, constant viscosity (variable):
+//   0.27 million sites  41 /  49 ( 46 /  53)   29 /  39 ( 33 /  41)
+//   0.55                64 /  79 ( 74 /  91)   64 /  98 ( 72 / 105)
+//   0.82                82 /  94 ( 90 / 111)  101 / 151 (115 / 160)
+//   1.08               114 / 135 (129 / 158)  135 / 202 (152 / 211)
+//   2.15               206 / 242 (237 / 287)  264 / 395 (297 / 410)
 bool marched(const hhg_problem* pb, const Level& lv) {
-  return pb->ov == 2 && int64_t(lv.g.nx + 1) * (lv.g.ny + 1) * (lv.g.nz + 1) > 1000000;
+  return pb->ov == 2 && int64_t(lv.g.nx + 1) * (lv.g.ny + 1) * (lv.g.nz + 1) > 500000;
 }
 // the streaming kernels of the full operator if the level's shape selects them (true if launched)
 template <class T>

@@ -19,7 +19,7 @@
 // these replace read a weight and an offset per term from memory (dependent
 // loads), divided a row's terms over lanes and took two launches each.
 // Measured (FP32, P2-P1, 2x1x1 cubes at level 6, restriction and prolongation):
-// 248 us before, 64 us now (79 us with single sites instead of pairs); their
+// 248 us before, 61 us now (79 us with single sites instead of pairs); their
 // vectors once over HBM would take 26 us.  Level 7: restriction 372 us before,
 // 92 us now; prolongation 558 us before, 127 us now.
 #include <cuda_runtime.h>

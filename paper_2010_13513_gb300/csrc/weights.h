@@ -7,7 +7,7 @@
 // parts: rounded to FP32 it would be a relative error of up to 6e-8 common to
 // all rows, which the sweeps of a smoother add up (P2-P1 level 5, a smoothing
 // step: velocity error 1.0e-7 with weights rounded one by one, 1.9e-7 with
-// integers and a rounded 1 / diagonal).  FP64 rows take the weights of h = 1 and
+// integers and a rounded 1 / diagonal, 7.4e-8 now).  FP64 rows take the weights of h = 1 and
 // a rounded factor.
 #pragma once
 
